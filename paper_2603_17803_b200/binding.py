@@ -224,8 +224,8 @@ def swarm_cache_admit(score: torch.Tensor, cluster_size: torch.Tensor, capacity_
                                             ctypes.c_int64(capacity_pages), _ptr(ws), ctypes.c_int64(ws.numel()),
                                             _ptr(resident, "resident"), _ptr(info, "info"), _stream(stream)),
            "swarm_cache_admit")
-    if stream is None:
-        torch.cuda.current_stream(score.device).synchronize()     # the scratch is freed when this returns
+    if stream is not None:
+        ws.record_stream(stream)      # (on the current stream the allocator's own order protects the scratch)
 
 
 def swarm_build_clusters_workspace_bytes(n_entries: int) -> int:
@@ -247,16 +247,22 @@ def swarm_build_clusters(dist: torch.Tensor, tau: float, members_cap: Optional[i
     cap = int(members_cap if members_cap is not None else 16 * n)
     i32 = dict(dtype=torch.int32, device=dev)
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
-    density, ptr, medoid = torch.empty(n, **i32), torch.empty(n + 4, **i32), torch.empty(n, **i32)
-    members, info = torch.empty(max(cap, 4), **i32), torch.zeros(8, **i32)
+    density, medoid, members = torch.empty(n, **i32), torch.empty(n, **i32), torch.empty(max(cap, 4), **i32)
+    head = torch.empty(n + 12, **i32)                # [0] clusters, [4] status, [8:] cluster_ptr: one copy to the host
+    ptr = head[8:]
     _check(lib.swarm_build_clusters(_ptr(dist, "dist"), ctypes.c_int32(n), ctypes.c_float(tau), _ptr(ws),
                                     ctypes.c_int64(ws_bytes), _ptr(density), _ptr(ptr), _ptr(members),
-                                    ctypes.c_int64(cap), _ptr(medoid), _ptr(info[0:4]), _ptr(info[4:8]),
+                                    ctypes.c_int64(cap), _ptr(medoid), _ptr(head), _ptr(head[4:]),
                                     _stream(stream)), "swarm_build_clusters")
-    n_clusters, status = int(info[0]), int(info[4])
+    if stream is not None and stream != torch.cuda.current_stream(dev):   # the copy waits for the caller's stream
+        torch.cuda.current_stream(dev).wait_stream(stream)
+    host = head.cpu()
+    n_clusters, status = int(host[0]), int(host[4])
+    if status == 2:
+        raise SwarmError(ERR_CUDA, "swarm_build_clusters (a bounded wait ran out)")
     if status != 0:
         raise SwarmError(ERR_WORKSPACE_TOO_SMALL, "swarm_build_clusters (members_cap)")
-    return density, ptr[: n_clusters + 1], members[: int(ptr[n_clusters])], medoid[:n_clusters]
+    return density, ptr[: n_clusters + 1], members[: int(host[8 + n_clusters])], medoid[:n_clusters]
 
 
 def swarm_set_submit_order(ctx, submit_order=None, submit_info=None) -> None:

@@ -1,187 +1,528 @@
 // Algorithm 1: offline co-activation clustering on a given distance matrix (Sec. 4.1, Steps 3 and 4).
 //
-//   density_kernel   rho[i] = #{ j != i : D[i][j] <= tau }  -- one warp per row, 16-byte loads; the only part
-//                    that touches the whole n x n matrix, bound by HBM bandwidth (4 n^2 bytes read once)
-//   queue_kernel     medoid queue: entries by (rho descending, index ascending), each entry's place found by
-//                    counting the entries that precede it (n^2 integer compares on data held in shared memory)
-//   expand_kernel    one CTA walks the queue.  For an uncovered medoid m: the candidates { e != m : D[m][e] <= tau }
-//                    are compacted in index order, placed by (distance, index) rank, and then joined greedily.
-//                    Between two joins neither the running sums nor the bound tau * |C| change, so the next
-//                    candidate to join is the first one in queue order whose sum passes: a block-wide minimum
-//                    finds it, and the number of dependent steps is the cluster size, not the candidate count.
-//                    A candidate's sum is a plain fp32 accumulation in joining order over D[member][candidate],
-//                    so every decision is the one a sequential fp32 walk takes.
-// Covered entries remain candidates of later medoids: an entry can sit in several clusters (the paper's replicas).
+//   density_kernel   rho[i] = #{ j != i : D[i][j] <= tau } and the adjacency bits behind it -- one warp per row,
+//                    16-byte loads; the only pass over the whole n x n matrix, bound by HBM bandwidth (4 n^2 bytes read
+//                    once, n^2 / 8 written)
+//   rounds_kernel    everything else in one cooperative launch, see below
+//
+// The listing walks the entries by (rho descending, index ascending) and grows a cluster from every entry that no
+// earlier cluster has covered.  Two facts make that walk parallel without changing a single decision:
+//   - what a cluster contains depends on its medoid and the matrix alone (covered entries remain candidates, which is
+//     where the paper's replicas come from), so clusters of different medoids can grow side by side;
+//   - the members of m's cluster lie within tau of m, so an uncovered entry that has no uncovered entry in front of it
+//     (in queue order) within tau is a medoid no matter what the others turn out to be.
+// The kernel works in rounds: mark every uncovered entry that an earlier uncovered one might still cover (adjacency
+// bits), grow the clusters of the unmarked ones -- one CTA each -- and cover their members behind them in the queue.  8192 entries in 64 topics:
+// 102 clusters in 12 rounds.  At the end every cluster's place in the output follows from the keys and sizes.
+//
+// Growing one cluster: the candidates are sorted by (distance, index) in shared memory.  Between two joins neither the
+// running sums nor the bound tau * |C| change, so the next candidate to join is the first undecided one whose sum
+// passes.  One warp decides, its candidates' sums in registers (no CTA-wide barrier on the chain); the other warps
+// fetch the candidates' matrix rows, restricted to the candidates behind them, into a ring of shared memory ahead of
+// the decisions: the walk used to pay a trip to memory and two CTA-wide barriers per join (1.3 us).
+// A candidate's sum is a plain fp32 accumulation in joining order over D[member][candidate], so every decision is the
+// one a sequential fp32 walk takes.
 #include "swarm_internal.cuh"
+
+#include <algorithm>
 
 namespace swarm {
 namespace {
 
-constexpr int kExpandThreads = 1024;
+// ---- adjacency bits ------------------------------------------------------------------------------------------
+// A row's bits come in blocks of 128 columns = 4 words: bit l of word c of block k stands for column 128 k + 4 l + c
+// (the lanes of a warp hold four neighbouring columns each, so a ballot per component is a word).
+__host__ __device__ inline int adj_words(int n) { return (n + 127) / 128 * 4; }
+__device__ __forceinline__ int adj_column(int word, int bit) { return (word >> 2) * 128 + 4 * bit + (word & 3); }
 
-__global__ void __launch_bounds__(256)
-density_kernel(const float* __restrict__ dist, int n, float tau, int32_t* __restrict__ rho) {
-  const int lane = threadIdx.x & 31;
-  const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  if (row >= n) return;
-  const float* r = dist + (long long)row * n;
-  int cnt = 0;
-  if ((n & 3) == 0) {                                     // rows are 16-byte aligned
-    for (int j = lane * 4; j < n; j += 128) {
-      const uint4 v = ldg_nc_v4(r + j);
-      cnt += (__uint_as_float(v.x) <= tau && j != row) + (__uint_as_float(v.y) <= tau && j + 1 != row) +
-             (__uint_as_float(v.z) <= tau && j + 2 != row) + (__uint_as_float(v.w) <= tau && j + 3 != row);
-    }
-  } else {
-    for (int j = lane; j < n; j += 32) cnt += (__ldg(r + j) <= tau && j != row);
-  }
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
-  if (lane == 0) rho[row] = cnt;
-}
-
-// queue[place] = i with place = #{ j : rho[j] > rho[i] or (rho[j] == rho[i] and j < i) }
-__global__ void __launch_bounds__(256)
-queue_kernel(const int32_t* __restrict__ rho, int n, int32_t* __restrict__ queue) {
-  __shared__ int s_rho[2048];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int mine = i < n ? rho[i] : 0;
-  int place = 0;
-  for (int base = 0; base < n; base += 2048) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < 2048 && base + t < n; t += blockDim.x) s_rho[t] = rho[base + t];
-    __syncthreads();
-    const int lim = min(2048, n - base);
-    for (int t = 0; t < lim; ++t) {
-      const int other = s_rho[t];
-      place += (other > mine) || (other == mine && base + t < i);
-    }
-  }
-  if (i < n) queue[place] = i;
-}
-
-struct ExpandArgs {
+struct ClusterArgs {
   const float* dist;
   int n;
   float tau;
-  const int32_t* queue;
-  // scratch, n entries each
-  int32_t* cand_raw;     // candidates in index order
-  int32_t* cand;         // candidates in (distance, index) order
-  float* sum;            // running sum of the candidate's distances to the members
-  uint8_t* covered;
+  int32_t* rho;
+  // scratch (see build_clusters_workspace_bytes)
+  uint32_t* adj;         // [n][adj_words(n)]
+  uint32_t* covered;     // bit e: entry e is covered
+  uint32_t* blocked;     // two arrays of such bits, used by alternate rounds
+  unsigned* ctl;         // kCtl* below
+  int32_t* tab_medoid;   // clusters in the order they were finished
+  int32_t* tab_size;
+  int32_t* tab_at;       // start in the arena, or -1: the arena was full, the cluster is grown again for the output
+  int32_t* arena;
+  int arena_cap;
   // outputs
   int32_t* ptr;
   int32_t* members;
   long long members_cap;
   int32_t* medoid;
   int32_t* n_clusters;
-  int32_t* dev_status;   // 0 ok, 1 members_cap too small
+  int32_t* dev_status;   // 0 ok, 1 members_cap too small, 2 a bounded wait ran out
+};
+constexpr int kCtlArrived = 0, kCtlClusters = 1, kCtlArena = 2, kCtlFailed = 3, kCtlWords = 64;
+__host__ __device__ inline int bit_words(int n) { return (n + 31) / 32; }
+
+__global__ void __launch_bounds__(256) density_kernel(ClusterArgs a) {
+  const int lane = threadIdx.x & 31, n = a.n;
+  if (blockIdx.x == 0 && threadIdx.x < kCtlWords) a.ctl[threadIdx.x] = 0u;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < bit_words(n); i += gridDim.x * blockDim.x) {
+    a.covered[i] = 0u;
+    a.blocked[i] = a.blocked[bit_words(n) + i] = 0u;
+  }
+  const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+  if (row >= n) return;
+  const float* r = a.dist + (long long)row * n;
+  uint32_t* bits = a.adj + (long long)row * adj_words(n);
+  int cnt = 0;
+  const bool vec = (n & 3) == 0;                          // rows are 16-byte aligned
+#pragma unroll 4
+  for (int j0 = 0; j0 < n; j0 += 128) {
+    const int j = j0 + lane * 4;
+    bool near[4] = {false, false, false, false};
+    if (vec) {
+      if (j < n) {
+        const uint4 v = ldg_nc_v4(r + j);
+        near[0] = __uint_as_float(v.x) <= a.tau; near[1] = __uint_as_float(v.y) <= a.tau;
+        near[2] = __uint_as_float(v.z) <= a.tau; near[3] = __uint_as_float(v.w) <= a.tau;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) near[c] = j + c < n && __ldg(r + j + c) <= a.tau;
+    }
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint32_t w = __ballot_sync(0xFFFFFFFFu, near[c] && j + c != row);
+      cnt += __popc(w);
+      if (lane == c) mine = w;
+    }
+    if (lane < 4) bits[j0 / 32 + lane] = mine;
+  }
+  if (lane == 0) a.rho[row] = cnt;
+}
+
+// ---- rounds ----------------------------------------------------------------------------------------------------
+constexpr int kRoundThreads = 512;
+constexpr int kRoundWarps = kRoundThreads / 32;
+constexpr int kFastCand = 1024;                           // candidates one deciding warp holds (32 per lane)
+constexpr int kFetchWarps = kRoundWarps - 1;
+constexpr int kRingSlots = 4 * kFetchWarps;               // (a multiple of the fetching warps: every slot has one owner)
+constexpr int kRingBytes = 128 * 1024;
+constexpr int kMineCap = 1024;
+constexpr unsigned kGridWaitLimit = 1u << 23;
+constexpr unsigned kRingWaitLimit = 1u << 24;
+
+// Order-preserving key of a distance (-0 folded onto +0) and back.
+__device__ __forceinline__ uint32_t dist_key(float d) {
+  uint32_t u = __float_as_uint(d);
+  if (u == 0x80000000u) u = 0u;
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float key_dist(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k); }
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+struct RoundShared {
+  unsigned long long full[kRingSlots];                    // mbarriers: the 32 lanes' copies of a row have landed
+  unsigned issued[kRingSlots];                            // rows a slot has carried for earlier clusters (its barrier's phases)
+  int warp_tot[kRoundWarps];
+  int n_mine, size, next;
+  int failed;
+  int arena_at;
+  volatile int done;                                      // candidates before it are decided: their rows are free
+  uint16_t mine[kMineCap];                                // the medoids this CTA grows in this round
+  uint16_t member[kFastCand + 1];
 };
 
-__global__ void __launch_bounds__(kExpandThreads) expand_kernel(ExpandArgs a) {
-  __shared__ int s_warp[32];
-  __shared__ int s_total, s_next, s_newly;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = a.n;
-  pdl_wait();                                             // the queue comes from the previous kernel
-  for (int i = tid; i < n; i += kExpandThreads) a.covered[i] = 0;
-  if (tid == 0) a.ptr[0] = 0;
+// Exclusive prefix of v over the CTA and the total (two barriers).
+__device__ __forceinline__ int block_prefix(RoundShared& sh, int v, int& total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane >= o) incl += t;
+  }
   __syncthreads();
-  int n_cov = 0, n_clu = 0;
-  long long fill = 0;
-  bool overflow = false;
-  for (int qi = 0; qi < n && n_cov < n && !overflow; ++qi) {
-    const int m = a.queue[qi];
-    if (a.covered[m]) continue;                           // uniform: every thread reads the same byte
-    const float* row_m = a.dist + (long long)m * n;
+  if (lane == 31) sh.warp_tot[warp] = incl;
+  __syncthreads();
+  int before = 0;
+  total = 0;
+#pragma unroll
+  for (int w = 0; w < kRoundWarps; ++w) {
+    if (w < warp) before += sh.warp_tot[w];
+    total += sh.warp_tot[w];
+  }
+  return before + incl - v;
+}
 
-    // ---- candidates in index order (ordered compaction, chunks of kExpandThreads entries) ----
-    int n_cand = 0;
-    for (int base = 0; base < n; base += kExpandThreads) {
-      const int e = base + tid;
-      const bool is_cand = e < n && e != m && row_m[e] <= a.tau;
-      const unsigned bal = __ballot_sync(0xFFFFFFFFu, is_cand);
-      if (lane == 0) s_warp[warp] = __popc(bal);
-      __syncthreads();
-      int before = 0, total = 0;
-      for (int w = 0; w < kExpandThreads / 32; ++w) {
-        const int c = s_warp[w];
-        if (w < warp) before += c;
-        total += c;
-      }
-      if (is_cand) a.cand_raw[n_cand + before + __popc(bal & ((1u << lane) - 1u))] = e;
-      n_cand += total;
-      __syncthreads();
-    }
-    // ---- place them by (distance to the medoid, index); the sum starts as that distance ----
-    for (int i = tid; i < n_cand; i += kExpandThreads) {
-      const int e = a.cand_raw[i];
-      const float de = row_m[e];
-      int place = 0;
-      for (int j = 0; j < n_cand; ++j) {
-        const int o = a.cand_raw[j];
-        const float d_o = row_m[o];
-        place += (d_o < de) || (d_o == de && o < e);
-      }
-      a.cand[place] = e;
-      a.sum[place] = de;
-    }
-    __syncthreads();
+// Every CTA of the (cooperative) grid has arrived for the nth time; false when that wait, or one inside a CTA, ran out.
+__device__ __forceinline__ bool grid_barrier(const ClusterArgs& a, RoundShared& sh, unsigned nth) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned* p = a.ctl + kCtlArrived;
+    if (sh.failed) atomicExch(a.ctl + kCtlFailed, 1u);
+    red_release_add(p, 1u);
+    const unsigned target = nth * gridDim.x;
+    unsigned polls = 0, v = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    } while ((int)(v - target) < 0 && ++polls < kGridWaitLimit);
+    if ((int)(v - target) < 0) atomicExch(a.ctl + kCtlFailed, 1u);
+    if (*reinterpret_cast<volatile unsigned*>(a.ctl + kCtlFailed) != 0u) sh.failed = 1;
+  }
+  __syncthreads();
+  return sh.failed == 0;
+}
 
-    // ---- greedy joins ----
-    if (fill + 1 > a.members_cap) { overflow = true; break; }
-    if (tid == 0) a.members[fill] = m;
-    int size = 1, from = 0;                               // members so far; candidates before `from` are decided
-    while (from < n_cand) {
-      const float bound = a.tau * (float)size;
-      int first = n_cand;                                 // first undecided candidate whose average passes
-      for (int i = from + tid; i < n_cand; i += kExpandThreads)
-        if (a.sum[i] <= bound) { first = i; break; }
-      first = __reduce_min_sync(0xFFFFFFFFu, first);
-      if (lane == 0) s_warp[warp] = first;
+// Ascending bitonic sort of (key, index) pairs, `m` a power of two.
+__device__ __forceinline__ void sort_pairs(uint32_t* key, uint16_t* idx, int m) {
+  for (int k = 2; k <= m; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
       __syncthreads();
-      if (warp == 0) {
-        int v = s_warp[lane];
-        v = __reduce_min_sync(0xFFFFFFFFu, v);
-        if (lane == 0) s_next = v;
+      for (int t = threadIdx.x; t < m / 2; t += kRoundThreads) {
+        const int lo = ((t & ~(j - 1)) << 1) | (t & (j - 1)), hi = lo | j;
+        const uint32_t ka = key[lo], kb = key[hi];
+        const uint16_t ia = idx[lo], ib = idx[hi];
+        const bool after = ka > kb || (ka == kb && ia > ib);
+        if (after == ((lo & k) == 0)) { key[lo] = kb; key[hi] = ka; idx[lo] = ib; idx[hi] = ia; }
       }
-      __syncthreads();
-      const int at = s_next;
-      if (at >= n_cand) break;
-      if (fill + size + 1 > a.members_cap) { overflow = true; break; }
-      const int e = a.cand[at];
-      if (tid == 0) a.members[fill + size] = e;
-      ++size;
-      const float* row_e = a.dist + (long long)e * n;
-      for (int i = at + 1 + tid; i < n_cand; i += kExpandThreads) a.sum[i] = a.sum[i] + row_e[a.cand[i]];
-      from = at + 1;
-      __syncthreads();
     }
-    if (overflow) break;
-    // ---- the cluster is final: cover its members ----
-    __syncthreads();
-    if (tid == 0) s_newly = 0;
-    __syncthreads();
-    int newly = 0;
-    for (int i = tid; i < size; i += kExpandThreads) {
-      const int e = a.members[fill + i];
-      if (!a.covered[e]) { a.covered[e] = 1; ++newly; }   // members of one cluster are distinct
+  }
+  __syncthreads();
+}
+
+// The joins of a cluster with at most 32 * NR candidates, by one warp: candidate 32 r + lane's running sum in s[r];
+// decided candidates hold NaN, which passes no bound.  Returns the cluster's size (members in sh.member), or -1 when a wait ran out.
+template <int NR>
+__device__ __forceinline__ int decide(const ClusterArgs& a, RoundShared& sh, const uint32_t* key, const uint16_t* idx,
+                                      const float* ring, int pitch, int slots, int n_cand) {
+  const int lane = threadIdx.x & 31;
+  const float decided = __int_as_float(0x7FFFFFFF);
+  float s[NR];
+#pragma unroll
+  for (int r = 0; r < NR; ++r) s[r] = 32 * r + lane < n_cand ? key_dist(key[32 * r + lane]) : decided;
+  int size = 1;
+  for (;;) {
+    const float bound = a.tau * (float)size;
+    int first = n_cand;
+#pragma unroll
+    for (int r = NR - 1; r >= 0; --r) first = s[r] <= bound ? 32 * r + lane : first;
+    const int at = __reduce_min_sync(0xFFFFFFFFu, first);
+    if (at >= n_cand) break;
+    if (lane == 0) {
+      sh.member[size] = idx[at];
+      sh.done = at;                                       // rows in front of `at` are not needed any more
     }
-    if (newly) atomicAdd(&s_newly, newly);
-    __syncthreads();
-    n_cov += s_newly;
-    fill += size;
-    if (tid == 0) {
-      a.medoid[n_clu] = m;
-      a.ptr[n_clu + 1] = (int32_t)fill;
+    ++size;
+    const int slot = at % slots;
+    unsigned polls = 0;
+    const uint32_t bar = smem_u32(&sh.full[slot]);
+    const unsigned parity = (sh.issued[slot] + (unsigned)(at / slots)) & 1u;
+    unsigned ok = 0u;
+    do {
+      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                   : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    } while (!ok && ++polls < kRingWaitLimit);
+    if (__any_sync(0xFFFFFFFFu, !ok)) return -1;
+    const float* row = ring + slot * pitch + lane;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (32 * r + 31 > at && 32 * r < n_cand) {          // (uniform)
+        const int i = 32 * r + lane;
+        const float v = i < n_cand && i > at ? row[32 * r] : 0.f;
+        s[r] = i > at ? s[r] + v : decided;
+      } else {
+        s[r] = decided;
+      }
     }
-    ++n_clu;
+  }
+  return size;
+}
+
+// One of the other warps (number w of kFetchWarps): rows of candidates w, w + kFetchWarps, ... into the ring.
+// Returns the first row of its own it has not issued.
+__device__ __forceinline__ int fetch_rows(const ClusterArgs& a, RoundShared& sh, const uint16_t* idx, float* ring,
+                                           int pitch, int slots, int n_cand, int w) {
+  const int lane = threadIdx.x & 31;
+  auto landed = [&](int j) -> bool {                      // row j's copies (bounded)
+    const int slot = j % slots;
+    const uint32_t bar = smem_u32(&sh.full[slot]);
+    const unsigned parity = (sh.issued[slot] + (unsigned)(j / slots)) & 1u;
+    unsigned ok = 0u, polls = 0u;
+    do {
+      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                   : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    } while (!ok && ++polls < kRingWaitLimit);
+    return !__any_sync(0xFFFFFFFFu, !ok);
+  };
+  int j = w;
+  for (; j < n_cand; j += kFetchWarps) {
+    int go = 1;
+    if (lane == 0) {
+      unsigned polls = 0;
+      while (sh.done <= j - slots && ++polls < kRingWaitLimit) __nanosleep(20);
+      if (sh.done <= j - slots) sh.failed = 1;
+      go = sh.done > j - slots && sh.done < n_cand;
+    }
+    if (!__shfl_sync(0xFFFFFFFFu, go, 0)) break;
+    if (j >= slots && !landed(j - slots)) { sh.failed = 1; break; }
+    const float* row = a.dist + (long long)idx[j] * a.n;
+    float* dst = ring + (j % slots) * pitch;
+    for (int i = ((j + 1) & ~31) + lane; i < n_cand; i += 32)
+      if (i > j) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + i)), "l"(row + idx[i]) : "memory");
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sh.full[j % slots])) : "memory");
+  }
+  // the last rows issued (one per slot of this warp) may still be in flight: nothing may land behind the cluster
+  for (int b = j - slots; b < j; b += kFetchWarps)
+    if (b >= 0 && !landed(b)) sh.failed = 1;
+  return j;
+}
+
+// Grows the cluster of medoid m (all threads of the CTA).  Returns its size; member(i), i >= 1, is in `*members`
+// (shared memory).  `smem`: the CTA's dynamic shared memory.
+__device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, int sort_cap, int m, const uint16_t** members) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = a.n, words = adj_words(n);
+  uint32_t* key = reinterpret_cast<uint32_t*>(smem);
+  const uint32_t* bits = a.adj + (long long)m * words;
+  const float* row_m = a.dist + (long long)m * n;
+
+  // ---- candidates, their keys, the sort ----
+  const int n_cand = a.rho[m];
+  const bool fast = n_cand <= kFastCand;
+  uint16_t* idx = reinterpret_cast<uint16_t*>(smem + (fast ? kFastCand : sort_cap) * 4);
+  int base = 0;
+  for (int w0 = 0; w0 < words; w0 += kRoundThreads) {
+    uint32_t b = w0 + tid < words ? bits[w0 + tid] : 0u;
+    int total;
+    int at = base + block_prefix(sh, __popc(b), total);
+    for (; b; b &= b - 1u) {
+      const int e = adj_column(w0 + tid, __ffs(b) - 1);
+      idx[at] = (uint16_t)e;
+      key[at] = dist_key(row_m[e]);
+      ++at;
+    }
+    base += total;
+  }
+  int m2 = 1;
+  while (m2 < n_cand) m2 <<= 1;
+  for (int i = n_cand + tid; i < m2; i += kRoundThreads) { key[i] = 0xFFFFFFFFu; idx[i] = 0xFFFFu; }
+  if (m2 > 1) sort_pairs(key, idx, m2);
+  else __syncthreads();
+
+  if (fast) {
+    float* ring = reinterpret_cast<float*>(smem + kFastCand * 6);
+    const int pitch = max(32, (n_cand + 31) & ~31);
+    const int slots = min(kRingSlots / kFetchWarps, kRingBytes / (pitch * 4) / kFetchWarps) * kFetchWarps;
+    int next_row = 0;
+    if (tid == 0) sh.done = 0;
+    __syncthreads();
+    if (warp == 0) {
+      int size;
+      if (n_cand <= 128) size = decide<4>(a, sh, key, idx, ring, pitch, slots, n_cand);
+      else if (n_cand <= 256) size = decide<8>(a, sh, key, idx, ring, pitch, slots, n_cand);
+      else if (n_cand <= 512) size = decide<16>(a, sh, key, idx, ring, pitch, slots, n_cand);
+      else size = decide<32>(a, sh, key, idx, ring, pitch, slots, n_cand);
+      if (lane == 0) {
+        sh.done = 0x7FFFFFFF;
+        sh.size = size;
+        if (size < 0) sh.failed = 1;
+      }
+    } else {
+      next_row = fetch_rows(a, sh, idx, ring, pitch, slots, n_cand, warp - 1);
+    }
+    __syncthreads();
+    if (warp > 0 && lane == 0)                            // the phases the barriers of this warp's slots went through
+      for (int slot = warp - 1; slot < slots && slot < next_row; slot += kFetchWarps)
+        sh.issued[slot] += (unsigned)((next_row - 1 - slot) / slots + 1);
+    *members = sh.member;
+    return max(sh.size, 1);
+  }
+
+  // ---- more candidates than one warp holds: the whole CTA decides, sums in place of the keys ----
+  float* sum = reinterpret_cast<float*>(key);
+  for (int i = tid; i < n_cand; i += kRoundThreads) sum[i] = key_dist(key[i]);
+  __syncthreads();
+  int size = 1, from = 0;                                 // members so far; candidates before `from` are decided
+  while (from < n_cand) {
+    const float bound = a.tau * (float)size;
+    int first = n_cand;
+    for (int i = from + tid; i < n_cand; i += kRoundThreads)
+      if (sum[i] <= bound) { first = i; break; }
+    first = __reduce_min_sync(0xFFFFFFFFu, first);
+    if (lane == 0) sh.warp_tot[warp] = first;
+    __syncthreads();
+    int at = n_cand;
+#pragma unroll
+    for (int w = 0; w < kRoundWarps; ++w) at = min(at, sh.warp_tot[w]);
+    if (at >= n_cand) break;
+    const uint16_t e = idx[at];
+    __syncthreads();                                      // everyone has read warp_tot and idx[at]
+    if (tid == 0) idx[size - 1] = e;                      // members take the places of decided candidates
+    ++size;
+    const float* row_e = a.dist + (long long)e * n;
+    for (int i = at + 1 + tid; i < n_cand; i += kRoundThreads) sum[i] = sum[i] + row_e[idx[i]];
+    from = at + 1;
     __syncthreads();
   }
-  if (tid == 0) {
-    *a.n_clusters = n_clu;
-    *a.dev_status = overflow ? 1 : 0;
+  __syncthreads();
+  *members = idx - 1;
+  return size;
+}
+
+__global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a, int sort_cap) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ RoundShared sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = a.n, words = adj_words(n), bwords = bit_words(n);
+  if (tid < kRingSlots) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sh.full[tid])), "r"(32));
+    sh.issued[tid] = 0u;
+  }
+  if (tid == 0) { sh.failed = 0; sh.done = 0; }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  __syncthreads();
+  // marking phase: the covered bits and this CTA's marks
+  uint32_t* s_cov = reinterpret_cast<uint32_t*>(dyn);
+  uint32_t* s_blk = s_cov + bwords;
+  unsigned nth = 0;
+  bool fine = true;
+
+  for (int round = 0; fine; ++round) {
+    uint32_t* blocked = a.blocked + (round & 1) * bwords;
+    uint32_t* blocked_next = a.blocked + ((round + 1) & 1) * bwords;
+    // ---- who may still be covered by an earlier entry ----
+    int open = 0;
+    for (int w = tid; w < bwords; w += kRoundThreads) {
+      const uint32_t c = __ldcg(a.covered + w), all = w * 32 + 32 <= n ? 0xFFFFFFFFu : (1u << (n - w * 32)) - 1u;
+      s_cov[w] = c;
+      s_blk[w] = 0u;
+      open |= (c & all) != all;
+    }
+    if (!__syncthreads_or(open)) break;                   // (uniform over the grid: nobody covers before the next barrier)
+    for (int u = blockIdx.x * kRoundWarps + warp; u < n; u += gridDim.x * kRoundWarps) {
+      if ((s_cov[u >> 5] >> (u & 31)) & 1u) continue;
+      const int rho_u = a.rho[u];
+      const uint32_t* bits = a.adj + (long long)u * words;
+      for (int w = lane; w < words; w += 32) {
+        for (uint32_t b = __ldg(bits + w); b; b &= b - 1u) {
+          const int e = adj_column(w, __ffs(b) - 1);
+          const uint32_t bit = 1u << (e & 31);
+          if ((s_cov[e >> 5] | s_blk[e >> 5]) & bit) continue;
+          const int rho_e = a.rho[e];
+          if (rho_u > rho_e || (rho_u == rho_e && u < e)) atomicOr(&s_blk[e >> 5], bit);
+        }
+      }
+    }
+    __syncthreads();
+    for (int w = tid; w < bwords; w += kRoundThreads)
+      if (s_blk[w]) atomicOr(blocked + w, s_blk[w]);
+    if (!(fine = grid_barrier(a, sh, ++nth))) break;
+    // ---- the medoids of this round, dealt to the CTAs ----
+    if (tid == 0) sh.n_mine = 0;
+    int base = 0;
+    for (int w0 = 0; w0 < bwords; w0 += kRoundThreads) {
+      const int w = w0 + tid;
+      uint32_t b = 0u;
+      if (w < bwords) {
+        const uint32_t all = w * 32 + 32 <= n ? 0xFFFFFFFFu : (1u << (n - w * 32)) - 1u;
+        b = all & ~__ldcg(blocked + w) & ~s_cov[w];
+      }
+      int total;
+      int rank = base + block_prefix(sh, __popc(b), total);
+      for (; b; b &= b - 1u, ++rank) {
+        // (what does not fit the list stays open and comes up in the next round)
+        if (rank % (int)gridDim.x == (int)blockIdx.x && rank / (int)gridDim.x < kMineCap) {
+          sh.mine[rank / (int)gridDim.x] = (uint16_t)(w * 32 + __ffs(b) - 1);
+          atomicMax(&sh.n_mine, rank / (int)gridDim.x + 1);
+        }
+      }
+      base += total;
+    }
+    for (int w = blockIdx.x * kRoundThreads + tid; w < bwords; w += gridDim.x * kRoundThreads) blocked_next[w] = 0u;
+    __syncthreads();
+    const int n_mine = sh.n_mine;
+    for (int k = 0; k < n_mine; ++k) {
+      const int m = sh.mine[k], rho_m = a.rho[m];
+      const uint16_t* members;
+      const int size = grow(a, sh, dyn, sort_cap, m, &members);
+      if (tid == 0) {
+        const unsigned slot = atomicAdd(a.ctl + kCtlClusters, 1u);
+        // (a full arena stays full: the start is only ever moved up while the cluster fits)
+        int at = (int)atomicAdd(a.ctl + kCtlArena, 0u);
+        while (at + size <= a.arena_cap) {
+          const int seen = (int)atomicCAS(a.ctl + kCtlArena, (unsigned)at, (unsigned)(at + size));
+          if (seen == at) break;
+          at = seen;
+        }
+        sh.arena_at = at + size <= a.arena_cap ? at : -1;
+        a.tab_medoid[slot] = m;
+        a.tab_size[slot] = size;
+        a.tab_at[slot] = sh.arena_at;
+        atomicOr(a.covered + (m >> 5), 1u << (m & 31));
+      }
+      __syncthreads();
+      const int at = sh.arena_at;
+      for (int i = 1 + tid; i < size; i += kRoundThreads) {
+        const int e = members[i];
+        if (at >= 0) a.arena[at + i] = e;
+        // (an entry in front of the medoid is decided before it: with an asymmetric matrix it may still be open)
+        const int rho_e = a.rho[e];
+        if (rho_m > rho_e || (rho_m == rho_e && m < e)) atomicOr(a.covered + (e >> 5), 1u << (e & 31));
+      }
+      __syncthreads();
+    }
+    fine = grid_barrier(a, sh, ++nth);
+  }
+
+  // ---- output: clusters in queue order ----
+  if (!fine || __ldcg(a.ctl + kCtlFailed) != 0u) {
+    if (tid == 0 && blockIdx.x == 0) { *a.n_clusters = 0; *a.dev_status = 2; }
+    return;
+  }
+  const int n_clu = (int)__ldcg(a.ctl + kCtlClusters);
+  if (blockIdx.x == 0 && tid == 0) a.ptr[0] = 0;
+  for (int c = blockIdx.x; c < n_clu; c += gridDim.x) {
+    const int m = __ldcg(a.tab_medoid + c), rho_m = a.rho[m];
+    int before = 0;                                       // clusters in front of this one, and their members
+    long long fill = 0;
+    for (int o = tid; o < n_clu; o += kRoundThreads) {
+      const int mo = __ldcg(a.tab_medoid + o), rho_o = a.rho[mo];
+      if (rho_o > rho_m || (rho_o == rho_m && mo < m)) { ++before; fill += __ldcg(a.tab_size + o); }
+    }
+    __shared__ int s_before[kRoundWarps];
+    __shared__ long long s_fill[kRoundWarps];
+    __syncthreads();
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+      fill += __shfl_xor_sync(0xFFFFFFFFu, fill, o);
+    }
+    if (lane == 0) { s_before[warp] = before; s_fill[warp] = fill; }
+    __syncthreads();
+    before = 0;
+    fill = 0;
+    for (int w = 0; w < kRoundWarps; ++w) { before += s_before[w]; fill += s_fill[w]; }
+    const int size = __ldcg(a.tab_size + c), at = __ldcg(a.tab_at + c);
+    if (fill + size <= a.members_cap) {
+      if (tid == 0) {
+        a.medoid[before] = m;
+        a.ptr[before + 1] = (int32_t)(fill + size);
+        a.members[fill] = m;
+        if (before == n_clu - 1) { *a.n_clusters = n_clu; *a.dev_status = 0; }
+      }
+      if (at >= 0) {
+        for (int i = 1 + tid; i < size; i += kRoundThreads) a.members[fill + i] = __ldcg(a.arena + at + i);
+      } else {
+        const uint16_t* members;
+        grow(a, sh, dyn, sort_cap, m, &members);
+        for (int i = 1 + tid; i < size; i += kRoundThreads) a.members[fill + i] = members[i];
+        __syncthreads();
+      }
+    } else if (fill <= a.members_cap && tid == 0) {       // the first cluster that does not fit ends the output
+      *a.n_clusters = before;
+      *a.dev_status = 1;
+    }
   }
 }
 
@@ -190,78 +531,152 @@ __global__ void __launch_bounds__(kExpandThreads) expand_kernel(ExpandArgs a) {
 // ---- admission to the fast tier (Sec. 4.2, Tier 1 (3)): clusters in descending Eq. 6 score while they fit -------
 namespace {
 
-// order[place] = c with place = #{ j : score[j] > score[c] or (score[j] == score[c] and j < c) }
-__global__ void __launch_bounds__(256)
-score_order_kernel(const float* __restrict__ score, int n, int32_t* __restrict__ order) {
-  __shared__ float s_sc[2048];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const float mine = i < n ? score[i] : 0.f;
-  int place = 0;
-  for (int base = 0; base < n; base += 2048) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < 2048 && base + t < n; t += blockDim.x) s_sc[t] = score[base + t];
-    __syncthreads();
-    const int lim = min(2048, n - base);
-    for (int t = 0; t < lim; ++t) {
-      const float other = s_sc[t];
-      place += (other > mine) || (other == mine && base + t < i);
-    }
-  }
-  if (i < n) order[place] = i;
-}
+constexpr int kAdmitThreads = 1024;
+constexpr int kAdmitBins = 4096;
+constexpr int kAdmitDigit = 12;
 
-// One CTA walks the order: running page count by a block scan per chunk; a cluster is admitted while the count
-// stays within the capacity, and the first one that does not fit ends the admission (everything after it is out).
-__global__ void __launch_bounds__(1024)
-admit_kernel(const int32_t* __restrict__ order, const uint16_t* __restrict__ size, int n, long long capacity,
+// The admitted set is everything above a threshold score plus, in index order, the first clusters at it, so nothing has
+// to be sorted: a radix select whose bins hold pages instead of counts finds the score at which the running page count
+// leaves the capacity (12-bit digits relative to the scores' own range), an ordered scan the place inside its ties.
+// One CTA; latency-bound, n * 4 bytes from L2 per level.  (A full sort by counting took n^2 compares: 84 + 20 us at
+// 7 K clusters.)
+__global__ void __launch_bounds__(kAdmitThreads)
+admit_kernel(const float* __restrict__ score, const uint16_t* __restrict__ size, int n, long long capacity,
              uint8_t* __restrict__ resident, int32_t* __restrict__ info) {
-  __shared__ long long s_warp[32];
-  __shared__ long long s_used_final;
-  __shared__ int s_first_out;
+  __shared__ uint32_t hist[kAdmitBins];                    // pages per digit (at most 65536 * 65535 in all)
+  __shared__ uint32_t s_warp[32], s_lo[32], s_hi[32];
+  __shared__ uint32_t s_base;
+  __shared__ int s_bits, s_all, s_admitted;
+  __shared__ long long s_left;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  pdl_wait();
-  long long used = 0;                                      // pages of the clusters before the current chunk
-  int admitted = 0;
-  bool closed = false;
-  for (int base = 0; base < n; base += 1024) {
-    const int r = base + tid;
-    const int c = r < n ? order[r] : -1;
-    const long long mine = c >= 0 ? (long long)size[c] : 0;
-    long long incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (tid == 0) s_first_out = 1 << 30;
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    long long before = used;
-    for (int w = 0; w < warp; ++w) before += s_warp[w];
-    const bool fits = !closed && c >= 0 && before + incl <= capacity;
-    if (c >= 0 && !fits) atomicMin(&s_first_out, r);
-    __syncthreads();
-    const int first_out = s_first_out;                     // rank of the first cluster that does not fit (if any)
-    const bool in = c >= 0 && !closed && r < first_out;
-    if (c >= 0) resident[c] = in ? 1 : 0;
-    if (!closed) {
-      if (first_out < (1 << 30)) {
-        if (r == first_out) s_used_final = before + incl - mine;   // pages used when the admission ended
-        admitted += first_out - base;
-      } else {
-        for (int w = 0; w < 32; ++w) used += s_warp[w];
-        admitted += min(1024, n - base);
+  auto key_of = [&](int c) -> uint32_t {
+    uint32_t u = __float_as_uint(__ldg(score + c));
+    if (u == 0x80000000u) u = 0u;
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  };
+  for (int i = tid; i < kAdmitBins; i += kAdmitThreads) hist[i] = 0u;
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll 4
+  for (int c = tid; c < n; c += kAdmitThreads) {
+    const uint32_t k = key_of(c);
+    lo = min(lo, k);
+    hi = max(hi, k);
+  }
+  lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+  hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+  if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+  __syncthreads();
+  if (warp == 0) {
+    lo = __reduce_min_sync(0xFFFFFFFFu, s_lo[lane]);
+    hi = __reduce_max_sync(0xFFFFFFFFu, s_hi[lane]);
+    if (lane == 0) { s_base = lo; s_bits = 32 - __clz(hi - lo); s_left = capacity; s_all = 0; s_admitted = 0; }
+  }
+  __syncthreads();
+
+  // s_left: capacity behind everything above the candidates, which are the keys with key - base < 2^bits
+  for (bool first = true; first || s_bits > 0; first = false) {
+    const uint32_t base = s_base;
+    const int bits = s_bits, shift = max(bits - kAdmitDigit, 0);
+    const long long left = s_left;
+    const uint32_t width_m1 = bits >= 32 ? 0xFFFFFFFFu : ((1u << bits) - 1u);
+#pragma unroll 4
+    for (int c = tid; c < n; c += kAdmitThreads) {
+      const uint32_t rel = key_of(c) - base;
+      // bin b from the top at word (b % 4) * threads + b / 4: thread t owns bins 4t .. 4t + 3
+      if (rel <= width_m1) {
+        const uint32_t b = (uint32_t)(kAdmitBins - 1) - (rel >> shift);
+        atomicAdd(&hist[(b & 3u) * kAdmitThreads + (b >> 2)], (uint32_t)size[c]);
       }
     }
     __syncthreads();
-    if (!closed && first_out < (1 << 30)) {
-      used = s_used_final;
-      closed = true;
+    uint32_t p[4], sum = 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      p[j] = hist[j * kAdmitThreads + tid];
+      hist[j * kAdmitThreads + tid] = 0u;
+      sum += p[j];
     }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t before = 0u, total = 0u;
+    {
+      const uint32_t v = s_warp[lane];
+      total = __reduce_add_sync(0xFFFFFFFFu, v);
+      before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? v : 0u);
+    }
+    long long above = (long long)before + incl - sum;
+    if ((long long)total <= left) {                        // (only at the first level: everything fits)
+      if (tid == 0) { s_all = 1; s_left = left - total; s_bits = 0; }
+    } else if (above <= left && left < above + sum) {      // one thread holds the bin in which the capacity ends
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (above <= left && left < above + p[j]) {
+          s_base = base + ((uint32_t)(kAdmitBins - 1 - (4 * tid + j)) << shift);
+          s_bits = shift;
+          s_left = left - above;
+          break;
+        }
+        above += p[j];
+      }
+    }
+    __syncthreads();
   }
-  if (tid == 0 && info != nullptr) {
-    info[0] = admitted;
-    info[1] = (int32_t)min(used, 0x7FFFFFFFLL);
+
+  const uint32_t T = s_base;
+  const bool all = s_all != 0;
+  // ties at T in index order: warp w owns a contiguous span
+  const int seg = ((n + 31) / 32 + 31) & ~31;
+  const int w_lo = min(n, warp * seg), w_hi = min(n, w_lo + seg);
+  uint32_t ties = 0u;
+  if (!all) {
+#pragma unroll 4
+    for (int c = w_lo + lane; c < w_hi; c += 32)
+      if (key_of(c) == T) ties += size[c];
+  }
+  ties = __reduce_add_sync(0xFFFFFFFFu, ties);
+  if (lane == 0) s_warp[warp] = ties;
+  __syncthreads();
+  long long left = s_left;                                 // capacity left for this warp's ties
+  left -= (long long)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? s_warp[lane] : 0u);
+  __shared__ uint32_t s_tie_pages;
+  if (tid == 0) s_tie_pages = 0u;
+  __syncthreads();
+  int admitted = 0;
+  uint32_t tie_pages = 0u;
+  for (int c0 = w_lo; c0 < w_hi; c0 += 32) {
+    const int c = c0 + lane;
+    const uint32_t k = c < w_hi ? key_of(c) : 0u;
+    bool in = c < w_hi && (all || k > T);
+    const bool tie = !all && c < w_hi && k == T;
+    if (__any_sync(0xFFFFFFFFu, tie)) {
+      const uint32_t mine = tie ? size[c] : 0u;
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (tie && (long long)incl <= left) { in = true; tie_pages += mine; }
+      left -= (long long)__shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+    if (c < w_hi) resident[c] = in ? 1 : 0;
+    admitted += in;
+  }
+  if (info != nullptr) {
+    admitted = __reduce_add_sync(0xFFFFFFFFu, admitted);
+    tie_pages = __reduce_add_sync(0xFFFFFFFFu, tie_pages);
+    if (lane == 0) { atomicAdd(&s_admitted, admitted); atomicAdd(&s_tie_pages, tie_pages); }
+    __syncthreads();
+    if (tid == 0) {
+      info[0] = s_admitted;
+      info[1] = (int32_t)min(capacity - s_left + (long long)s_tie_pages, 0x7FFFFFFFLL);
+    }
   }
 }
 
@@ -271,41 +686,65 @@ long long cache_admit_workspace_bytes(int n) { return ((long long)n * 4 + 255) /
 
 cudaError_t launch_cache_admit(const float* score, const uint16_t* size, int n, long long capacity, void* workspace,
                                uint8_t* resident, int32_t* info, cudaStream_t st) {
-  int32_t* order = static_cast<int32_t*>(workspace);
-  score_order_kernel<<<dim3((n + 255) / 256), dim3(256), 0, st>>>(score, n, order);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_pdl(admit_kernel, dim3(1), dim3(1024), 0, st, true, order, size, n, capacity, resident, info);
+  (void)workspace;                                         // nothing is sorted any more
+  admit_kernel<<<dim3(1), dim3(kAdmitThreads), 0, st>>>(score, size, n, capacity, resident, info);
+  return cudaGetLastError();
 }
 
+namespace {
+long long padded(long long bytes) { return (bytes + 255) / 256 * 256; }
+int arena_entries(int n) { return 16 * n; }
+}  // namespace
+
 long long build_clusters_workspace_bytes(int n) {
-  // queue, cand_raw, cand (int32), sum (float), covered (bytes), each padded to 256 bytes
-  const long long words = ((long long)n * 4 + 255) / 256 * 256;
-  return 4 * words + ((long long)n + 255) / 256 * 256;
+  const long long b = bit_words(n);
+  return padded(4LL * n * adj_words(n)) + padded(4 * b) + padded(8 * b) + padded(4 * kCtlWords) + 3 * padded(4LL * n) +
+         padded(4LL * arena_entries(n));
 }
 
 cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* workspace, int32_t* rho, int32_t* ptr,
                                   int32_t* members, long long members_cap, int32_t* medoid, int32_t* n_clusters,
                                   int32_t* dev_status, cudaStream_t st) {
-  const long long words = ((long long)n * 4 + 255) / 256 * 256;
   char* ws = static_cast<char*>(workspace);
-  ExpandArgs a;
-  a.dist = dist; a.n = n; a.tau = tau;
-  int32_t* queue = reinterpret_cast<int32_t*>(ws);
-  a.queue = queue;
-  a.cand_raw = reinterpret_cast<int32_t*>(ws + words);
-  a.cand = reinterpret_cast<int32_t*>(ws + 2 * words);
-  a.sum = reinterpret_cast<float*>(ws + 3 * words);
-  a.covered = reinterpret_cast<uint8_t*>(ws + 4 * words);
+  auto take = [&](long long bytes) { char* p = ws; ws += padded(bytes); return p; };
+  ClusterArgs a;
+  a.dist = dist; a.n = n; a.tau = tau; a.rho = rho;
+  a.adj = reinterpret_cast<uint32_t*>(take(4LL * n * adj_words(n)));
+  a.covered = reinterpret_cast<uint32_t*>(take(4LL * bit_words(n)));
+  a.blocked = reinterpret_cast<uint32_t*>(take(8LL * bit_words(n)));
+  a.ctl = reinterpret_cast<unsigned*>(take(4 * kCtlWords));
+  a.tab_medoid = reinterpret_cast<int32_t*>(take(4LL * n));
+  a.tab_size = reinterpret_cast<int32_t*>(take(4LL * n));
+  a.tab_at = reinterpret_cast<int32_t*>(take(4LL * n));
+  a.arena = reinterpret_cast<int32_t*>(take(4LL * arena_entries(n)));
+  a.arena_cap = arena_entries(n);
   a.ptr = ptr; a.members = members; a.members_cap = members_cap; a.medoid = medoid; a.n_clusters = n_clusters;
   a.dev_status = dev_status;
-  density_kernel<<<dim3((n + 7) / 8), dim3(256), 0, st>>>(dist, n, tau, rho);
-  cudaError_t e = cudaGetLastError();
+
+  int sort_cap = kFastCand;                                // power of two >= n: the candidates of one cluster
+  while (sort_cap < n) sort_cap <<= 1;
+  const int smem = std::max(kFastCand * 6 + kRingBytes, sort_cap * 6);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  queue_kernel<<<dim3((n + 255) / 256), dim3(256), 0, st>>>(rho, n, queue);
+  density_kernel<<<dim3((n + 7) / 8), dim3(256), 0, st>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_pdl(expand_kernel, dim3(1), dim3(kExpandThreads), 0, st, true, a);
+  // A round has far fewer medoids than entries; one CTA per 64 entries keeps the barriers of small problems short.
+  const int grid = std::max(1, std::min(sms, (n + 63) / 64));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kRoundThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;             // the rounds end in a barrier over the grid
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, rounds_kernel, a, sort_cap);
 }
 
 }  // namespace swarm

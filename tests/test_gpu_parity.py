@@ -885,6 +885,40 @@ def test_algorithm1_matches_oracle(n, topics, tau):
         assert n_clusters == 1 and n_members == n           # radius above every distance: one cluster
 
 
+@pytest.mark.parametrize("n,frac,symmetric", [(1, 0.5, True), (33, 0.5, False), (129, 0.9, False), (513, 0.45, True),
+                                              (1025, 0.999, True), (1026, 0.999, False), (1300, 0.9, True),
+                                              (2049, 0.03, False), (2304, 0.5, True)])
+def test_algorithm1_on_unstructured_distances(n, frac, symmetric):
+    """Uniform random distances, every candidate-list length of the growing kernel (up to 128, 256, 512, 1024 and more
+    candidates per medoid), asymmetric matrices, ties (distances on a grid of 1/512)."""
+    g = torch.Generator(device=DEV).manual_seed(n)
+    dist = torch.randint(0, 512, (n, n), generator=g, device=DEV).to(torch.float32) / 512
+    if symmetric:
+        dist = torch.minimum(dist, dist.T).contiguous()
+        tau = 1.0 - (1.0 - frac) ** 0.5                     # a fraction `frac` of the entries lies within tau
+    else:
+        tau = frac
+    dist.fill_diagonal_(0.0)
+    rho, ptr_ref, members_ref, medoid_ref = oracle.build_clusters(dist.cpu().numpy(), tau, members_cap=400 * n)
+    density, ptr, members, medoid = B.swarm_build_clusters(dist, tau, members_cap=400 * n)
+    assert np.array_equal(density.cpu().numpy(), rho) and np.array_equal(medoid.cpu().numpy(), medoid_ref)
+    assert np.array_equal(ptr.cpu().numpy(), ptr_ref) and np.array_equal(members.cpu().numpy(), members_ref)
+    if len(members_ref) > n:                                # one place too few: flagged, nothing written past the end
+        with pytest.raises(B.SwarmError):
+            B.swarm_build_clusters(dist, tau, members_cap=max(n, len(members_ref) - 1))
+
+
+def test_algorithm1_with_more_members_than_the_scratch_holds():
+    """40 entries sit within reach of all 600, the others only of those: about 555 clusters of 41 members, more than the
+    scratch list's 16 per entry, so most clusters are grown a second time for the output."""
+    n, hubs, tau = 600, 40, 0.1
+    d = np.ones((n, n), dtype=np.float32)
+    d[:hubs, :] = d[:, :hubs] = 0.03125
+    np.fill_diagonal(d, 0.0)
+    n_clusters, n_members = check_clusters(torch.from_numpy(d).to(DEV), tau, cap=64 * n)
+    assert n_members > 16 * n and n_clusters > 500
+
+
 def test_algorithm1_hand_case_and_capacity():
     d = np.full((5, 5), 0.9, dtype=np.float32)
     np.fill_diagonal(d, 0.0)
