@@ -1,19 +1,17 @@
 // Algorithm 1: offline co-activation clustering on a given distance matrix (Sec. 4.1, Steps 3 and 4).
 //
-//   density_kernel   rho[i] = #{ j != i : D[i][j] <= tau } and the adjacency bits behind it -- one warp per row,
-//                    16-byte loads; the only pass over the whole n x n matrix, bound by HBM bandwidth (4 n^2 bytes read
-//                    once, n^2 / 8 written)
-//   rounds_kernel    everything else in one cooperative launch, see below
+//   density_kernel   rho[i] = #{ j != i : D[i][j] <= tau } -- one warp per row, 16-byte loads; the only pass over the
+//                    whole n x n matrix, bound by HBM bandwidth (4 n^2 bytes read once)
+//   rounds_kernel    everything else in one cooperative launch
 //
 // The listing walks the entries by (rho descending, index ascending) and grows a cluster from every entry that no
-// earlier cluster has covered.  Two facts make that walk parallel without changing a single decision:
-//   - what a cluster contains depends on its medoid and the matrix alone (covered entries remain candidates, which is
-//     where the paper's replicas come from), so clusters of different medoids can grow side by side;
-//   - the members of m's cluster lie within tau of m, so an uncovered entry that has no uncovered entry in front of it
-//     (in queue order) within tau is a medoid no matter what the others turn out to be.
-// The kernel works in rounds: mark every uncovered entry that an earlier uncovered one might still cover (adjacency
-// bits), grow the clusters of the unmarked ones -- one CTA each -- and cover their members behind them in the queue.  8192 entries in 64 topics:
-// 102 clusters in 12 rounds.  At the end every cluster's place in the output follows from the keys and sizes.
+// earlier cluster has covered.  What a cluster contains depends on its medoid and the matrix alone (covered entries
+// remain candidates, which is where the paper's replicas come from), so clusters can be grown before it is known
+// whether the walk will want them.  The kernel works in rounds: the next uncovered entries of the walk, one per CTA, are
+// all grown side by side, and each CTA notes which of the round's entries its cluster holds.  Behind a barrier every CTA
+// repeats the walk over those notes (a few hundred bits per step), which settles who is a medoid, and the medoids' CTAs
+// write their clusters to their final places.  Clusters that the walk does not want are dropped: they cost SMs that had
+// nothing else to do.  8192 entries in 64 topics: 102 clusters in 5 rounds.
 //
 // Growing one cluster: the candidates are sorted by (distance, index) in shared memory.  Between two joins neither the
 // running sums nor the bound tau * |C| change, so the next candidate to join is the first undecided one whose sum
@@ -29,27 +27,18 @@
 namespace swarm {
 namespace {
 
-// ---- adjacency bits ------------------------------------------------------------------------------------------
-// A row's bits come in blocks of 128 columns = 4 words: bit l of word c of block k stands for column 128 k + 4 l + c
-// (the lanes of a warp hold four neighbouring columns each, so a ballot per component is a word).
-__host__ __device__ inline int adj_words(int n) { return (n + 127) / 128 * 4; }
-__device__ __forceinline__ int adj_column(int word, int bit) { return (word >> 2) * 128 + 4 * bit + (word & 3); }
-
 struct ClusterArgs {
   const float* dist;
   int n;
   float tau;
   int32_t* rho;
   // scratch (see build_clusters_workspace_bytes)
-  uint32_t* adj;         // [n][adj_words(n)]
-  uint32_t* covered;     // bit e: entry e is covered
-  uint32_t* blocked;     // two arrays of such bits, used by alternate rounds
+  int32_t* queue;        // [n] entries in the order of the walk
+  int32_t* place;        // [n] and back: where an entry stands in it
+  uint32_t* covered;     // bit p: the entry at place p is covered
+  uint32_t* holds;       // [grid][kNoteWords] bit j of row i: the cluster grown by CTA i holds the round's entry j
+  int32_t* size;         // [grid] its size
   unsigned* ctl;         // kCtl* below
-  int32_t* tab_medoid;   // clusters in the order they were finished
-  int32_t* tab_size;
-  int32_t* tab_at;       // start in the arena, or -1: the arena was full, the cluster is grown again for the output
-  int32_t* arena;
-  int arena_cap;
   // outputs
   int32_t* ptr;
   int32_t* members;
@@ -58,45 +47,31 @@ struct ClusterArgs {
   int32_t* n_clusters;
   int32_t* dev_status;   // 0 ok, 1 members_cap too small, 2 a bounded wait ran out
 };
-constexpr int kCtlArrived = 0, kCtlClusters = 1, kCtlArena = 2, kCtlFailed = 3, kCtlWords = 64;
+constexpr int kCtlArrived = 0, kCtlFailed = 1, kCtlWords = 64;
+constexpr int kMaxPicks = 256;                            // entries grown per round: one per CTA
+constexpr int kNoteWords = kMaxPicks / 32;
 __host__ __device__ inline int bit_words(int n) { return (n + 31) / 32; }
 
 __global__ void __launch_bounds__(256) density_kernel(ClusterArgs a) {
   const int lane = threadIdx.x & 31, n = a.n;
   if (blockIdx.x == 0 && threadIdx.x < kCtlWords) a.ctl[threadIdx.x] = 0u;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < bit_words(n); i += gridDim.x * blockDim.x) {
-    a.covered[i] = 0u;
-    a.blocked[i] = a.blocked[bit_words(n) + i] = 0u;
-  }
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < bit_words(n); i += gridDim.x * blockDim.x) a.covered[i] = 0u;
   const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   if (row >= n) return;
   const float* r = a.dist + (long long)row * n;
-  uint32_t* bits = a.adj + (long long)row * adj_words(n);
   int cnt = 0;
-  const bool vec = (n & 3) == 0;                          // rows are 16-byte aligned
+  if ((n & 3) == 0) {                                     // rows are 16-byte aligned
 #pragma unroll 4
-  for (int j0 = 0; j0 < n; j0 += 128) {
-    const int j = j0 + lane * 4;
-    bool near[4] = {false, false, false, false};
-    if (vec) {
-      if (j < n) {
-        const uint4 v = ldg_nc_v4(r + j);
-        near[0] = __uint_as_float(v.x) <= a.tau; near[1] = __uint_as_float(v.y) <= a.tau;
-        near[2] = __uint_as_float(v.z) <= a.tau; near[3] = __uint_as_float(v.w) <= a.tau;
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) near[c] = j + c < n && __ldg(r + j + c) <= a.tau;
+    for (int j = lane * 4; j < n; j += 128) {
+      const uint4 v = ldg_nc_v4(r + j);
+      cnt += (__uint_as_float(v.x) <= a.tau && j != row) + (__uint_as_float(v.y) <= a.tau && j + 1 != row) +
+             (__uint_as_float(v.z) <= a.tau && j + 2 != row) + (__uint_as_float(v.w) <= a.tau && j + 3 != row);
     }
-    uint32_t mine = 0u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const uint32_t w = __ballot_sync(0xFFFFFFFFu, near[c] && j + c != row);
-      cnt += __popc(w);
-      if (lane == c) mine = w;
-    }
-    if (lane < 4) bits[j0 / 32 + lane] = mine;
+  } else {
+#pragma unroll 4
+    for (int j = lane; j < n; j += 32) cnt += (__ldg(r + j) <= a.tau && j != row);
   }
+  cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
   if (lane == 0) a.rho[row] = cnt;
 }
 
@@ -107,7 +82,6 @@ constexpr int kFastCand = 1024;                           // candidates one deci
 constexpr int kFetchWarps = kRoundWarps - 1;
 constexpr int kRingSlots = 4 * kFetchWarps;               // (a multiple of the fetching warps: every slot has one owner)
 constexpr int kRingBytes = 128 * 1024;
-constexpr int kMineCap = 1024;
 constexpr unsigned kGridWaitLimit = 1u << 23;
 constexpr unsigned kRingWaitLimit = 1u << 24;
 
@@ -125,11 +99,13 @@ struct RoundShared {
   unsigned long long full[kRingSlots];                    // mbarriers: the 32 lanes' copies of a row have landed
   unsigned issued[kRingSlots];                            // rows a slot has carried for earlier clusters (its barrier's phases)
   int warp_tot[kRoundWarps];
-  int n_mine, size, next;
+  int n_cand, size;
   int failed;
-  int arena_at;
   volatile int done;                                      // candidates before it are decided: their rows are free
-  uint16_t mine[kMineCap];                                // the medoids this CTA grows in this round
+  int pick[kMaxPicks];                                    // the round's entries, in the order of the walk
+  int pick_size[kMaxPicks];
+  uint32_t holds[kMaxPicks][kNoteWords];
+  uint32_t taken[kNoteWords];                             // the medoids among them
   uint16_t member[kFastCand + 1];
 };
 
@@ -278,37 +254,68 @@ __device__ __forceinline__ int fetch_rows(const ClusterArgs& a, RoundShared& sh,
   return j;
 }
 
-// Grows the cluster of medoid m (all threads of the CTA).  Returns its size; member(i), i >= 1, is in `*members`
-// (shared memory).  `smem`: the CTA's dynamic shared memory.
+// Grows the cluster of medoid m (all threads of the CTA).  Returns its size; member i >= 1 is (*members)[i] (shared
+// memory).  `smem`: the CTA's dynamic shared memory.
 __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, int sort_cap, int m, const uint16_t** members) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = a.n, words = adj_words(n);
-  uint32_t* key = reinterpret_cast<uint32_t*>(smem);
-  const uint32_t* bits = a.adj + (long long)m * words;
+  const int n = a.n;
   const float* row_m = a.dist + (long long)m * n;
-
-  // ---- candidates, their keys, the sort ----
   const int n_cand = a.rho[m];
   const bool fast = n_cand <= kFastCand;
+  // few candidates: (distance key << 32 | entry) pairs as collected, then sorted keys and entries; many: sorted in place
+  uint32_t* key = reinterpret_cast<uint32_t*>(smem);
   uint16_t* idx = reinterpret_cast<uint16_t*>(smem + (fast ? kFastCand : sort_cap) * 4);
-  int base = 0;
-  for (int w0 = 0; w0 < words; w0 += kRoundThreads) {
-    uint32_t b = w0 + tid < words ? bits[w0 + tid] : 0u;
-    int total;
-    int at = base + block_prefix(sh, __popc(b), total);
-    for (; b; b &= b - 1u) {
-      const int e = adj_column(w0 + tid, __ffs(b) - 1);
-      idx[at] = (uint16_t)e;
-      key[at] = dist_key(row_m[e]);
-      ++at;
+  uint64_t* raw = reinterpret_cast<uint64_t*>(smem + kFastCand * 6);   // (in the ring's place)
+
+  // ---- candidates in any order ----
+  if (tid == 0) sh.n_cand = 0;
+  __syncthreads();
+  auto append = [&](bool is, int e, float d) {            // (whole warps)
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, is);
+    if (bal == 0u) return;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&sh.n_cand, __popc(bal));
+    at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+    if (is && at < n_cand) {
+      if (fast) raw[at] = ((uint64_t)dist_key(d) << 32) | (uint32_t)e;
+      else { key[at] = dist_key(d); idx[at] = (uint16_t)e; }
     }
-    base += total;
+  };
+  if ((n & 3) == 0) {
+#pragma unroll 2
+    for (int j0 = warp * 128; j0 < n; j0 += kRoundThreads * 4) {
+      const int j = j0 + lane * 4;
+      const float4 v = j < n ? __ldg(reinterpret_cast<const float4*>(row_m + j)) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+      append(j < n && v.x <= a.tau && j != m, j, v.x);
+      append(j < n && v.y <= a.tau && j + 1 != m, j + 1, v.y);
+      append(j < n && v.z <= a.tau && j + 2 != m, j + 2, v.z);
+      append(j < n && v.w <= a.tau && j + 3 != m, j + 3, v.w);
+    }
+  } else {
+    for (int j0 = warp * 32; j0 < n; j0 += kRoundThreads) {
+      const int j = j0 + lane;
+      const float v = j < n ? __ldg(row_m + j) : 0.f;
+      append(j < n && v <= a.tau && j != m, j, v);
+    }
   }
-  int m2 = 1;
-  while (m2 < n_cand) m2 <<= 1;
-  for (int i = n_cand + tid; i < m2; i += kRoundThreads) { key[i] = 0xFFFFFFFFu; idx[i] = 0xFFFFu; }
-  if (m2 > 1) sort_pairs(key, idx, m2);
-  else __syncthreads();
+  __syncthreads();
+  // ---- sorted by (distance, index) ----
+  if (fast) {                                             // each candidate's place by counting the ones in front of it
+    for (int i = tid; i < n_cand; i += kRoundThreads) {
+      const uint64_t mine = raw[i];
+      int at = 0;
+#pragma unroll 8
+      for (int j = 0; j < n_cand; ++j) at += raw[j] < mine;
+      key[at] = (uint32_t)(mine >> 32);
+      idx[at] = (uint16_t)mine;
+    }
+    __syncthreads();
+  } else {
+    int m2 = 1;
+    while (m2 < n_cand) m2 <<= 1;
+    for (int i = n_cand + tid; i < m2; i += kRoundThreads) { key[i] = 0xFFFFFFFFu; idx[i] = 0xFFFFu; }
+    sort_pairs(key, idx, m2);
+  }
 
   if (fast) {
     float* ring = reinterpret_cast<float*>(smem + kFastCand * 6);
@@ -374,155 +381,122 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ RoundShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = a.n, words = adj_words(n), bwords = bit_words(n);
+  const int n = a.n, bwords = bit_words(n), G = gridDim.x, me = blockIdx.x;
   if (tid < kRingSlots) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sh.full[tid])), "r"(32));
     sh.issued[tid] = 0u;
   }
   if (tid == 0) { sh.failed = 0; sh.done = 0; }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  __syncthreads();
-  // marking phase: the covered bits and this CTA's marks
-  uint32_t* s_cov = reinterpret_cast<uint32_t*>(dyn);
-  uint32_t* s_blk = s_cov + bwords;
-  unsigned nth = 0;
-  bool fine = true;
+  if (me == 0 && tid == 0) a.ptr[0] = 0;
 
-  for (int round = 0; fine; ++round) {
-    uint32_t* blocked = a.blocked + (round & 1) * bwords;
-    uint32_t* blocked_next = a.blocked + ((round + 1) & 1) * bwords;
-    // ---- who may still be covered by an earlier entry ----
-    int open = 0;
-    for (int w = tid; w < bwords; w += kRoundThreads) {
-      const uint32_t c = __ldcg(a.covered + w), all = w * 32 + 32 <= n ? 0xFFFFFFFFu : (1u << (n - w * 32)) - 1u;
-      s_cov[w] = c;
-      s_blk[w] = 0u;
-      open |= (c & all) != all;
-    }
-    if (!__syncthreads_or(open)) break;                   // (uniform over the grid: nobody covers before the next barrier)
-    for (int u = blockIdx.x * kRoundWarps + warp; u < n; u += gridDim.x * kRoundWarps) {
-      if ((s_cov[u >> 5] >> (u & 31)) & 1u) continue;
-      const int rho_u = a.rho[u];
-      const uint32_t* bits = a.adj + (long long)u * words;
-      for (int w = lane; w < words; w += 32) {
-        for (uint32_t b = __ldg(bits + w); b; b &= b - 1u) {
-          const int e = adj_column(w, __ffs(b) - 1);
-          const uint32_t bit = 1u << (e & 31);
-          if ((s_cov[e >> 5] | s_blk[e >> 5]) & bit) continue;
-          const int rho_e = a.rho[e];
-          if (rho_u > rho_e || (rho_u == rho_e && u < e)) atomicOr(&s_blk[e >> 5], bit);
-        }
+  // ---- the order of the walk: a warp per entry counts the entries in front of it ----
+  for (int e = me * kRoundWarps + warp; e < n; e += G * kRoundWarps) {
+    const int mine = a.rho[e];
+    int at = 0;
+    for (int o0 = 0; o0 < n; o0 += 32 * 8) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int o = o0 + 32 * u + lane;
+        const int r = o < n ? a.rho[o] : -1;
+        at += r > mine || (r == mine && o < e);
       }
     }
-    __syncthreads();
-    for (int w = tid; w < bwords; w += kRoundThreads)
-      if (s_blk[w]) atomicOr(blocked + w, s_blk[w]);
-    if (!(fine = grid_barrier(a, sh, ++nth))) break;
-    // ---- the medoids of this round, dealt to the CTAs ----
-    if (tid == 0) sh.n_mine = 0;
-    int base = 0;
-    for (int w0 = 0; w0 < bwords; w0 += kRoundThreads) {
+    at = __reduce_add_sync(0xFFFFFFFFu, at);
+    if (lane == 0) { a.queue[at] = e; a.place[e] = at; }
+  }
+  unsigned nth = 0;
+  bool fine = grid_barrier(a, sh, ++nth);
+  int n_clu = 0, from = 0, status = 0;                     // clusters written; bitmap words before `from` are all covered
+  long long fill = 0;
+
+  while (fine) {
+    // ---- the round's entries: the first G uncovered ones ----
+    int n_picks = 0;
+    for (int w0 = from; w0 < bwords && n_picks < G; w0 += kRoundThreads) {
       const int w = w0 + tid;
       uint32_t b = 0u;
-      if (w < bwords) {
-        const uint32_t all = w * 32 + 32 <= n ? 0xFFFFFFFFu : (1u << (n - w * 32)) - 1u;
-        b = all & ~__ldcg(blocked + w) & ~s_cov[w];
-      }
+      if (w < bwords) b = (w * 32 + 32 <= n ? 0xFFFFFFFFu : (1u << (n - w * 32)) - 1u) & ~__ldcg(a.covered + w);
       int total;
-      int rank = base + block_prefix(sh, __popc(b), total);
-      for (; b; b &= b - 1u, ++rank) {
-        // (what does not fit the list stays open and comes up in the next round)
-        if (rank % (int)gridDim.x == (int)blockIdx.x && rank / (int)gridDim.x < kMineCap) {
-          sh.mine[rank / (int)gridDim.x] = (uint16_t)(w * 32 + __ffs(b) - 1);
-          atomicMax(&sh.n_mine, rank / (int)gridDim.x + 1);
-        }
+      int rank = n_picks + block_prefix(sh, __popc(b), total);
+      for (; b && rank < G; b &= b - 1u, ++rank) {
+        const int p = w * 32 + __ffs(b) - 1;
+        sh.pick[rank] = __ldcg(a.queue + p);
       }
-      base += total;
+      n_picks = min(G, n_picks + total);
     }
-    for (int w = blockIdx.x * kRoundThreads + tid; w < bwords; w += gridDim.x * kRoundThreads) blocked_next[w] = 0u;
     __syncthreads();
-    const int n_mine = sh.n_mine;
-    for (int k = 0; k < n_mine; ++k) {
-      const int m = sh.mine[k], rho_m = a.rho[m];
-      const uint16_t* members;
-      const int size = grow(a, sh, dyn, sort_cap, m, &members);
-      if (tid == 0) {
-        const unsigned slot = atomicAdd(a.ctl + kCtlClusters, 1u);
-        // (a full arena stays full: the start is only ever moved up while the cluster fits)
-        int at = (int)atomicAdd(a.ctl + kCtlArena, 0u);
-        while (at + size <= a.arena_cap) {
-          const int seen = (int)atomicCAS(a.ctl + kCtlArena, (unsigned)at, (unsigned)(at + size));
-          if (seen == at) break;
-          at = seen;
-        }
-        sh.arena_at = at + size <= a.arena_cap ? at : -1;
-        a.tab_medoid[slot] = m;
-        a.tab_size[slot] = size;
-        a.tab_at[slot] = sh.arena_at;
-        atomicOr(a.covered + (m >> 5), 1u << (m & 31));
-      }
+    if (n_picks == 0) break;                               // (uniform over the grid: nobody covers before the next barrier)
+    // ---- every CTA grows one and notes which of the others its cluster holds ----
+    int size = 0;
+    const uint16_t* members = nullptr;
+    if (me < n_picks) {
+      const int m = sh.pick[me];
+      size = grow(a, sh, dyn, sort_cap, m, &members);
+      // marks of the members (few candidates: in the place of the sorted keys, else behind everything)
+      const bool fast = a.rho[m] <= kFastCand;
+      uint32_t* mark = reinterpret_cast<uint32_t*>(dyn + (fast ? kFastCand * 6 : sort_cap * 6));
+      for (int w = tid; w < bwords; w += kRoundThreads) mark[w] = 0u;
       __syncthreads();
-      const int at = sh.arena_at;
+      for (int i = 1 + tid; i < size; i += kRoundThreads) atomicOr(&mark[members[i] >> 5], 1u << (members[i] & 31));
+      __syncthreads();
+      if (tid < kMaxPicks) {
+        const int e = tid < n_picks ? sh.pick[tid] : m;
+        const uint32_t w = __ballot_sync(0xFFFFFFFFu, tid < n_picks && ((mark[e >> 5] >> (e & 31)) & 1u));
+        if (lane == 0) a.holds[me * kNoteWords + warp] = w;
+      }
+      if (tid == 0) a.size[me] = size;
+    }
+    if (!(fine = grid_barrier(a, sh, ++nth))) break;
+    // ---- the walk over them ----
+    for (int i = tid; i < n_picks * kNoteWords; i += kRoundThreads) (&sh.holds[0][0])[i] = __ldcg(a.holds + i);
+    if (tid < n_picks) sh.pick_size[tid] = __ldcg(a.size + tid);
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t cov = 0u, taken = 0u;                       // lane w: word w of the entries covered and taken
+      for (int i = 0; i < n_picks; ++i) {
+        const uint32_t row = lane < kNoteWords ? sh.holds[i][lane] : 0u;
+        const uint32_t c = __shfl_sync(0xFFFFFFFFu, cov, i >> 5);
+        if (!((c >> (i & 31)) & 1u)) {
+          cov |= row;
+          if (lane == (i >> 5)) taken |= 1u << (i & 31);
+        }
+      }
+      if (lane < kNoteWords) sh.taken[lane] = taken;
+    }
+    __syncthreads();
+    // ---- where the taken ones go ----
+    int my_at = -1, my_clu = 0;
+    long long my_fill = 0;
+    for (int i = 0; i < n_picks && status == 0; ++i) {
+      if (!((sh.taken[i >> 5] >> (i & 31)) & 1u)) continue;
+      if (fill + sh.pick_size[i] > a.members_cap) { status = 1; break; }   // it and everything behind it are left out
+      if (i == me) { my_at = i; my_clu = n_clu; my_fill = fill; }
+      ++n_clu;
+      fill += sh.pick_size[i];
+    }
+    if (my_at >= 0) {
+      const int m = sh.pick[me];
+      if (tid == 0) {
+        a.medoid[my_clu] = m;
+        a.ptr[my_clu + 1] = (int32_t)(my_fill + size);
+        a.members[my_fill] = m;
+        const int p = a.place[m];
+        atomicOr(a.covered + (p >> 5), 1u << (p & 31));
+      }
       for (int i = 1 + tid; i < size; i += kRoundThreads) {
-        const int e = members[i];
-        if (at >= 0) a.arena[at + i] = e;
-        // (an entry in front of the medoid is decided before it: with an asymmetric matrix it may still be open)
-        const int rho_e = a.rho[e];
-        if (rho_m > rho_e || (rho_m == rho_e && m < e)) atomicOr(a.covered + (e >> 5), 1u << (e & 31));
+        const int e = members[i], p = a.place[e];
+        a.members[my_fill + i] = e;
+        atomicOr(a.covered + (p >> 5), 1u << (p & 31));
       }
-      __syncthreads();
     }
+    if (status != 0) break;                                // (uniform over the grid)
     fine = grid_barrier(a, sh, ++nth);
+    from = __ldcg(a.place + sh.pick[0]) >> 5;              // everything in front of this round's first entry is covered
   }
-
-  // ---- output: clusters in queue order ----
-  if (!fine || __ldcg(a.ctl + kCtlFailed) != 0u) {
-    if (tid == 0 && blockIdx.x == 0) { *a.n_clusters = 0; *a.dev_status = 2; }
-    return;
-  }
-  const int n_clu = (int)__ldcg(a.ctl + kCtlClusters);
-  if (blockIdx.x == 0 && tid == 0) a.ptr[0] = 0;
-  for (int c = blockIdx.x; c < n_clu; c += gridDim.x) {
-    const int m = __ldcg(a.tab_medoid + c), rho_m = a.rho[m];
-    int before = 0;                                       // clusters in front of this one, and their members
-    long long fill = 0;
-    for (int o = tid; o < n_clu; o += kRoundThreads) {
-      const int mo = __ldcg(a.tab_medoid + o), rho_o = a.rho[mo];
-      if (rho_o > rho_m || (rho_o == rho_m && mo < m)) { ++before; fill += __ldcg(a.tab_size + o); }
-    }
-    __shared__ int s_before[kRoundWarps];
-    __shared__ long long s_fill[kRoundWarps];
-    __syncthreads();
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-      before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
-      fill += __shfl_xor_sync(0xFFFFFFFFu, fill, o);
-    }
-    if (lane == 0) { s_before[warp] = before; s_fill[warp] = fill; }
-    __syncthreads();
-    before = 0;
-    fill = 0;
-    for (int w = 0; w < kRoundWarps; ++w) { before += s_before[w]; fill += s_fill[w]; }
-    const int size = __ldcg(a.tab_size + c), at = __ldcg(a.tab_at + c);
-    if (fill + size <= a.members_cap) {
-      if (tid == 0) {
-        a.medoid[before] = m;
-        a.ptr[before + 1] = (int32_t)(fill + size);
-        a.members[fill] = m;
-        if (before == n_clu - 1) { *a.n_clusters = n_clu; *a.dev_status = 0; }
-      }
-      if (at >= 0) {
-        for (int i = 1 + tid; i < size; i += kRoundThreads) a.members[fill + i] = __ldcg(a.arena + at + i);
-      } else {
-        const uint16_t* members;
-        grow(a, sh, dyn, sort_cap, m, &members);
-        for (int i = 1 + tid; i < size; i += kRoundThreads) a.members[fill + i] = members[i];
-        __syncthreads();
-      }
-    } else if (fill <= a.members_cap && tid == 0) {       // the first cluster that does not fit ends the output
-      *a.n_clusters = before;
-      *a.dev_status = 1;
-    }
+  if (me == 0 && tid == 0) {
+    *a.n_clusters = fine ? n_clu : 0;
+    *a.dev_status = fine ? status : 2;
   }
 }
 
@@ -693,13 +667,11 @@ cudaError_t launch_cache_admit(const float* score, const uint16_t* size, int n, 
 
 namespace {
 long long padded(long long bytes) { return (bytes + 255) / 256 * 256; }
-int arena_entries(int n) { return 16 * n; }
 }  // namespace
 
 long long build_clusters_workspace_bytes(int n) {
-  const long long b = bit_words(n);
-  return padded(4LL * n * adj_words(n)) + padded(4 * b) + padded(8 * b) + padded(4 * kCtlWords) + 3 * padded(4LL * n) +
-         padded(4LL * arena_entries(n));
+  return 2 * padded(4LL * n) + padded(4LL * bit_words(n)) + padded(4LL * kMaxPicks * kNoteWords) + padded(4LL * kMaxPicks) +
+         padded(4LL * kCtlWords);
 }
 
 cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* workspace, int32_t* rho, int32_t* ptr,
@@ -709,21 +681,18 @@ cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* wor
   auto take = [&](long long bytes) { char* p = ws; ws += padded(bytes); return p; };
   ClusterArgs a;
   a.dist = dist; a.n = n; a.tau = tau; a.rho = rho;
-  a.adj = reinterpret_cast<uint32_t*>(take(4LL * n * adj_words(n)));
+  a.queue = reinterpret_cast<int32_t*>(take(4LL * n));
+  a.place = reinterpret_cast<int32_t*>(take(4LL * n));
   a.covered = reinterpret_cast<uint32_t*>(take(4LL * bit_words(n)));
-  a.blocked = reinterpret_cast<uint32_t*>(take(8LL * bit_words(n)));
-  a.ctl = reinterpret_cast<unsigned*>(take(4 * kCtlWords));
-  a.tab_medoid = reinterpret_cast<int32_t*>(take(4LL * n));
-  a.tab_size = reinterpret_cast<int32_t*>(take(4LL * n));
-  a.tab_at = reinterpret_cast<int32_t*>(take(4LL * n));
-  a.arena = reinterpret_cast<int32_t*>(take(4LL * arena_entries(n)));
-  a.arena_cap = arena_entries(n);
+  a.holds = reinterpret_cast<uint32_t*>(take(4LL * kMaxPicks * kNoteWords));
+  a.size = reinterpret_cast<int32_t*>(take(4LL * kMaxPicks));
+  a.ctl = reinterpret_cast<unsigned*>(take(4LL * kCtlWords));
   a.ptr = ptr; a.members = members; a.members_cap = members_cap; a.medoid = medoid; a.n_clusters = n_clusters;
   a.dev_status = dev_status;
 
   int sort_cap = kFastCand;                                // power of two >= n: the candidates of one cluster
   while (sort_cap < n) sort_cap <<= 1;
-  const int smem = std::max(kFastCand * 6 + kRingBytes, sort_cap * 6);
+  const int smem = std::max(kFastCand * 6 + kRingBytes, sort_cap * 6 + bit_words(n) * 4);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -732,15 +701,13 @@ cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* wor
   density_kernel<<<dim3((n + 7) / 8), dim3(256), 0, st>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // A round has far fewer medoids than entries; one CTA per 64 entries keeps the barriers of small problems short.
-  const int grid = std::max(1, std::min(sms, (n + 63) / 64));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = dim3(std::max(1, std::min({sms, n, kMaxPicks})));   // one CTA per SM, each grows one cluster per round
   cfg.blockDim = dim3(kRoundThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;             // the rounds end in a barrier over the grid
+  attr[0].id = cudaLaunchAttributeCooperative;             // the rounds end in barriers over the grid
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
