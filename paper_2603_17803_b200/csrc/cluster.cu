@@ -76,14 +76,14 @@ __global__ void __launch_bounds__(256) density_kernel(ClusterArgs a) {
 }
 
 // ---- rounds ----------------------------------------------------------------------------------------------------
-constexpr int kRoundThreads = 512;
-constexpr int kRoundWarps = kRoundThreads / 32;
+constexpr int kFetchWarps = 16;                           // (a power of two, like the ring: every slot has one owner)
+constexpr int kRoundWarps = 1 + kFetchWarps, kRoundThreads = kRoundWarps * 32;
 constexpr int kFastCand = 1024;                           // candidates one deciding warp holds (32 per lane)
-constexpr int kFetchWarps = kRoundWarps - 1;
-constexpr int kRingSlots = 4 * kFetchWarps;               // (a multiple of the fetching warps: every slot has one owner)
+constexpr int kLogRingSlots = 6, kRingSlots = 1 << kLogRingSlots;
 constexpr int kRingBytes = 128 * 1024;
 constexpr unsigned kGridWaitLimit = 1u << 23;
-constexpr unsigned kRingWaitLimit = 1u << 24;
+constexpr unsigned kDoneWaitLimit = 1u << 24;
+constexpr unsigned kRingWaitLimit = 1u << 18;             // polls of a try_wait that itself blocks for microseconds
 
 // Order-preserving key of a distance (-0 folded onto +0) and back.
 __device__ __forceinline__ uint32_t dist_key(float d) {
@@ -96,11 +96,11 @@ __device__ __forceinline__ float key_dist(uint32_t k) { return __uint_as_float((
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 struct RoundShared {
-  unsigned long long full[kRingSlots];                    // mbarriers: the 32 lanes' copies of a row have landed
-  unsigned issued[kRingSlots];                            // rows a slot has carried for earlier clusters (its barrier's phases)
+  unsigned long long full[kFastCand];                     // mbarriers, one per candidate: the 32 lanes' copies of its row have landed
   int warp_tot[kRoundWarps];
   int n_cand, size;
   int failed;
+  uint8_t phase[kFastCand];                               // the phase each barrier is in (they are initialised once)
   volatile int done;                                      // candidates before it are decided: their rows are free
   int pick[kMaxPicks];                                    // the round's entries, in the order of the walk
   int pick_size[kMaxPicks];
@@ -167,90 +167,95 @@ __device__ __forceinline__ void sort_pairs(uint32_t* key, uint16_t* idx, int m) 
   __syncthreads();
 }
 
+// Row j's copies have landed (bounded).  A candidate has a barrier of its own, used for one phase per cluster: which rows
+// the deciding warp waits for, and how far the fetching warps are behind it, is not known in advance, and the parity of
+// a ring slot's barrier would not tell its phases apart.  (Barriers initialised anew for every cluster lost arrivals.)
+__device__ __forceinline__ bool row_landed(RoundShared& sh, int j, unsigned phase) {
+  const uint32_t bar = smem_u32(&sh.full[j]);
+  unsigned ok = 0u, polls = 0u;
+  do {
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(phase) : "memory");
+  } while (!ok && ++polls < kRingWaitLimit);
+  return ok != 0u;
+}
+
 // The joins of a cluster with at most 32 * NR candidates, by one warp: candidate 32 r + lane's running sum in s[r];
-// decided candidates hold NaN, which passes no bound.  Returns the cluster's size (members in sh.member), or -1 when a wait ran out.
+// decided candidates hold NaN, which passes no bound.  Returns the cluster's size (members in sh.member), or -1 when
+// a wait ran out.  This is the chain the kernel waits for: the minimum over r is a tree, ring slots are a power of two.
 template <int NR>
 __device__ __forceinline__ int decide(const ClusterArgs& a, RoundShared& sh, const uint32_t* key, const uint16_t* idx,
-                                      const float* ring, int pitch, int slots, int n_cand) {
+                                      const float* ring, int pitch, int log_slots, int n_cand) {
   const int lane = threadIdx.x & 31;
   const float decided = __int_as_float(0x7FFFFFFF);
   float s[NR];
+  int code[NR];                                           // candidate << 1 | phase of its barrier
 #pragma unroll
-  for (int r = 0; r < NR; ++r) s[r] = 32 * r + lane < n_cand ? key_dist(key[32 * r + lane]) : decided;
+  for (int r = 0; r < NR; ++r) {
+    const int i = 32 * r + lane;
+    s[r] = i < n_cand ? key_dist(key[i]) : decided;
+    code[r] = i << 1 | (i < n_cand ? sh.phase[i] : 0);
+  }
   int size = 1;
+  bool late = false;                                      // a wait of this lane ran out
   for (;;) {
     const float bound = a.tau * (float)size;
-    int first = n_cand;
+    int first[NR];
 #pragma unroll
-    for (int r = NR - 1; r >= 0; --r) first = s[r] <= bound ? 32 * r + lane : first;
-    const int at = __reduce_min_sync(0xFFFFFFFFu, first);
+    for (int r = 0; r < NR; ++r) first[r] = s[r] <= bound ? code[r] : n_cand << 1;
+#pragma unroll
+    for (int w = NR / 2; w >= 1; w >>= 1)
+#pragma unroll
+      for (int r = 0; r < w; ++r) first[r] = min(first[r], first[r + w]);
+    const int next = __reduce_min_sync(0xFFFFFFFFu, late ? -1 : first[0]), at = next >> 1;
+    if (next < 0) return -1;
     if (at >= n_cand) break;
+    const int slot = at & ((1 << log_slots) - 1);
     if (lane == 0) {
       sh.member[size] = idx[at];
       sh.done = at;                                       // rows in front of `at` are not needed any more
     }
     ++size;
-    const int slot = at % slots;
-    unsigned polls = 0;
-    const uint32_t bar = smem_u32(&sh.full[slot]);
-    const unsigned parity = (sh.issued[slot] + (unsigned)(at / slots)) & 1u;
-    unsigned ok = 0u;
-    do {
-      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                   : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    } while (!ok && ++polls < kRingWaitLimit);
-    if (__any_sync(0xFFFFFFFFu, !ok)) return -1;
+    late = !row_landed(sh, at, (unsigned)next & 1u);
+    __syncwarp();
     const float* row = ring + slot * pitch + lane;
+    float v[NR];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      if (32 * r + 31 > at && 32 * r < n_cand) {          // (uniform)
-        const int i = 32 * r + lane;
-        const float v = i < n_cand && i > at ? row[32 * r] : 0.f;
-        s[r] = i > at ? s[r] + v : decided;
-      } else {
-        s[r] = decided;
-      }
-    }
+    for (int r = 0; r < NR; ++r) v[r] = 32 * r < n_cand ? row[32 * r] : 0.f;   // (columns up to `at` hold anything)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) s[r] = 32 * r + lane > at ? s[r] + v[r] : decided;
   }
   return size;
 }
 
 // One of the other warps (number w of kFetchWarps): rows of candidates w, w + kFetchWarps, ... into the ring.
-// Returns the first row of its own it has not issued.
+// Returns the first of them it has not issued.
 __device__ __forceinline__ int fetch_rows(const ClusterArgs& a, RoundShared& sh, const uint16_t* idx, float* ring,
-                                           int pitch, int slots, int n_cand, int w) {
-  const int lane = threadIdx.x & 31;
-  auto landed = [&](int j) -> bool {                      // row j's copies (bounded)
-    const int slot = j % slots;
-    const uint32_t bar = smem_u32(&sh.full[slot]);
-    const unsigned parity = (sh.issued[slot] + (unsigned)(j / slots)) & 1u;
-    unsigned ok = 0u, polls = 0u;
-    do {
-      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                   : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    } while (!ok && ++polls < kRingWaitLimit);
-    return !__any_sync(0xFFFFFFFFu, !ok);
-  };
+                                           int pitch, int log_slots, int n_cand, int w) {
+  const int lane = threadIdx.x & 31, slots = 1 << log_slots;
   int j = w;
+  bool fine = true;
   for (; j < n_cand; j += kFetchWarps) {
     int go = 1;
     if (lane == 0) {
       unsigned polls = 0;
-      while (sh.done <= j - slots && ++polls < kRingWaitLimit) __nanosleep(20);
+      while (sh.done <= j - slots && ++polls < kDoneWaitLimit) __nanosleep(20);
       if (sh.done <= j - slots) sh.failed = 1;
       go = sh.done > j - slots && sh.done < n_cand;
     }
     if (!__shfl_sync(0xFFFFFFFFu, go, 0)) break;
-    if (j >= slots && !landed(j - slots)) { sh.failed = 1; break; }
+    if (j >= slots) fine = row_landed(sh, j - slots, sh.phase[j - slots]) && fine;   // (a row nobody may have waited for)
+    __syncwarp();
     const float* row = a.dist + (long long)idx[j] * a.n;
-    float* dst = ring + (j % slots) * pitch;
+    float* dst = ring + (j & (slots - 1)) * pitch;
     for (int i = ((j + 1) & ~31) + lane; i < n_cand; i += 32)
       if (i > j) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + i)), "l"(row + idx[i]) : "memory");
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sh.full[j % slots])) : "memory");
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sh.full[j])) : "memory");
   }
-  // the last rows issued (one per slot of this warp) may still be in flight: nothing may land behind the cluster
-  for (int b = j - slots; b < j; b += kFetchWarps)
-    if (b >= 0 && !landed(b)) sh.failed = 1;
+  // the last rows issued may still be in flight: nothing may land behind the cluster
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  for (int b = max(w, ((j - slots) & ~(kFetchWarps - 1)) | w); b < j; b += kFetchWarps) fine = row_landed(sh, b, sh.phase[b]) && fine;
+  if (!fine) sh.failed = 1;
   return j;
 }
 
@@ -320,28 +325,27 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
   if (fast) {
     float* ring = reinterpret_cast<float*>(smem + kFastCand * 6);
     const int pitch = max(32, (n_cand + 31) & ~31);
-    const int slots = min(kRingSlots / kFetchWarps, kRingBytes / (pitch * 4) / kFetchWarps) * kFetchWarps;
+    const int log_slots = pitch * 4 * kRingSlots <= kRingBytes ? kLogRingSlots : kLogRingSlots - 1;
     int next_row = 0;
     if (tid == 0) sh.done = 0;
     __syncthreads();
     if (warp == 0) {
       int size;
-      if (n_cand <= 128) size = decide<4>(a, sh, key, idx, ring, pitch, slots, n_cand);
-      else if (n_cand <= 256) size = decide<8>(a, sh, key, idx, ring, pitch, slots, n_cand);
-      else if (n_cand <= 512) size = decide<16>(a, sh, key, idx, ring, pitch, slots, n_cand);
-      else size = decide<32>(a, sh, key, idx, ring, pitch, slots, n_cand);
+      if (n_cand <= 128) size = decide<4>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
+      else if (n_cand <= 256) size = decide<8>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
+      else if (n_cand <= 512) size = decide<16>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
+      else size = decide<32>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
       if (lane == 0) {
         sh.done = 0x7FFFFFFF;
         sh.size = size;
         if (size < 0) sh.failed = 1;
       }
     } else {
-      next_row = fetch_rows(a, sh, idx, ring, pitch, slots, n_cand, warp - 1);
+      next_row = fetch_rows(a, sh, idx, ring, pitch, log_slots, n_cand, warp - 1);
     }
     __syncthreads();
-    if (warp > 0 && lane == 0)                            // the phases the barriers of this warp's slots went through
-      for (int slot = warp - 1; slot < slots && slot < next_row; slot += kFetchWarps)
-        sh.issued[slot] += (unsigned)((next_row - 1 - slot) / slots + 1);
+    if (warp > 0)                                         // the barriers of the rows issued are one phase on
+      for (int j = warp - 1 + kFetchWarps * lane; j < next_row && j < n_cand; j += kFetchWarps * 32) sh.phase[j] ^= 1;
     *members = sh.member;
     return max(sh.size, 1);
   }
@@ -382,12 +386,12 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
   __shared__ RoundShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = a.n, bwords = bit_words(n), G = gridDim.x, me = blockIdx.x;
-  if (tid < kRingSlots) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sh.full[tid])), "r"(32));
-    sh.issued[tid] = 0u;
+  for (int j = tid; j < kFastCand; j += kRoundThreads) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sh.full[j])), "r"(32));
+    sh.phase[j] = 0;
   }
-  if (tid == 0) { sh.failed = 0; sh.done = 0; }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (tid == 0) sh.failed = 0;
   if (me == 0 && tid == 0) a.ptr[0] = 0;
 
   // ---- the order of the walk: a warp per entry counts the entries in front of it ----
