@@ -13,11 +13,12 @@
 // write their clusters to their final places.  Clusters that the walk does not want are dropped: they cost SMs that had
 // nothing else to do.  8192 entries in 64 topics: 102 clusters in 5 rounds.
 //
-// Growing one cluster: the candidates are sorted by (distance, index) in shared memory.  Between two joins neither the
-// running sums nor the bound tau * |C| change, so the next candidate to join is the first undecided one whose sum
-// passes.  One warp decides, its candidates' sums in registers (no CTA-wide barrier on the chain); the other warps
-// fetch the candidates' matrix rows, restricted to the candidates behind them, into a ring of shared memory ahead of
-// the decisions: the walk used to pay a trip to memory and two CTA-wide barriers per join (1.3 us).
+// Growing one cluster: the candidates are sorted by (distance, index) in shared memory and visited in that order; one
+// joins when its running sum is within tau * |C|.  A CTA does this 32 candidates at a time, a thread per candidate: the
+// warp that owns the 32 decides them one after the other (a ballot and an add per join, operands in registers), the
+// others then add the rows of those that joined.  The matrix entries a thread will need for the next 32 are loaded while
+// the present ones are decided.  Bound by those gathers: n_c^2 / 2 scattered words per cluster of n_c candidates, about
+// one 32-byte sector per two cycles and SM.  (As a walk that went to memory for every join it took 1.3 us per join.)
 // A candidate's sum is a plain fp32 accumulation in joining order over D[member][candidate], so every decision is the
 // one a sequential fp32 walk takes.
 #include "swarm_internal.cuh"
@@ -76,14 +77,9 @@ __global__ void __launch_bounds__(256) density_kernel(ClusterArgs a) {
 }
 
 // ---- rounds ----------------------------------------------------------------------------------------------------
-constexpr int kFetchWarps = 16;                           // (a power of two, like the ring: every slot has one owner)
-constexpr int kRoundWarps = 1 + kFetchWarps, kRoundThreads = kRoundWarps * 32;
-constexpr int kFastCand = 1024;                           // candidates one deciding warp holds (32 per lane)
-constexpr int kLogRingSlots = 6, kRingSlots = 1 << kLogRingSlots;
-constexpr int kRingBytes = 128 * 1024;
+constexpr int kRoundThreads = 512, kRoundWarps = kRoundThreads / 32;
+constexpr int kCountedCand = 1024;                        // up to here candidates are sorted by counting
 constexpr unsigned kGridWaitLimit = 1u << 23;
-constexpr unsigned kDoneWaitLimit = 1u << 24;
-constexpr unsigned kRingWaitLimit = 1u << 18;             // polls of a try_wait that itself blocks for microseconds
 
 // Order-preserving key of a distance (-0 folded onto +0) and back.
 __device__ __forceinline__ uint32_t dist_key(float d) {
@@ -93,20 +89,17 @@ __device__ __forceinline__ uint32_t dist_key(float d) {
 }
 __device__ __forceinline__ float key_dist(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k); }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 struct RoundShared {
-  unsigned long long full[kFastCand];                     // mbarriers, one per candidate: the 32 lanes' copies of its row have landed
   int warp_tot[kRoundWarps];
-  int n_cand, size;
-  int failed;
-  uint8_t phase[kFastCand];                               // the phase each barrier is in (they are initialised once)
-  volatile int done;                                      // candidates before it are decided: their rows are free
+  int n_cand, failed;
+  int my_clu;                                             // where this CTA's cluster goes, -1: nowhere
+  long long my_fill;
   int pick[kMaxPicks];                                    // the round's entries, in the order of the walk
   int pick_size[kMaxPicks];
   uint32_t holds[kMaxPicks][kNoteWords];
   uint32_t taken[kNoteWords];                             // the medoids among them
-  uint16_t member[kFastCand + 1];
+  uint32_t joined[1024];                                  // bit k of word b: candidate 32 b + k is a member
+  uint32_t likely[kRoundWarps];                           // candidates of the first 512 whose rows are worth loading ahead
 };
 
 // Exclusive prefix of v over the CTA and the total (two barriers).
@@ -167,110 +160,34 @@ __device__ __forceinline__ void sort_pairs(uint32_t* key, uint16_t* idx, int m) 
   __syncthreads();
 }
 
-// Row j's copies have landed (bounded).  A candidate has a barrier of its own, used for one phase per cluster: which rows
-// the deciding warp waits for, and how far the fetching warps are behind it, is not known in advance, and the parity of
-// a ring slot's barrier would not tell its phases apart.  (Barriers initialised anew for every cluster lost arrivals.)
-__device__ __forceinline__ bool row_landed(RoundShared& sh, int j, unsigned phase) {
-  const uint32_t bar = smem_u32(&sh.full[j]);
-  unsigned ok = 0u, polls = 0u;
-  do {
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(phase) : "memory");
-  } while (!ok && ++polls < kRingWaitLimit);
-  return ok != 0u;
-}
-
-// The joins of a cluster with at most 32 * NR candidates, by one warp: candidate 32 r + lane's running sum in s[r];
-// decided candidates hold NaN, which passes no bound.  Returns the cluster's size (members in sh.member), or -1 when
-// a wait ran out.  This is the chain the kernel waits for: the minimum over r is a tree, ring slots are a power of two.
-template <int NR>
-__device__ __forceinline__ int decide(const ClusterArgs& a, RoundShared& sh, const uint32_t* key, const uint16_t* idx,
-                                      const float* ring, int pitch, int log_slots, int n_cand) {
-  const int lane = threadIdx.x & 31;
-  const float decided = __int_as_float(0x7FFFFFFF);
-  float s[NR];
-  int code[NR];                                           // candidate << 1 | phase of its barrier
+// One thread's operands for the 32 candidates of block b: value k is D[row of candidate 32 b + k][entry c], loaded for
+// the candidates in `want` that stand in front of candidate i (the ones this thread's sum can still need).
+__device__ __forceinline__ void load_block(const ClusterArgs& a, const uint16_t* idx, int b, uint32_t want, int i, int c, float (&val)[32]) {
+  const uint4* rows = reinterpret_cast<const uint4*>(idx + 32 * b);
 #pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    const int i = 32 * r + lane;
-    s[r] = i < n_cand ? key_dist(key[i]) : decided;
-    code[r] = i << 1 | (i < n_cand ? sh.phase[i] : 0);
-  }
-  int size = 1;
-  bool late = false;                                      // a wait of this lane ran out
-  for (;;) {
-    const float bound = a.tau * (float)size;
-    int first[NR];
+  for (int q = 0; q < 4; ++q) {
+    const uint4 r = rows[q];                              // eight 16-bit entries
+    const uint32_t words[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-    for (int r = 0; r < NR; ++r) first[r] = s[r] <= bound ? code[r] : n_cand << 1;
-#pragma unroll
-    for (int w = NR / 2; w >= 1; w >>= 1)
-#pragma unroll
-      for (int r = 0; r < w; ++r) first[r] = min(first[r], first[r + w]);
-    const int next = __reduce_min_sync(0xFFFFFFFFu, late ? -1 : first[0]), at = next >> 1;
-    if (next < 0) return -1;
-    if (at >= n_cand) break;
-    const int slot = at & ((1 << log_slots) - 1);
-    if (lane == 0) {
-      sh.member[size] = idx[at];
-      sh.done = at;                                       // rows in front of `at` are not needed any more
+    for (int h = 0; h < 8; ++h) {
+      const int k = 8 * q + h;
+      const uint32_t e = (h & 1) ? words[h >> 1] >> 16 : words[h >> 1] & 0xFFFFu;
+      val[k] = (((want >> k) & 1u) && 32 * b + k < i) ? __ldg(a.dist + (long long)e * a.n + c) : 0.f;
     }
-    ++size;
-    late = !row_landed(sh, at, (unsigned)next & 1u);
-    __syncwarp();
-    const float* row = ring + slot * pitch + lane;
-    float v[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) v[r] = 32 * r < n_cand ? row[32 * r] : 0.f;   // (columns up to `at` hold anything)
-#pragma unroll
-    for (int r = 0; r < NR; ++r) s[r] = 32 * r + lane > at ? s[r] + v[r] : decided;
   }
-  return size;
-}
-
-// One of the other warps (number w of kFetchWarps): rows of candidates w, w + kFetchWarps, ... into the ring.
-// Returns the first of them it has not issued.
-__device__ __forceinline__ int fetch_rows(const ClusterArgs& a, RoundShared& sh, const uint16_t* idx, float* ring,
-                                           int pitch, int log_slots, int n_cand, int w) {
-  const int lane = threadIdx.x & 31, slots = 1 << log_slots;
-  int j = w;
-  bool fine = true;
-  for (; j < n_cand; j += kFetchWarps) {
-    int go = 1;
-    if (lane == 0) {
-      unsigned polls = 0;
-      while (sh.done <= j - slots && ++polls < kDoneWaitLimit) __nanosleep(20);
-      if (sh.done <= j - slots) sh.failed = 1;
-      go = sh.done > j - slots && sh.done < n_cand;
-    }
-    if (!__shfl_sync(0xFFFFFFFFu, go, 0)) break;
-    if (j >= slots) fine = row_landed(sh, j - slots, sh.phase[j - slots]) && fine;   // (a row nobody may have waited for)
-    __syncwarp();
-    const float* row = a.dist + (long long)idx[j] * a.n;
-    float* dst = ring + (j & (slots - 1)) * pitch;
-    for (int i = ((j + 1) & ~31) + lane; i < n_cand; i += 32)
-      if (i > j) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + i)), "l"(row + idx[i]) : "memory");
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sh.full[j])) : "memory");
-  }
-  // the last rows issued may still be in flight: nothing may land behind the cluster
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  for (int b = max(w, ((j - slots) & ~(kFetchWarps - 1)) | w); b < j; b += kFetchWarps) fine = row_landed(sh, b, sh.phase[b]) && fine;
-  if (!fine) sh.failed = 1;
-  return j;
 }
 
 // Grows the cluster of medoid m (all threads of the CTA).  Returns its size; member i >= 1 is (*members)[i] (shared
 // memory).  `smem`: the CTA's dynamic shared memory.
-__device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, int sort_cap, int m, const uint16_t** members) {
+__device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, int cap, int m, const uint16_t** members) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = a.n;
   const float* row_m = a.dist + (long long)m * n;
   const int n_cand = a.rho[m];
-  const bool fast = n_cand <= kFastCand;
-  // few candidates: (distance key << 32 | entry) pairs as collected, then sorted keys and entries; many: sorted in place
-  uint32_t* key = reinterpret_cast<uint32_t*>(smem);
-  uint16_t* idx = reinterpret_cast<uint16_t*>(smem + (fast ? kFastCand : sort_cap) * 4);
-  uint64_t* raw = reinterpret_cast<uint64_t*>(smem + kFastCand * 6);   // (in the ring's place)
+  const bool counted = n_cand <= kCountedCand;
+  uint32_t* key = reinterpret_cast<uint32_t*>(smem);      // [cap] distance keys; then the running sums; then the members
+  uint16_t* idx = reinterpret_cast<uint16_t*>(smem + cap * 4);           // [cap] entries
+  uint64_t* raw = reinterpret_cast<uint64_t*>(smem + cap * 6);           // (key << 32 | entry) as collected, if counted
 
   // ---- candidates in any order ----
   if (tid == 0) sh.n_cand = 0;
@@ -282,19 +199,26 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
     if (lane == 0) at = atomicAdd(&sh.n_cand, __popc(bal));
     at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
     if (is && at < n_cand) {
-      if (fast) raw[at] = ((uint64_t)dist_key(d) << 32) | (uint32_t)e;
+      if (counted) raw[at] = ((uint64_t)dist_key(d) << 32) | (uint32_t)e;
       else { key[at] = dist_key(d); idx[at] = (uint16_t)e; }
     }
   };
   if ((n & 3) == 0) {
-#pragma unroll 2
-    for (int j0 = warp * 128; j0 < n; j0 += kRoundThreads * 4) {
-      const int j = j0 + lane * 4;
-      const float4 v = j < n ? __ldg(reinterpret_cast<const float4*>(row_m + j)) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-      append(j < n && v.x <= a.tau && j != m, j, v.x);
-      append(j < n && v.y <= a.tau && j + 1 != m, j + 1, v.y);
-      append(j < n && v.z <= a.tau && j + 2 != m, j + 2, v.z);
-      append(j < n && v.w <= a.tau && j + 3 != m, j + 3, v.w);
+    for (int j0 = warp * 128; j0 < n; j0 += kRoundThreads * 16) {
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {                       // four loads in flight
+        const int j = j0 + u * kRoundThreads * 4 + lane * 4;
+        if (j < n) v[u] = __ldg(reinterpret_cast<const float4*>(row_m + j));
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + u * kRoundThreads * 4 + lane * 4;
+        append(j < n && v[u].x <= a.tau && j != m, j, v[u].x);
+        append(j < n && v[u].y <= a.tau && j + 1 != m, j + 1, v[u].y);
+        append(j < n && v[u].z <= a.tau && j + 2 != m, j + 2, v[u].z);
+        append(j < n && v[u].w <= a.tau && j + 3 != m, j + 3, v[u].w);
+      }
     }
   } else {
     for (int j0 = warp * 32; j0 < n; j0 += kRoundThreads) {
@@ -305,7 +229,7 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
   }
   __syncthreads();
   // ---- sorted by (distance, index) ----
-  if (fast) {                                             // each candidate's place by counting the ones in front of it
+  if (counted) {                                          // each candidate's place by counting the ones in front of it
     for (int i = tid; i < n_cand; i += kRoundThreads) {
       const uint64_t mine = raw[i];
       int at = 0;
@@ -322,92 +246,133 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
     sort_pairs(key, idx, m2);
   }
 
-  if (fast) {
-    float* ring = reinterpret_cast<float*>(smem + kFastCand * 6);
-    const int pitch = max(32, (n_cand + 31) & ~31);
-    const int log_slots = pitch * 4 * kRingSlots <= kRingBytes ? kLogRingSlots : kLogRingSlots - 1;
-    int next_row = 0;
-    if (tid == 0) sh.done = 0;
-    __syncthreads();
-    if (warp == 0) {
-      int size;
-      if (n_cand <= 128) size = decide<4>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
-      else if (n_cand <= 256) size = decide<8>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
-      else if (n_cand <= 512) size = decide<16>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
-      else size = decide<32>(a, sh, key, idx, ring, pitch, log_slots, n_cand);
-      if (lane == 0) {
-        sh.done = 0x7FFFFFFF;
-        sh.size = size;
-        if (size < 0) sh.failed = 1;
+  // ---- the walk over the candidates, 32 at a time ----
+  const int blocks = (n_cand + 31) / 32;
+  float* sum = reinterpret_cast<float*>(key);
+  for (int i = tid; i < 32 * blocks; i += kRoundThreads) {
+    if (i < n_cand) sum[i] = key_dist(key[i]);
+    else { sum[i] = __int_as_float(0x7FFFFFFF); idx[i] = (uint16_t)m; }   // no candidate: NaN passes no bound
+  }
+  if (tid < kRoundWarps) sh.likely[tid] = 0xFFFFFFFFu;
+  __syncthreads();
+  // thread t holds candidate t's sum in a register; candidates from kRoundThreads on have theirs in shared memory
+  const bool have = tid < 32 * blocks;
+  float s = have ? sum[tid] : 0.f;
+  const int c0 = have ? idx[tid] : m;
+  int size = 1;
+  float cur[32], nxt[32];
+  uint32_t cur_have = 0u, nxt_have = 0u;                  // rows loaded (a row is left out while its candidate looks hopeless)
+  auto fetch = [&](int b, float (&val)[32], uint32_t& loaded) {
+    loaded = 0u;
+    if (b < blocks && b < kRoundWarps && warp >= b && warp < blocks) {
+      loaded = *reinterpret_cast<volatile uint32_t*>(&sh.likely[b]);
+      load_block(a, idx, b, loaded, tid, c0, val);
+    }
+  };
+  auto step = [&](int b, float (&val)[32], uint32_t loaded) {
+    const int owner = b & (kRoundWarps - 1);
+    if (warp == owner) {
+      const int i = 32 * b + lane;                        // this lane's candidate
+      float x = b < kRoundWarps ? s : sum[i];
+      if (b >= kRoundWarps) { load_block(a, idx, b, 0xFFFFFFFFu, i, idx[i], val); loaded = 0xFFFFFFFFu; }
+      uint32_t joined = 0u;
+      int sz = size;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const unsigned pass = __ballot_sync(0xFFFFFFFFu, x <= a.tau * (float)sz) >> k;
+        if (pass == 0u) break;                            // nobody left in this block joins
+        if (pass & 1u) {
+          joined |= 1u << k;
+          ++sz;
+          float v = val[k];
+          if (!((loaded >> k) & 1u) && lane > k) v = __ldg(a.dist + (long long)idx[32 * b + k] * n + idx[i]);
+          if (lane > k) x += v;
+        }
       }
-    } else {
-      next_row = fetch_rows(a, sh, idx, ring, pitch, log_slots, n_cand, warp - 1);
+      if (lane == 0) sh.joined[b] = joined;
     }
     __syncthreads();
-    if (warp > 0)                                         // the barriers of the rows issued are one phase on
-      for (int j = warp - 1 + kFetchWarps * lane; j < next_row && j < n_cand; j += kFetchWarps * 32) sh.phase[j] ^= 1;
-    *members = sh.member;
-    return max(sh.size, 1);
-  }
-
-  // ---- more candidates than one warp holds: the whole CTA decides, sums in place of the keys ----
-  float* sum = reinterpret_cast<float*>(key);
-  for (int i = tid; i < n_cand; i += kRoundThreads) sum[i] = key_dist(key[i]);
-  __syncthreads();
-  int size = 1, from = 0;                                 // members so far; candidates before `from` are decided
-  while (from < n_cand) {
-    const float bound = a.tau * (float)size;
-    int first = n_cand;
-    for (int i = from + tid; i < n_cand; i += kRoundThreads)
-      if (sum[i] <= bound) { first = i; break; }
-    first = __reduce_min_sync(0xFFFFFFFFu, first);
-    if (lane == 0) sh.warp_tot[warp] = first;
-    __syncthreads();
-    int at = n_cand;
+    const uint32_t joined = sh.joined[b];
+    size += __popc(joined);
+    if (b < kRoundWarps && warp > b && warp < blocks) {   // the sums of the candidates behind the block
+      uint32_t late = joined & ~loaded;
+      while (late) {                                      // (joined against expectation: loaded now)
+        const int k = __ffs(late) - 1;
+        late &= late - 1u;
+        const float v = __ldg(a.dist + (long long)idx[32 * b + k] * n + c0);
 #pragma unroll
-    for (int w = 0; w < kRoundWarps; ++w) at = min(at, sh.warp_tot[w]);
-    if (at >= n_cand) break;
-    const uint16_t e = idx[at];
-    __syncthreads();                                      // everyone has read warp_tot and idx[at]
-    if (tid == 0) idx[size - 1] = e;                      // members take the places of decided candidates
-    ++size;
-    const float* row_e = a.dist + (long long)e * n;
-    for (int i = at + 1 + tid; i < n_cand; i += kRoundThreads) sum[i] = sum[i] + row_e[idx[i]];
-    from = at + 1;
-    __syncthreads();
+        for (int q = 0; q < 32; ++q) if (q == k) val[q] = v;
+      }
+#pragma unroll
+      for (int k = 0; k < 32; ++k) if ((joined >> k) & 1u) s += val[k];
+      const unsigned hint = __ballot_sync(0xFFFFFFFFu, s <= 1.25f * a.tau * (float)size);
+      if (lane == 0) sh.likely[warp] = hint;              // an average a quarter above the radius is not about to join
+    }
+    for (int i = tid + kRoundThreads; i < n_cand; i += kRoundThreads) {
+      if (i < 32 * (b + 1)) continue;
+      const int c = idx[i];
+      float v[32], x = sum[i];
+      load_block(a, idx, b, joined, i, c, v);
+#pragma unroll
+      for (int k = 0; k < 32; ++k) if ((joined >> k) & 1u) x += v[k];
+      sum[i] = x;
+    }
+  };
+  fetch(0, cur, cur_have);
+  for (int b = 0; b < blocks; b += 2) {
+    fetch(b + 1, nxt, nxt_have);
+    step(b, cur, cur_have);
+    if (b + 1 >= blocks) break;
+    fetch(b + 2, cur, cur_have);
+    step(b + 1, nxt, nxt_have);
+  }
+  // ---- its members, in the sums' place ----
+  __syncthreads();
+  uint16_t* list = reinterpret_cast<uint16_t*>(key);
+  int at = 1;
+  for (int b0 = 0; b0 < blocks; b0 += kRoundThreads) {    // (at most two turns)
+    const int b = b0 + tid;
+    uint32_t j = b < blocks ? sh.joined[b] : 0u;
+    int total;
+    int p = at + block_prefix(sh, __popc(j), total);
+    for (; j; j &= j - 1u) list[p++] = idx[32 * b + __ffs(j) - 1];
+    at += total;
   }
   __syncthreads();
-  *members = idx - 1;
+  *members = list;
   return size;
 }
 
-__global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a, int sort_cap) {
+__global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a, int cap) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ RoundShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = a.n, bwords = bit_words(n), G = gridDim.x, me = blockIdx.x;
-  for (int j = tid; j < kFastCand; j += kRoundThreads) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sh.full[j])), "r"(32));
-    sh.phase[j] = 0;
-  }
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   if (tid == 0) sh.failed = 0;
   if (me == 0 && tid == 0) a.ptr[0] = 0;
 
-  // ---- the order of the walk: a warp per entry counts the entries in front of it ----
-  for (int e = me * kRoundWarps + warp; e < n; e += G * kRoundWarps) {
-    const int mine = a.rho[e];
-    int at = 0;
-    for (int o0 = 0; o0 < n; o0 += 32 * 8) {
+  // ---- the order of the walk: the densities in shared memory, a warp counts the entries in front of four entries ----
+  int* s_rho = reinterpret_cast<int*>(dyn);
+  const int n4 = (n + 3) & ~3;
+  for (int i = tid; i < n4; i += kRoundThreads) s_rho[i] = i < n ? a.rho[i] : -1;
+  __syncthreads();
+  for (int e0 = (me * kRoundWarps + warp) * 4; e0 < n; e0 += G * kRoundWarps * 4) {
+    int mine[4], at[4] = {0, 0, 0, 0};
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int o = o0 + 32 * u + lane;
-        const int r = o < n ? a.rho[o] : -1;
-        at += r > mine || (r == mine && o < e);
+    for (int u = 0; u < 4; ++u) mine[u] = e0 + u < n ? s_rho[e0 + u] : 0;
+    for (int o = lane * 4; o < n4; o += 128) {
+      const int4 r = *reinterpret_cast<const int4*>(s_rho + o);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {                       // (an entry in front of e0 + u wins a tie)
+        const int m = mine[u], e = e0 + u;
+        at[u] += (r.x >= m + (o >= e)) + (r.y >= m + (o + 1 >= e)) + (r.z >= m + (o + 2 >= e)) + (r.w >= m + (o + 3 >= e));
       }
     }
-    at = __reduce_add_sync(0xFFFFFFFFu, at);
-    if (lane == 0) { a.queue[at] = e; a.place[e] = at; }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int p = __reduce_add_sync(0xFFFFFFFFu, at[u]);
+      if (lane == 0 && e0 + u < n) { a.queue[p] = e0 + u; a.place[e0 + u] = p; }
+    }
   }
   unsigned nth = 0;
   bool fine = grid_barrier(a, sh, ++nth);
@@ -436,10 +401,8 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
     const uint16_t* members = nullptr;
     if (me < n_picks) {
       const int m = sh.pick[me];
-      size = grow(a, sh, dyn, sort_cap, m, &members);
-      // marks of the members (few candidates: in the place of the sorted keys, else behind everything)
-      const bool fast = a.rho[m] <= kFastCand;
-      uint32_t* mark = reinterpret_cast<uint32_t*>(dyn + (fast ? kFastCand * 6 : sort_cap * 6));
+      size = grow(a, sh, dyn, cap, m, &members);
+      uint32_t* mark = reinterpret_cast<uint32_t*>(dyn + cap * 6);
       for (int w = tid; w < bwords; w += kRoundThreads) mark[w] = 0u;
       __syncthreads();
       for (int i = 1 + tid; i < size; i += kRoundThreads) atomicOr(&mark[members[i] >> 5], 1u << (members[i] & 31));
@@ -457,29 +420,31 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
     if (tid < n_picks) sh.pick_size[tid] = __ldcg(a.size + tid);
     __syncthreads();
     if (warp == 0) {
-      uint32_t cov = 0u, taken = 0u;                       // lane w: word w of the entries covered and taken
-      for (int i = 0; i < n_picks; ++i) {
-        const uint32_t row = lane < kNoteWords ? sh.holds[i][lane] : 0u;
-        const uint32_t c = __shfl_sync(0xFFFFFFFFu, cov, i >> 5);
-        if (!((c >> (i & 31)) & 1u)) {
-          cov |= row;
-          if (lane == (i >> 5)) taken |= 1u << (i & 31);
-        }
+      // lane w: word w of the entries still in the walk, and of the ones taken
+      uint32_t open = lane * 32 < n_picks ? (lane * 32 + 32 <= n_picks ? 0xFFFFFFFFu : (1u << (n_picks & 31)) - 1u) : 0u, taken = 0u;
+      for (;;) {
+        const int i = __reduce_min_sync(0xFFFFFFFFu, open ? lane * 32 + __ffs(open) - 1 : kMaxPicks);
+        if (i >= n_picks) break;
+        if (lane == (i >> 5)) { taken |= 1u << (i & 31); open &= ~(1u << (i & 31)); }
+        if (lane < kNoteWords) open &= ~sh.holds[i][lane];
       }
       if (lane < kNoteWords) sh.taken[lane] = taken;
     }
     __syncthreads();
     // ---- where the taken ones go ----
-    int my_at = -1, my_clu = 0;
-    long long my_fill = 0;
-    for (int i = 0; i < n_picks && status == 0; ++i) {
-      if (!((sh.taken[i >> 5] >> (i & 31)) & 1u)) continue;
-      if (fill + sh.pick_size[i] > a.members_cap) { status = 1; break; }   // it and everything behind it are left out
-      if (i == me) { my_at = i; my_clu = n_clu; my_fill = fill; }
-      ++n_clu;
-      fill += sh.pick_size[i];
-    }
-    if (my_at >= 0) {
+    const bool is = tid < n_picks && ((sh.taken[tid >> 5] >> (tid & 31)) & 1u);
+    int n_taken, n_members;
+    const int clu = n_clu + block_prefix(sh, is, n_taken);
+    const int at = block_prefix(sh, is ? sh.pick_size[tid] : 0, n_members);
+    const bool fits = is && fill + at + sh.pick_size[tid] <= a.members_cap;   // the first that does not fit ends the output
+    if (tid == me) { sh.my_clu = fits ? clu : -1; sh.my_fill = fill + at; }
+    const int n_fit = __syncthreads_count(fits);
+    status = n_fit < n_taken;
+    n_clu += n_fit;
+    fill += n_members;
+    const int my_clu = me < n_picks ? sh.my_clu : -1;
+    const long long my_fill = sh.my_fill;
+    if (my_clu >= 0) {
       const int m = sh.pick[me];
       if (tid == 0) {
         a.medoid[my_clu] = m;
@@ -694,9 +659,9 @@ cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* wor
   a.ptr = ptr; a.members = members; a.members_cap = members_cap; a.medoid = medoid; a.n_clusters = n_clusters;
   a.dev_status = dev_status;
 
-  int sort_cap = kFastCand;                                // power of two >= n: the candidates of one cluster
-  while (sort_cap < n) sort_cap <<= 1;
-  const int smem = std::max(kFastCand * 6 + kRingBytes, sort_cap * 6 + bit_words(n) * 4);
+  int cap = 1024;                                          // power of two >= n: the candidates of one cluster
+  while (cap < n) cap <<= 1;
+  const int smem = cap * 6 + std::max(kCountedCand * 8, bit_words(n) * 4);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -715,7 +680,7 @@ cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* wor
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, rounds_kernel, a, sort_cap);
+  return cudaLaunchKernelEx(&cfg, rounds_kernel, a, cap);
 }
 
 }  // namespace swarm
