@@ -34,6 +34,76 @@ constexpr int kSlotsPerThread = 4;
 constexpr size_t kItemStageBytes = 96 * 1024;            // shared-memory stage of the serial pass's operands
 constexpr size_t kResolveSmemBytes = kItemStageBytes + kItemStageBytes / 2;   // + key and rank of the submission order
 
+// ---- the serial pass over equally heavy clusters with two replicas, 32 stretches at a time ------------------------------
+// The greedy is a chain: every choice depends on the loads the one before it left, and a link costs 49 cycles through
+// the lanes of a warp.  But with equal weights its loads forget where they came from: two runs over the same clusters
+// from different (equally heavy) loads fall into step after some tens to hundreds of clusters, because every choice they
+// take differently brings them closer.  So the list is cut into 32 stretches, one per lane, and each lane runs its own
+// from a guess -- the loads levelled out as far as the starting loads allow.  Then every lane takes the loads its left
+// neighbour ended with as its start, and the warp runs again until no start changes any more.  That state is the
+// sequential greedy's: lane 0 starts from the true loads and every other lane from where its neighbour ended.  It takes
+// at most 32 turns (lane i is right after i turns whatever the guess), so at worst about what the chain takes.
+// 560 clusters on 8 queues: 8 turns of 19 links, 1600 (half of them two-replica, 8 queues): 6 of 51, 8192 on 16: 4 of 257
+// -- at 60 cycles a link (two loads and a store in shared memory, rows of 32 lanes: no bank conflicts).
+//   code   [n] in shared memory: 128 * lower queue | 128 * higher queue << 16; bit 31 becomes 1 where the higher one wins
+//   load   lane q: queue q's load in clusters
+__device__ __forceinline__ void lanes_pass(uint32_t* code, int n, int D, unsigned load, unsigned* s_cur, unsigned* s_start) {
+  const int lane = threadIdx.x & 31;
+  const int seg = ((n + 31) / 32) | 1;                    // (odd: the lanes' reads fall into different banks)
+  const int first = min(n, lane * seg), last = min(n, first + seg);
+  // the guess: level L with sum of max(load, L) = all loads so far
+  unsigned total = lane < D ? load : 0u;
+  total = __reduce_add_sync(0xFFFFFFFFu, total) + (unsigned)first;
+  unsigned level = total / (unsigned)D, rest = total % (unsigned)D;
+  for (int turn = 0; turn < D; ++turn) {
+    unsigned above = 0u, n_above = 0u;
+    for (int q = 0; q < D; ++q) {
+      const unsigned l = __shfl_sync(0xFFFFFFFFu, load, q);
+      if (l > level) { above += l; ++n_above; }
+    }
+    const unsigned left = total - above, among = (unsigned)D - n_above;   // (never all of them: the level is at most the mean)
+    const bool lower = left / among < level;
+    level = left / among;
+    rest = left % among;
+    if (!__any_sync(0xFFFFFFFFu, lower)) break;
+  }
+  for (int q = 0; q < D; ++q) {
+    const unsigned l = __shfl_sync(0xFFFFFFFFu, load, q);
+    unsigned v = l;
+    if (lane > 0 && l <= level) {
+      v = level + (rest > 0u ? 1u : 0u);
+      if (rest > 0u) --rest;
+    }
+    s_start[q * 32 + lane] = v;
+  }
+  char* cur = reinterpret_cast<char*>(s_cur + lane);
+  for (int turn = 0; turn <= 32; ++turn) {
+    for (int q = 0; q < D; ++q) s_cur[q * 32 + lane] = s_start[q * 32 + lane];
+    uint32_t c = first < last ? code[first] : 0u;
+#pragma unroll 4
+    for (int i = first; i < last; ++i) {
+      const uint32_t next = i + 1 < last ? code[i + 1] : 0u;
+      unsigned* pa = reinterpret_cast<unsigned*>(cur + (c & 0xFFFFu));
+      unsigned* pb = reinterpret_cast<unsigned*>(cur + ((c >> 16) & 0x7FFFu));
+      const unsigned la = *pa, lb = *pb;
+      const bool lower = la <= lb;                        // a tie goes to the lower queue
+      *(lower ? pa : pb) = (lower ? la : lb) + 1u;
+      code[i] = (c & 0x7FFFFFFFu) | (lower ? 0u : 0x80000000u);
+      c = next;
+    }
+    __syncwarp();
+    bool moved = false;
+    for (int q = 0; q < D; ++q) {
+      const unsigned v = lane > 0 ? s_cur[q * 32 + lane - 1] : s_start[q * 32];
+      moved = moved || v != s_start[q * 32 + lane];
+      s_start[q * 32 + lane] = v;
+    }
+    if (!__any_sync(0xFFFFFFFFu, moved && first < last)) break;
+    __syncwarp();
+  }
+}
+constexpr int kLanesMin = 64;                            // fewer clusters than this: the plain chain is as quick
+
 __device__ __forceinline__ int nonzero_bytes(uint32_t w) {
   // number of non-zero bytes in w (flags are 0 or 1, but any non-zero byte counts)
   const uint32_t t = (w | (w >> 1) | (w >> 2) | (w >> 3) | (w >> 4) | (w >> 5) | (w >> 6) | (w >> 7)) & 0x01010101u;
@@ -67,7 +137,8 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   __shared__ int2 s_seg[kWarps];                         // (start, length) of each warp's segment of the item list
   __shared__ int warp_cnt[kWarps];
   __shared__ int s_load[32];
-  __shared__ unsigned s_classes;
+  __shared__ unsigned s_classes, s_wmin, s_wmax;         // of the serial pass: replica classes, smallest and largest weight
+  __shared__ unsigned s_lanes[2][32 * 32];               // loads of the 32 stretches of lanes_pass, and their starts
   __shared__ unsigned s_item_m[32], s_item_w[32];
   __shared__ bool s_last;
   __shared__ int s_hits;
@@ -148,7 +219,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   // Every lane takes 4 flags (one word) at a time, so that up to 1024 clusters keep all 256 threads busy in a
   // single pass; warp w owns a contiguous range of words, which keeps the ids in ascending order.
   if (tid < 32) s_load[tid] = 0;
-  if (tid == 0) s_classes = 0u;
+  if (tid == 0) { s_classes = 0u; s_wmin = 0xFFFFFFFFu; s_wmax = 0u; }
   const int n_vec = (C + 3) / 4;                         // the flag array is padded to 16 bytes
   const int vec_per_warp = (n_vec + kWarps - 1) / kWarps;
   const int v_lo = min(n_vec, warp * vec_per_warp), v_hi = min(n_vec, v_lo + vec_per_warp);
@@ -268,7 +339,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   const bool order_keys_early = r.submit_order != nullptr && staged;
   const int seg_base = before;
   int seg_len = 0;
-  unsigned classes = 0u;
+  unsigned classes = 0u, wmin = 0xFFFFFFFFu, wmax = 0u;
   Row cur = keep;
   for (int v0 = v_lo; v0 < v_hi; v0 += 32) {
     const int v = v0 + lane;
@@ -320,6 +391,8 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
         const unsigned wgt = unit ? 1u : size;
         if ((serial_bits >> j) & 1u) {
           classes |= 1u << (__popc(m) - 1);
+          wmin = min(wmin, wgt);
+          wmax = max(wmax, wgt);
           const uint4 item = make_uint4(m, wgt << 5, (unsigned)i, 0u);   // what the serial pass needs
           if (staged) s_items[spos] = item;                // the serial pass then never waits on global memory
           else items[spos] = item;
@@ -346,10 +419,45 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     for (int k = seg_base + seg_len + lane; k < before; k += 32)   // blank the rest of this warp's slots
       s_items[k] = make_uint4(0u, 0u, 0u, 0u);
   SWARM_STAMP_ANY_CTA(status, 2);
-  if (classes) atomicOr(&s_classes, classes);
+  if (classes) {
+    atomicOr(&s_classes, classes);
+    atomicMin(&s_wmin, wmin);
+    atomicMax(&s_wmax, wmax);
+  }
   if (err) atomicOr(status, err);
   __syncthreads();
   SWARM_STAMP_ANY_CTA(status, 3);
+
+  // ---- equally heavy clusters with two replicas: 32 stretches side by side (see lanes_pass) ------------
+  int n_serial = 0, serial_before = 0;
+  for (int w2 = 0; w2 < kWarps; ++w2) {
+    if (w2 < warp) serial_before += s_seg[w2].y;
+    n_serial += s_seg[w2].y;
+  }
+  bool even = staged && s_classes == 2u && s_wmin == s_wmax && s_wmin > 0u && n_serial >= kLanesMin;   // (uniform)
+  if (even)
+    for (int q = 0; q < geo.D; ++q) even = even && (unsigned)s_load[q] % s_wmin == 0u;
+  if (even) {
+    uint32_t* code = reinterpret_cast<uint32_t*>(s_items + items_cap) + items_cap;   // (where the submission order's ranks go later)
+    const unsigned unit_w = s_wmin;
+    const int2 mine = s_seg[warp];
+    for (int i = lane; i < mine.y; i += 32) {
+      const unsigned m = s_items[mine.x + i].x;
+      code[serial_before + i] = (unsigned)(__ffs(m) - 1) * 128u | (unsigned)(31 - __clz(m)) * 128u << 16;
+    }
+    __syncthreads();
+    if (warp == 0) lanes_pass(code, n_serial, geo.D, (unsigned)s_load[lane] / unit_w, s_lanes[0], s_lanes[1]);
+    __syncthreads();
+    for (int i = lane; i < mine.y; i += 32) {
+      const uint32_t c = code[serial_before + i];
+      const unsigned q = ((c >> 31) ? (c >> 16) & 0x7FFFu : c & 0xFFFFu) / 128u;
+      const unsigned slot = s_items[mine.x + i].z;
+      queue_of[slot] = (uint8_t)q;
+      if (order_keys_early) order_key[slot] = (by_id ? 0u : 64u) + q;
+      atomicAdd(&s_load[q], (int)unit_w);
+    }
+    __syncthreads();
+  }
 
   // ---- the ordered greedy, one warp ------------------------------------------------------------------
   // It walks the warps' segments in order, which is id order (from shared memory: all of them as one list,
@@ -364,7 +472,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     // flat loop over each segment: no per-batch staging, the next item fetched while the current one is decided;
     // lane r of every group of 32 keeps the queue of the group's r-th cluster.
     const bool flat = staged && __popc(todo) <= 1;
-    if (flat && todo != 0u) {
+    if (flat && todo != 0u && !even) {
       for (int w2 = 0; w2 < kWarps; ++w2) {
         const int base = s_seg[w2].x, len = s_seg[w2].y;
         for (int g0 = 0; g0 < len; g0 += 32) {
@@ -427,7 +535,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     }
     SWARM_STAMP_ANY_CTA(status, 4);
     SWARM_KERNEL_END(status, 3);
-    if (staged) {
+    if (staged && !even) {
       __syncwarp();
       for (int k = lane; k < n; k += 32) {
         const uint4 item = s_items[k];

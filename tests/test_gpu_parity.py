@@ -283,6 +283,31 @@ def test_replication_extremes(replication, D):
     sess.close()
 
 
+@pytest.mark.parametrize("replication", ["two", "half_two"])
+@pytest.mark.parametrize("D,sizes", [(2, (8,)), (3, (8, 1)), (4, (7,)), (8, (8,)), (8, (1, 2, 3)), (8, (40, 63)),
+                                     (8, (900, 1023)), (8, (1500, 60000)), (8, (0,)), (8, (0, 9)), (9, (8,)), (12, (8, 1)),
+                                     (15, (3, 4, 5, 6)), (16, (8,)), (16, (62, 63)), (16, (64, 70)), (17, (8,))])
+def test_schedules_of_two_replicas(replication, D, sizes):
+    """The serial pass over two-replica clusters keeps the loads as bytes or halfwords while they fit and falls back to
+    the lanes where they do not: queue counts and weights on both sides of every limit, single-replica clusters that
+    spread the starting loads, and groups of 32 clusters that end in a remainder.  Every cluster is activated."""
+    cfg = small("c3_batched", batch=3, ctx_len=16 * 1501, top_k=1501, n_q_heads=2, n_kv_heads=2, n_topics=6,
+                replication=replication, n_queues=D)
+    w = W.generate(cfg, seed=D, device=DEV)
+    rng = np.random.default_rng(D * 1000 + len(sizes))
+    w.cluster_size.copy_(torch.from_numpy(rng.choice(sizes, size=w.n_clusters).astype(np.uint16).view(np.int16)))
+    for flags in (0, B.ORDER_BY_ID) if len(sizes) == 1 else (0,):
+        sess = Session(w, flags=flags)
+        sess.step()
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        o = sess.o
+        uniq, _, _ = parity.check_resolve(w, parity.host_tables(w), o.sel.cpu().numpy(), o.n_sel.cpu().numpy(), o.uniq.cpu().numpy(),
+                                          o.queue_of.cpu().numpy(), o.n_uniq.cpu().numpy()[0], o.queue_load.cpu().numpy(), flags)
+        assert len(uniq) == w.n_clusters
+        sess.close()
+
+
 def test_all_equal_scores_pick_lowest_ids_and_signed_zero_ties():
     cfg = small("c1_tiny", ctx_len=16 * 300, top_k=20)
     w = W.generate(cfg, seed=8, device=DEV)
