@@ -703,6 +703,7 @@ int32_t step_impl(swarm_ctx* ctx, const swarm_inputs* in, const swarm_outputs* o
   // serial pass is the longest item of the step).
   a.n_splits = pick_splits(ctx, true, /*fused=*/true);
   a.n_more = pick_more(ctx, true, a.n_splits, /*fused=*/true);
+  rs.rehearse = links.tk.selmap_ll != nullptr;
   SWARM_TRY(launch_attention(ctx->geo, a, status, st, /*overlap=*/true, &rs));
   return SWARM_OK;
 }

@@ -37,7 +37,6 @@ ResolveArgs make_resolve_args(const Geometry& geo, const int32_t* sel, const int
   r.sel = sel; r.n_sel = n_sel; r.page_base = page_base; r.page2cluster = page2cluster; r.cluster_base = cluster_base;
   r.replica_mask = replica_mask; r.cluster_size = cluster_size; r.flags = flags_ws; r.ticket = ticket; r.items = items;
   r.uniq = uniq; r.queue_of = queue_of; r.n_uniq = n_uniq; r.queue_load = queue_load; r.status = status;
-  r.items_cap = (int)(kItemStageBytes / sizeof(uint4));
   return r;
 }
 

@@ -213,7 +213,6 @@ struct ResolveArgs {
   int32_t* n_uniq;
   int32_t* queue_load;
   uint32_t* status;
-  int items_cap;
   int32_t* submit_order;   // optional: submission order (indices into uniq), see resolve_body.cuh
   int32_t* submit_info;    // optional: [0] batches, [1] clusters submitted
   HostMirror host{};
@@ -221,6 +220,7 @@ struct ResolveArgs {
   // StepTickets, and the distance between the two flag arrays that alternate steps mark.  Null / 0 otherwise.
   unsigned* tail_ctl = nullptr;
   long long flags_alt = 0;
+  bool rehearse = false;   // one CTA inside a step that is one chain: run the body once on made-up flags while the selection runs
 };
 ResolveArgs make_resolve_args(const Geometry& geo, const int32_t* sel, const int32_t* n_sel, const int64_t* page_base,
                               const int32_t* page2cluster, const int64_t* cluster_base, const uint32_t* replica_mask,

@@ -679,9 +679,20 @@ constexpr size_t kSmemKeyBytes = 160 * 1024;
 
 int topk_threads(int Pmax) { return Pmax <= 1024 ? 128 : Pmax <= 2048 ? 256 : Pmax <= 4096 ? 512 : 1024; }
 
+// A CTA can only join an SM whose shared-memory carve-out is the one its kernel asks for: beside the scorer's CTAs
+// that is the largest.
+template <class K>
+static cudaError_t share_sm(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 cudaError_t configure_topk() {
-  return cudaFuncSetAttribute(topk_generic_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kSmemKeyBytes);
+  cudaError_t e = cudaFuncSetAttribute(topk_generic_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKeyBytes);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, true>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, true>);
+  return e;
 }
 
 cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t* ctx_len, int32_t* sel,

@@ -308,6 +308,31 @@ def test_schedules_of_two_replicas(replication, D, sizes):
         sess.close()
 
 
+@pytest.mark.parametrize("batch,replication,sizes", [(2, "two", (8,)), (2, "two", (1, 2, 7)), (2, "hot_three", (3, 5)), (4, "two", (2,)),
+                                                     (4, "two", (1, 9))])
+def test_schedules_longer_than_the_shared_list(batch, replication, sizes):
+    """8192 and 16384 activated clusters: around the capacity of the serial pass's list in shared memory, with (smaller)
+    and without the submission order."""
+    cfg = small("c3_batched", batch=batch, ctx_len=16 * 8192, top_k=8192, n_q_heads=1, n_kv_heads=1, n_topics=4, cluster_pages=2,
+                replication=replication, n_queues=12)
+    w = W.generate(cfg, seed=batch, device=DEV)
+    rng = np.random.default_rng(batch)
+    w.cluster_size.copy_(torch.from_numpy(rng.choice(sizes, size=w.n_clusters).astype(np.uint16).view(np.int16)))
+    for order in (False, True):
+        sess = Session(w)
+        if order:
+            sess.enable_submit_order()
+        sess.step()
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        o = sess.o
+        parity.check_resolve(w, parity.host_tables(w), o.sel.cpu().numpy(), o.n_sel.cpu().numpy(), o.uniq.cpu().numpy(),
+                             o.queue_of.cpu().numpy(), o.n_uniq.cpu().numpy()[0], o.queue_load.cpu().numpy())
+        if order:
+            check_submit_order(w, sess)
+        sess.close()
+
+
 def test_all_equal_scores_pick_lowest_ids_and_signed_zero_ties():
     cfg = small("c1_tiny", ctx_len=16 * 300, top_k=20)
     w = W.generate(cfg, seed=8, device=DEV)
