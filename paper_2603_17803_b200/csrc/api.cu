@@ -787,9 +787,8 @@ int32_t swarm_build_medoid_index(swarm_ctx* ctx, const swarm_inputs* in, const i
   if (in == nullptr || bad(in->ksum) || bad(in->page_base) || bad(in->cluster_base) || bad(medoid_page) ||
       bad(medoid_ksum_out) || bad(cluster_ctx_len_out))
     return SWARM_ERR_INVALID_ARG;
-  SWARM_TRY(launch_cluster_len(ctx->geo, in->cluster_base, cluster_ctx_len_out, static_cast<cudaStream_t>(stream)));
   SWARM_TRY(launch_medoid_rows(ctx->geo, static_cast<const uint16_t*>(in->ksum), in->page_base, in->cluster_base,
-                               medoid_page, static_cast<uint16_t*>(medoid_ksum_out),
+                               medoid_page, static_cast<uint16_t*>(medoid_ksum_out), cluster_ctx_len_out,
                                ws_ptr<uint32_t>(ctx, ctx->lay.status), static_cast<cudaStream_t>(stream)));
   return SWARM_OK;
 }

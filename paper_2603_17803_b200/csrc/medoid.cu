@@ -5,8 +5,8 @@
 // The scoring and the top-k are the page kernels run over a context whose "pages" are the clusters: the
 // index holds the key summary of each cluster's medoid page, one row per cluster, requests back to back
 // exactly like cluster_base.  What this file adds is the glue around them:
-//   medoid_rows_kernel     index build: copy the summary rows of the medoid pages into the index
-//   cluster_len_kernel     pseudo context lengths (clusters of the request x page size) for the page kernels
+//   medoid_rows_kernel     index build: copy the summary rows of the medoid pages into the index, and the pseudo
+//                          context lengths (clusters of the request x page size) for the page kernels
 //   expand_clusters_kernel selected clusters -> per-head bitmap of their member pages plus the local window (what
 //                          the attention kernel reads) and the cluster flags (what the resolve kernel reads)
 #include "swarm_internal.cuh"
@@ -14,38 +14,43 @@
 namespace swarm {
 namespace {
 
-// One CTA per cluster: 2 * d bf16 per KV head = 512 bytes per head, 16-byte vectors.
-__global__ void __launch_bounds__(128)
+// One warp per cluster: 2 * d bf16 = 512 contiguous bytes per KV head, eight 512-byte rows in flight.  Bound by the chain
+// of small loads in front of them (one wave of CTAs at up to 9472 clusters).  The first CTA also writes the pseudo
+// lengths.  Launched behind whatever precedes it (in an index build the summaries).
+constexpr int kRowThreads = 256;
+__global__ void __launch_bounds__(kRowThreads)
 medoid_rows_kernel(Geometry geo, const uint16_t* __restrict__ ksum, const int64_t* __restrict__ page_base,
                    const int64_t* __restrict__ cluster_base, const int32_t* __restrict__ medoid_page,
-                   uint16_t* __restrict__ medoid_ksum, uint32_t* __restrict__ status) {
-  const long long c = blockIdx.x;
+                   uint16_t* __restrict__ medoid_ksum, int32_t* __restrict__ len, uint32_t* __restrict__ status) {
+  pdl_launch_dependents();
+  pdl_wait();
+  if (blockIdx.x == 0)
+    for (int b = threadIdx.x; b < geo.B; b += kRowThreads)
+      len[b] = (int32_t)min((long long)(cluster_base[b + 1] - cluster_base[b]) * geo.S, 0x7FFFFFFFLL);
+  const long long c = (long long)blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
   if (c >= cluster_base[geo.B]) return;
-  int b = 0;                                              // request of cluster c (binary search over cluster_base)
-  {
-    int lo = 0, hi = geo.B;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) / 2;
-      if (cluster_base[mid] <= c) lo = mid; else hi = mid;
-    }
-    b = lo;
+  const int p = medoid_page[c];
+  // request of cluster c: the last b with cluster_base[b] <= c, the bases taken 32 at a time
+  int b = 0;
+  for (int b0 = 0; b0 < geo.B; b0 += 32) {
+    const unsigned below = __ballot_sync(0xFFFFFFFFu, b0 + lane < geo.B && cluster_base[b0 + lane] <= c);
+    if (below == 0u) break;
+    b = b0 + 31 - __clz(below);
   }
   const long long pb = page_base[b];
-  const int p = medoid_page[c];
-  const int vec_per_row = geo.Hkv * 2 * kHeadDim / 8;
-  uint4* dst = reinterpret_cast<uint4*>(medoid_ksum + c * geo.Hkv * 2 * kHeadDim);
-  if (p < 0 || p >= page_base[b + 1] - pb) {
-    if (threadIdx.x == 0) atomicOr(status, SWARM_DEV_BAD_PAGE);
-    for (int i = threadIdx.x; i < vec_per_row; i += blockDim.x) dst[i] = make_uint4(0, 0, 0, 0);
-    return;
+  const bool ok = p >= 0 && p < page_base[b + 1] - pb;
+  if (!ok && lane == 0) atomicOr(status, SWARM_DEV_BAD_PAGE);
+  const uint4* src = reinterpret_cast<const uint4*>(ksum + (pb + (ok ? p : 0)) * geo.Hkv * 2 * kHeadDim) + lane;
+  uint4* dst = reinterpret_cast<uint4*>(medoid_ksum + c * geo.Hkv * 2 * kHeadDim) + lane;
+  for (int h0 = 0; h0 < geo.Hkv; h0 += 8) {
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = ok && h0 + i < geo.Hkv ? src[(h0 + i) * 32] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (h0 + i < geo.Hkv) dst[(h0 + i) * 32] = v[i];
   }
-  const uint16_t* src = ksum + (pb + p) * geo.Hkv * 2 * kHeadDim;
-  for (int i = threadIdx.x; i < vec_per_row; i += blockDim.x) dst[i] = ldg_nc_v4(src + (long long)i * 8);
-}
-
-__global__ void cluster_len_kernel(int B, int S, const int64_t* __restrict__ cluster_base, int32_t* __restrict__ len) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) len[b] = (int32_t)min((long long)(cluster_base[b + 1] - cluster_base[b]) * S, 0x7FFFFFFFLL);
 }
 
 // One CTA per (request, query head).  The head's bitmap row is assembled in shared memory (bit p % 8 of byte
@@ -116,15 +121,9 @@ cudaError_t configure_medoid() {
 
 cudaError_t launch_medoid_rows(const Geometry& geo, const uint16_t* ksum, const int64_t* page_base,
                                const int64_t* cluster_base, const int32_t* medoid_page, uint16_t* medoid_ksum,
-                               uint32_t* status, cudaStream_t st) {
-  medoid_rows_kernel<<<dim3((unsigned)geo.Cmax), dim3(128), 0, st>>>(geo, ksum, page_base, cluster_base, medoid_page,
-                                                                    medoid_ksum, status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cluster_len(const Geometry& geo, const int64_t* cluster_base, int32_t* len, cudaStream_t st) {
-  cluster_len_kernel<<<dim3((geo.B + 127) / 128), dim3(128), 0, st>>>(geo.B, geo.S, cluster_base, len);
-  return cudaGetLastError();
+                               int32_t* len, uint32_t* status, cudaStream_t st) {
+  return launch_pdl(medoid_rows_kernel, dim3((unsigned)(((long long)geo.Cmax * 32 + kRowThreads - 1) / kRowThreads)), dim3(kRowThreads), 0, st, true, geo,
+                    ksum, page_base, cluster_base, medoid_page, medoid_ksum, len, status);
 }
 
 cudaError_t launch_expand_clusters(const Geometry& geo, int k_c, const int32_t* sel_c, const int32_t* n_sel_c,

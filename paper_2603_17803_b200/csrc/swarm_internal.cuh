@@ -274,8 +274,7 @@ cudaError_t launch_selmap_from_sel(const Geometry& geo, const int32_t* sel, cons
 constexpr int kMaxExpandRowBytes = 160 * 1024;            // longest per-head page bitmap the expansion assembles in shared memory
 cudaError_t launch_medoid_rows(const Geometry& geo, const uint16_t* ksum, const int64_t* page_base,
                                const int64_t* cluster_base, const int32_t* medoid_page, uint16_t* medoid_ksum,
-                               uint32_t* status, cudaStream_t st);
-cudaError_t launch_cluster_len(const Geometry& geo, const int64_t* cluster_base, int32_t* len, cudaStream_t st);
+                               int32_t* len, uint32_t* status, cudaStream_t st);
 cudaError_t launch_expand_clusters(const Geometry& geo, int k_c, const int32_t* sel_c, const int32_t* n_sel_c,
                                    const int64_t* cluster_base, const int64_t* cluster_page_ptr,
                                    const int32_t* cluster_pages, const int32_t* ctx_len, uint8_t* selmap, uint8_t* flags,
