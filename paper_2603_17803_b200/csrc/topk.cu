@@ -20,8 +20,12 @@
 namespace swarm {
 namespace {
 
-constexpr int kBins = 4096;
-constexpr int kDigitBits = 12;
+// Histogram bins and the digit they count: four bins per thread, so that finding the digit's bin costs a thread the
+// same few registers and loads whatever the CTA's size (with 4096 bins for all, a 256-thread CTA held 16 bins per
+// thread: 96 registers, two CTAs per SM, and twice the time per list once the scorer had left the SM).
+template <int THREADS> constexpr int kBins = 4 * THREADS;
+template <int THREADS> constexpr int kDigitBits = THREADS == 1024 ? 12 : THREADS == 512 ? 11 : THREADS == 256 ? 10 : 9;
+constexpr int kLevels = 4;                                 // four digits of 9 to 12 bits cover a key
 constexpr int kRankMax = 64;                               // finish by direct ranking at or below this many candidates
 
 __device__ __forceinline__ uint32_t score_key(float s) {
@@ -165,25 +169,28 @@ __device__ __forceinline__ void mark_cluster(const Geometry& geo, const TopkExtr
   else x.flags[rb.cb + c] = 1;
 }
 
-// Shared state of one radix-select run.
+// Shared state of one radix-select run.  (Arrays used by neighbouring phases are separate ones: a phase needs no barrier
+// against the readers of the one before.)
+template <int THREADS>
 struct SelectState {
-  int hist[kBins];
-  int warp_tot[32];
+  int hist[kBins<THREADS>];
+  int warp_tot[32], warp_out[32];
   uint32_t red_min[32], red_max[32];
   uint32_t cand[kRankMax]; // candidate keys of the chosen bin, when few enough to finish by direct ranking
-  int n_cand;          // number of keys in the chosen bin (set by narrow), then the fill counter of cand[]
+  int n_fill;          // fill counter of cand[]; zero at the start
+  int n_cand;          // number of keys in the chosen bin
   uint32_t base;       // keys below `base` are out; candidates satisfy key - base < 2^bits
   int bits;            // undecided low bits of the candidates
   int remaining;       // rank still to find among the candidates (counted from the top)
 };
 
-// Where digit `bin` is counted.  Thread t owns the PER consecutive digits below (kBins - 1 - t*PER); its
+// Where digit `bin` is counted.  Thread t owns the PER consecutive digits below (bins - 1 - t*PER); its
 // j-th digit lives at word j*THREADS + t, so the threads of a warp touch consecutive words when they read
 // or clear their digits (no bank conflicts).
 template <int THREADS>
 __device__ __forceinline__ int hist_slot(uint32_t bin) {
-  constexpr int PER = kBins / THREADS;
-  const uint32_t idx = (uint32_t)(kBins - 1) - bin;         // rank of the digit from the top
+  constexpr int PER = kBins<THREADS> / THREADS;
+  const uint32_t idx = (uint32_t)(kBins<THREADS> - 1) - bin;         // rank of the digit from the top
   return (int)((idx % PER) * THREADS + idx / PER);
 }
 
@@ -200,8 +207,8 @@ __device__ __forceinline__ int totals_before(const int* warp_tot, int warp, int 
 // After the histogram of the current level is complete: locate the bin holding rank `remaining`
 // from the top, narrow (base, bits, remaining), clear the histogram.  All threads call it.
 template <int THREADS>
-__device__ __forceinline__ void narrow(SelectState& st, int tid, int shift) {
-  constexpr int PER = kBins / THREADS;                      // bins per thread, highest bins first
+__device__ __forceinline__ void narrow(SelectState<THREADS>& st, int tid, int shift, uint32_t base, int remaining) {
+  constexpr int PER = kBins<THREADS> / THREADS;             // bins per thread, highest bins first
   const int lane = tid & 31, warp = tid >> 5;
   int c[PER], sum = 0;
 #pragma unroll
@@ -216,8 +223,6 @@ __device__ __forceinline__ void narrow(SelectState& st, int tid, int shift) {
     if (lane >= o) incl += t;
   }
   if (lane == 31) st.warp_tot[warp] = incl;
-  const uint32_t base = st.base;
-  const int remaining = st.remaining;
   __syncthreads();
   int above = incl - sum + totals_before<THREADS>(st.warp_tot, warp, lane);
 #pragma unroll
@@ -226,7 +231,7 @@ __device__ __forceinline__ void narrow(SelectState& st, int tid, int shift) {
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       if (above < remaining && remaining <= above + c[j]) {
-        st.base = base + ((uint32_t)(kBins - 1 - (tid * PER + j)) << shift);
+        st.base = base + ((uint32_t)(kBins<THREADS> - 1 - (tid * PER + j)) << shift);
         st.bits = shift;
         st.remaining = remaining - above;
         st.n_cand = c[j];
@@ -239,32 +244,23 @@ __device__ __forceinline__ void narrow(SelectState& st, int tid, int shift) {
   __syncthreads();
 }
 
+// Smallest and largest key of the CTA, in every thread.
 template <int THREADS>
-__device__ __forceinline__ void block_minmax(SelectState& st, int tid, uint32_t lo, uint32_t hi) {
+__device__ __forceinline__ void block_minmax(SelectState<THREADS>& st, int tid, uint32_t& lo, uint32_t& hi) {
   const int lane = tid & 31, warp = tid >> 5;
   lo = __reduce_min_sync(0xFFFFFFFFu, lo);
   hi = __reduce_max_sync(0xFFFFFFFFu, hi);
   if (lane == 0) { st.red_min[warp] = lo; st.red_max[warp] = hi; }
   __syncthreads();
-  if (warp == 0) {
-    lo = lane < THREADS / 32 ? st.red_min[lane] : 0xFFFFFFFFu;
-    hi = lane < THREADS / 32 ? st.red_max[lane] : 0u;
-    lo = __reduce_min_sync(0xFFFFFFFFu, lo);
-    hi = __reduce_max_sync(0xFFFFFFFFu, hi);
-    if (lane == 0) {
-      st.base = lo;
-      st.bits = 32 - __clz(hi - lo);                        // 0 when every key is equal
-    }
-  }
-  __syncthreads();
+  lo = __reduce_min_sync(0xFFFFFFFFu, lane < THREADS / 32 ? st.red_min[lane] : 0xFFFFFFFFu);
+  hi = __reduce_max_sync(0xFFFFFFFFu, lane < THREADS / 32 ? st.red_max[lane] : 0u);
 }
 
 // The chosen bin holds few keys (already gathered in st.cand[0 .. n)): rank them directly.  The key whose
 // rank interval contains `remaining` is the k-th best key; ties share the interval, so every thread that
 // finds it writes the same values.
 template <int THREADS>
-__device__ __forceinline__ void finish_by_ranking(SelectState& st, int tid, int n) {
-  const int remaining = st.remaining;
+__device__ __forceinline__ void finish_by_ranking(SelectState<THREADS>& st, int tid, int n, int remaining) {
   const int lane = tid & 31, warp = tid >> 5;
   __syncthreads();
   // one warp per candidate: the lanes hold all (at most 64) candidates, two ballots count those above and equal
@@ -287,7 +283,7 @@ __device__ __forceinline__ void finish_by_ranking(SelectState& st, int tid, int 
 // The selection of one list with ITEMS consecutive pages per thread (the kernel was launched for lists of up to
 // THREADS * MAX_ITEMS pages; rows of the page bitmap are that long).
 template <int THREADS, int ITEMS, int MAX_ITEMS, bool kEarly>
-__device__ __forceinline__ bool topk_regs_body(SelectState& st, const Geometry& geo, const TopkExtras& x,
+__device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const Geometry& geo, const TopkExtras& x,
                                                const RequestBases& rb, const float* __restrict__ s,
                                                int32_t* __restrict__ out, int32_t* __restrict__ n_sel,
                                                uint32_t* __restrict__ status, int bh, int b, int kvh, int len_b, bool* s_flag,
@@ -342,7 +338,6 @@ __device__ __forceinline__ bool topk_regs_body(SelectState& st, const Geometry& 
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) key[j] = p0 + j < P ? score_key(__ldcg(s + p0 + j)) : 0u;
   }
-  if (tid == 0) st.remaining = k_sel;
   SWARM_STAMP(status, 2);
 
   uint32_t T = 0u;
@@ -362,10 +357,10 @@ __device__ __forceinline__ bool topk_regs_body(SelectState& st, const Geometry& 
     }
     block_minmax<THREADS>(st, tid, lo, hi);
     SWARM_STAMP(status, 3);
-    for (int level = 0; level < 4 && st.bits > 0; ++level) {
-      const uint32_t base = st.base;
-      const int bits = st.bits;
-      const int shift = max(bits - kDigitBits, 0);
+    uint32_t base = lo;
+    int bits = 32 - __clz(hi - lo), remaining = k_sel;      // 0 bits when every key is equal
+    for (int level = 0; level < kLevels && bits > 0; ++level) {
+      const int shift = max(bits - kDigitBits<THREADS>, 0);
       const uint32_t width_m1 = bits >= 32 ? 0xFFFFFFFFu : ((1u << bits) - 1u);
       if (full) {
 #pragma unroll
@@ -382,24 +377,26 @@ __device__ __forceinline__ bool topk_regs_body(SelectState& st, const Geometry& 
       }
       __syncthreads();
       SWARM_STAMP(status, 4 + 2 * level);
-      narrow<THREADS>(st, tid, shift);
+      narrow<THREADS>(st, tid, shift, base, remaining);
       SWARM_STAMP(status, 5 + 2 * level);
+      base = st.base;
+      bits = st.bits;
+      remaining = st.remaining;
       const int n_cand = st.n_cand;
-      if (st.bits > 0 && n_cand <= kRankMax) {
+      if (bits > 0 && n_cand <= kRankMax) {
         // few keys left: gather them and rank directly instead of running more digit levels
-        const uint32_t cbase = st.base;
-        const uint32_t cwidth_m1 = (1u << st.bits) - 1u;
-        __syncthreads();                                    // everyone has read n_cand before it becomes the fill counter
-        if (tid == 0) st.n_cand = 0;
-        __syncthreads();
+        const uint32_t cwidth_m1 = (1u << bits) - 1u;
 #pragma unroll
         for (int j = 0; j < ITEMS; ++j)
-          if ((full || p0 + j < Pw) && key[j] - cbase <= cwidth_m1) st.cand[atomicAdd(&st.n_cand, 1)] = key[j];
-        finish_by_ranking<THREADS>(st, tid, n_cand);
+          if ((full || p0 + j < Pw) && key[j] - base <= cwidth_m1) st.cand[atomicAdd(&st.n_fill, 1)] = key[j];
+        finish_by_ranking<THREADS>(st, tid, n_cand, remaining);
+        base = st.base;
+        bits = 0;
+        remaining = st.remaining;
       }
     }
-    T = st.base;
-    need_eq = st.remaining;
+    T = base;
+    need_eq = remaining;
   }
   SWARM_STAMP(status, 12);
 
@@ -430,10 +427,9 @@ __device__ __forceinline__ bool topk_regs_body(SelectState& st, const Geometry& 
     const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += t;
   }
-  __syncthreads();                                          // warp_tot may still be read by narrow()
-  if (lane == 31) st.warp_tot[warp] = incl;
+  if (lane == 31) st.warp_out[warp] = incl;
   __syncthreads();
-  const int before = incl - cnt + totals_before<THREADS>(st.warp_tot, warp, lane);
+  const int before = incl - cnt + totals_before<THREADS>(st.warp_out, warp, lane);
   const int gt_before = before & 0xFFFF, eq_before = before >> 16;
   // The page bitmap goes out first and the head is announced to the attention CTAs right behind it: a release
   // waits for every store issued before it to be acknowledged, so the selection list, the cluster marks and the
@@ -518,14 +514,15 @@ template <int THREADS, int ITEMS, bool kEarly>
 __global__ void __launch_bounds__(THREADS)
 topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
                  int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x) {
-  __shared__ SelectState st;
+  __shared__ SelectState<THREADS> st;
   __shared__ bool s_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int bh = blockIdx.x, b = bh / geo.Hq, kvh = (bh - b * geo.Hq) / geo.g;
   pdl_launch_dependents();
   SWARM_STAMP(status, 0);
   SWARM_KERNEL_BEGIN(status, 1);
-  for (int i = tid; i < kBins; i += THREADS) st.hist[i] = 0;
+  for (int i = tid; i < kBins<THREADS>; i += THREADS) st.hist[i] = 0;
+  if (tid == 0) st.n_fill = 0;
   prefetch_tables(geo, x);
   const RequestBases rb = load_bases(x, b);
   const int len_b = ctx_len[b];
@@ -561,13 +558,13 @@ __global__ void __launch_bounds__(kGenericThreads)
 topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
                     int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x) {
   extern __shared__ uint32_t skeys[];
-  __shared__ SelectState st;
+  __shared__ SelectState<kGenericThreads> st;
   __shared__ int warp_gt[32], warp_eq[32];
   __shared__ bool s_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int bh = blockIdx.x, b = bh / geo.Hq, kvh = (bh - b * geo.Hq) / geo.g;
   pdl_launch_dependents();
-  for (int i = tid; i < kBins; i += kGenericThreads) st.hist[i] = 0;
+  for (int i = tid; i < kBins<kGenericThreads>; i += kGenericThreads) st.hist[i] = 0;
   prefetch_tables(geo, x);
   const RequestBases rb = load_bases(x, b);
   const int len_b = ctx_len[b];
@@ -596,7 +593,6 @@ topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_
       hi = max(hi, key);
     }
   }
-  if (tid == 0) st.remaining = k_sel;
   uint32_t T = 0u;
   int need_eq = P;
   if (k_sel == 0) {
@@ -605,20 +601,23 @@ topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_
     __syncthreads();
   } else if (k_sel < Pw) {
     block_minmax<kGenericThreads>(st, tid, lo, hi);
-    for (int level = 0; level < 4 && st.bits > 0; ++level) {
-      const uint32_t base = st.base;
-      const int bits = st.bits;
-      const int shift = max(bits - kDigitBits, 0);
+    uint32_t base = lo;
+    int bits = 32 - __clz(hi - lo), remaining = k_sel;
+    for (int level = 0; level < kLevels && bits > 0; ++level) {
+      const int shift = max(bits - kDigitBits<kGenericThreads>, 0);
       const uint32_t width_m1 = bits >= 32 ? 0xFFFFFFFFu : ((1u << bits) - 1u);
       for (int i = tid; i < Pw; i += kGenericThreads) {
         const uint32_t rel = key_at(i) - base;
         if (rel <= width_m1) atomicAdd(&st.hist[hist_slot<kGenericThreads>(rel >> shift)], 1);
       }
       __syncthreads();
-      narrow<kGenericThreads>(st, tid, shift);
+      narrow<kGenericThreads>(st, tid, shift, base, remaining);
+      base = st.base;
+      bits = st.bits;
+      remaining = st.remaining;
     }
-    T = st.base;
-    need_eq = st.remaining;
+    T = base;
+    need_eq = remaining;
   } else {
     __syncthreads();
   }
