@@ -180,13 +180,14 @@ int reserved_sms(const swarm_ctx* ctx, const Geometry& g, bool tail) {
   if (!score_raises_tickets(g)) return 0;
   int n = ctx->select_sms;
   if (n < 0) {
-    // Selection CTAs of up to 256 threads fit on an SM beside a scorer CTA (registers and shared memory were
-    // sized for it): nothing to reserve.  Larger ones need an SM of their own: one per list, at most a
-    // quarter of the device (measured at 64 requests of up to 16384 pages: 37 reserved SMs beat both 0 and 54).
-    const int threads = topk_threads(g.Pmax);
+    // Selection CTAs of up to 512 threads with their keys in registers fit on an SM beside a scorer CTA (registers and
+    // shared memory were sized for it): nothing to reserve.  Larger ones need SMs of their own: enough for all lists at
+    // once, at most a quarter of the device (few lists, one CTA per SM), or a sixth where they share SMs (24 of 148: 64
+    // requests of up to 16384 pages 639 us with 8, 609 with 24, 641 with 44; 4 of 16384 pages 231, 230, 235).
     const long long lists = (long long)g.B * g.Hq;
-    const int per_sm = std::max(1, 1024 / threads);
-    n = threads <= 256 ? 0 : (int)std::min<long long>((lists + per_sm - 1) / per_sm, sm_count() / 4);
+    const int per_sm = select_per_sm(g.Pmax, lists);
+    const int most = sm_count() / (select_kind(g.Pmax, lists) == kSelectSmem512 ? 6 : 4);
+    n = per_sm == 0 ? 0 : (int)std::min<long long>((lists + per_sm - 1) / per_sm, most);
   }
   n += tail ? 1 : 0;
   return std::min(n, sm_count() - 8);

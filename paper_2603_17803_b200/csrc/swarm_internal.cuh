@@ -144,7 +144,9 @@ struct Geometry {   // plain copy of the shape in kernel-friendly form
 cudaError_t configure_score();
 int sm_count();         // SMs of the device current at configure_score() (148 on B200)
 cudaError_t configure_topk();
-int topk_threads(int Pmax);   // threads of the selection CTA launched for lists of up to Pmax pages
+enum SelectKind { kSelectRegs, kSelectSmem512, kSelectSmem1024, kSelectGeneric };
+SelectKind select_kind(int Pmax, long long lists);   // the selection kernel launched for `lists` lists of up to Pmax pages
+int select_per_sm(int Pmax, long long lists);        // its CTAs on an SM of their own; 0: they fit beside a scorer CTA
 cudaError_t configure_resolve();
 cudaError_t configure_attention();
 cudaError_t configure_medoid();

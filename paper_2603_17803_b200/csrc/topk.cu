@@ -13,7 +13,10 @@
 //
 // topk_regs keeps ITEMS consecutive pages per thread in registers (lists of up to 16384 pages; in the
 // largest instance a list of at most half that length is handled with half the pages per thread);
-// topk_generic walks lists of any length in shared or global memory with the same algorithm.
+// topk_smem keeps the keys in shared memory (many or longer lists); topk_generic walks lists of any length
+// in global memory with the same algorithm.
+#include <algorithm>
+
 #define SWARM_TRACE_FILE 1
 #include "swarm_internal.cuh"
 
@@ -29,9 +32,8 @@ constexpr int kLevels = 4;                                 // four digits of 9 t
 constexpr int kRankMax = 64;                               // finish by direct ranking at or below this many candidates
 
 __device__ __forceinline__ uint32_t score_key(float s) {
-  uint32_t u = __float_as_uint(s);
-  if (u == 0x80000000u) u = 0u;
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  const uint32_t u = __float_as_uint(__fadd_rn(s, 0.f));     // (-0 becomes +0)
+  return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
 }
 
 // Optional by-products of the selection, written while the selected pages are still in registers.
@@ -173,26 +175,20 @@ __device__ __forceinline__ void mark_cluster(const Geometry& geo, const TopkExtr
 // against the readers of the one before.)
 template <int THREADS>
 struct SelectState {
-  int hist[kBins<THREADS>];
+  alignas(16) int hist[kBins<THREADS>];
   int warp_tot[32], warp_out[32];
   uint32_t red_min[32], red_max[32];
   uint32_t cand[kRankMax]; // candidate keys of the chosen bin, when few enough to finish by direct ranking
   int n_fill;          // fill counter of cand[]; zero at the start
-  int n_cand;          // number of keys in the chosen bin
+  int n_cand;          // number of keys in the chosen bin; once `bits` is 0, of keys equal to `base`
   uint32_t base;       // keys below `base` are out; candidates satisfy key - base < 2^bits
   int bits;            // undecided low bits of the candidates
   int remaining;       // rank still to find among the candidates (counted from the top)
 };
 
-// Where digit `bin` is counted.  Thread t owns the PER consecutive digits below (bins - 1 - t*PER); its
-// j-th digit lives at word j*THREADS + t, so the threads of a warp touch consecutive words when they read
-// or clear their digits (no bank conflicts).
+// Where digit `bin` is counted: from the highest digit down, so that thread t owns the words 4 t .. 4 t + 3.
 template <int THREADS>
-__device__ __forceinline__ int hist_slot(uint32_t bin) {
-  constexpr int PER = kBins<THREADS> / THREADS;
-  const uint32_t idx = (uint32_t)(kBins<THREADS> - 1) - bin;         // rank of the digit from the top
-  return (int)((idx % PER) * THREADS + idx / PER);
-}
+__device__ __forceinline__ int hist_slot(uint32_t bin) { return (int)((uint32_t)(kBins<THREADS> - 1) - bin); }
 
 // Sum of the totals of the warps before `warp` (THREADS / 32 <= 32 totals in shared memory): every warp reduces
 // the masked totals with shuffles instead of each thread adding them up one by one.
@@ -208,14 +204,12 @@ __device__ __forceinline__ int totals_before(const int* warp_tot, int warp, int 
 // from the top, narrow (base, bits, remaining), clear the histogram.  All threads call it.
 template <int THREADS>
 __device__ __forceinline__ void narrow(SelectState<THREADS>& st, int tid, int shift, uint32_t base, int remaining) {
-  constexpr int PER = kBins<THREADS> / THREADS;             // bins per thread, highest bins first
+  constexpr int PER = 4;                                    // bins per thread, highest bins first
+  static_assert(kBins<THREADS> == PER * THREADS, "one 16-byte vector of bins per thread");
   const int lane = tid & 31, warp = tid >> 5;
-  int c[PER], sum = 0;
-#pragma unroll
-  for (int j = 0; j < PER; ++j) {
-    c[j] = st.hist[j * THREADS + tid];
-    sum += c[j];
-  }
+  int4* bins = reinterpret_cast<int4*>(st.hist) + tid;
+  const int4 c4 = *bins;
+  const int c[PER] = {c4.x, c4.y, c4.z, c4.w}, sum = (c4.x + c4.y) + (c4.z + c4.w);
   int incl = sum;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -225,8 +219,7 @@ __device__ __forceinline__ void narrow(SelectState<THREADS>& st, int tid, int sh
   if (lane == 31) st.warp_tot[warp] = incl;
   __syncthreads();
   int above = incl - sum + totals_before<THREADS>(st.warp_tot, warp, lane);
-#pragma unroll
-  for (int j = 0; j < PER; ++j) st.hist[j * THREADS + tid] = 0;
+  *bins = make_int4(0, 0, 0, 0);
   if (above < remaining && remaining <= above + sum) {
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
@@ -274,6 +267,7 @@ __device__ __forceinline__ void finish_by_ranking(SelectState<THREADS>& st, int 
       st.base = mine;
       st.bits = 0;
       st.remaining = remaining - gt;
+      st.n_cand = eq;
     }
   }
   __syncthreads();
@@ -342,9 +336,11 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
 
   uint32_t T = 0u;
   int need_eq = P;                                          // k_sel == Pw keeps everything
+  bool ties = false;                                        // only some of the pages at T are selected
   if (k_sel == 0) {
     T = 0xFFFFFFFFu;                                        // nothing but the window
     need_eq = 0;
+    ties = true;
   } else if (k_sel < Pw) {
     uint32_t lo = 0xFFFFFFFFu, hi = 0u;
     if (full) {
@@ -358,7 +354,7 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
     block_minmax<THREADS>(st, tid, lo, hi);
     SWARM_STAMP(status, 3);
     uint32_t base = lo;
-    int bits = 32 - __clz(hi - lo), remaining = k_sel;      // 0 bits when every key is equal
+    int bits = 32 - __clz(hi - lo), remaining = k_sel, n_eq = Pw;   // 0 bits when every key is equal
     for (int level = 0; level < kLevels && bits > 0; ++level) {
       const int shift = max(bits - kDigitBits<THREADS>, 0);
       const uint32_t width_m1 = bits >= 32 ? 0xFFFFFFFFu : ((1u << bits) - 1u);
@@ -394,9 +390,11 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
         bits = 0;
         remaining = st.remaining;
       }
+      n_eq = st.n_cand;
     }
     T = base;
     need_eq = remaining;
+    ties = need_eq < n_eq;
   }
   SWARM_STAMP(status, 12);
 
@@ -404,22 +402,19 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
   // its pages above the threshold (window pages rank above every score) and at it as two bit masks: about one
   // page in P / k is selected, so everything after the scan walks the set bits instead of all ITEMS pages.
   unsigned gt_mask = 0u, eq_mask = 0u;
-  if (full) {
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      gt_mask |= (unsigned)(key[j] > T) << j;
-      eq_mask |= (unsigned)(key[j] == T) << j;
-    }
-  } else {
+  for (int j = 0; j < ITEMS; ++j) gt_mask |= (unsigned)(key[j] >= T) << j;
+  if (ties) {                                               // (without: all pages at T are selected, like those above it)
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      if (p0 + j < P) {
-        const bool win = p0 + j >= Pw;
-        gt_mask |= (unsigned)(win || key[j] > T) << j;
-        eq_mask |= (unsigned)(!win && key[j] == T) << j;
-      }
-    }
+    for (int j = 0; j < ITEMS; ++j) eq_mask |= (unsigned)(key[j] == T) << j;
   }
+  if (!full) {
+    const unsigned exist = p0 >= P ? 0u : (1u << min(P - p0, ITEMS)) - 1u;
+    const unsigned win = p0 >= Pw ? 0xFFFFFFFFu : ~((1u << min(Pw - p0, ITEMS)) - 1u);
+    eq_mask &= exist & ~win;
+    gt_mask = (gt_mask | win) & exist;
+  }
+  gt_mask &= ~eq_mask;
   const int cnt = __popc(gt_mask) | (__popc(eq_mask) << 16);
   int incl = cnt;
 #pragma unroll
@@ -467,6 +462,18 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
         *reinterpret_cast<uint32_t*>(row + o) = 0u;
     }
   }
+  // The clusters of this thread's first selected pages: the reads travel while the head is announced (four at a time
+  // with all reads in front of the flag stores: a byte store may alias anything, so interleaving them would make
+  // every read wait for the store before it).
+  int c4[4] = {0, 0, 0, 0};
+  auto read_four = [&](unsigned todo) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (todo != 0u) c4[i] = x.page2cluster[rb.pb + p0 + __ffs(todo) - 1];
+      todo &= todo - 1u;                                    // 0 stays 0
+    }
+  };
+  if (!kEarly && x.flags != nullptr) read_four(picked);
   selection_announce(geo, x, b, kvh);
   for (unsigned todo = picked; todo != 0u; todo &= todo - 1u) {
     const unsigned bit = todo & (0u - todo), below = bit - 1u;
@@ -483,25 +490,16 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
       }
     }
   } else if (x.flags != nullptr) {
-    // four selected pages at a time: all the table reads first, then the flag stores -- a byte store may alias
-    // anything, so interleaving them would make every read wait for the store before it
     for (unsigned todo = picked; todo != 0u;) {
-      int c[4];
-      bool have[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        have[i] = todo != 0u;
-        const int j = __ffs(todo) - 1;
-        todo &= todo - 1u;                                  // 0 stays 0
-        c[i] = have[i] ? x.page2cluster[rb.pb + p0 + j] : 0;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (have[i]) {
-          if (c[i] < 0 || c[i] >= rb.cn - rb.cb || rb.cb + c[i] >= geo.Cmax) atomicOr(x.status, SWARM_DEV_BAD_CLUSTER);
-          else x.flags[rb.cb + c[i]] = 1;
+        if (todo != 0u) {
+          if (c4[i] < 0 || c4[i] >= rb.cn - rb.cb || rb.cb + c4[i] >= geo.Cmax) atomicOr(x.status, SWARM_DEV_BAD_CLUSTER);
+          else x.flags[rb.cb + c4[i]] = 1;
         }
+        todo &= todo - 1u;
       }
+      read_four(todo);
     }
   }
   for (int j = k_eff + tid; j < geo.k; j += THREADS) out[j] = -1;
@@ -510,8 +508,9 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
   return true;
 }
 
+// (up to 512 threads: 40 registers, which is what a scorer CTA leaves of each quarter of an SM's registers)
 template <int THREADS, int ITEMS, bool kEarly>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1536 / THREADS)
 topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
                  int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x) {
   __shared__ SelectState<THREADS> st;
@@ -550,14 +549,203 @@ topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
   SWARM_KERNEL_END(status, 1);
 }
 
-// ---- generic variant: any list length, keys in shared memory when they fit, else re-read ----------
+// ---- keys in shared memory: long lists ------------------------------------------------------------------------------
+// For lists too long for registers, and for many long lists: with the keys out of the registers two or three CTAs of 512
+// threads share an SM, so that one list's barriers are another's work (a 1024-thread CTA with its keys in registers has
+// the SM to itself).  A thread reads four neighbouring pages at a time, the same ones in every pass; at the end a warp
+// turns 32 pages into two words of bits (above the threshold, at it) with two ballots, and a thread per word places
+// them.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 3 : 1)
+topk_smem_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
+                 int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x) {
+  extern __shared__ uint4 skeys4[];
+  __shared__ SelectState<THREADS> st;
+  __shared__ bool s_flag;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int bh = blockIdx.x, b = bh / geo.Hq, kvh = (bh - b * geo.Hq) / geo.g;
+  pdl_launch_dependents();
+  SWARM_STAMP(status, 0);
+  SWARM_KERNEL_BEGIN(status, 1);
+  for (int i = tid; i < kBins<THREADS>; i += THREADS) st.hist[i] = 0;
+  if (tid == 0) st.n_fill = 0;
+  prefetch_tables(geo, x);
+  const RequestBases rb = load_bases(x, b);
+  const int len_b = ctx_len[b];
+  const float* s = scores + (long long)bh * geo.Pmax;
+  int32_t* out = sel + (long long)bh * geo.k;
+  if (x.flags_alt > 0) x.flags += (x.tk.ctl[kCtlMarked] & 1u) * x.flags_alt;
+  if (!scores_ready(geo, x, b, kvh, len_b, &s_flag)) {
+    write_empty_selection(geo, x, bh, out, n_sel, THREADS);
+    selection_announce(geo, x, b, kvh);
+    selection_done(geo, x);
+    return;
+  }
+  SWARM_STAMP(status, 1);
+  const int P = max(0, min(pages_of(len_b, geo.S), geo.Pmax));
+  const int k_eff = min(geo.k, P);
+  const int Pw = P - min(geo.W, P);                         // see topk_regs_kernel
+  const int k_sel = k_eff - (P - Pw);
+  uint32_t* skeys = reinterpret_cast<uint32_t*>(skeys4);
+  uint32_t* s_gt = skeys + ((geo.Pmax + 31) & ~31);         // a bit per page: above the threshold, at it
+  uint32_t* s_eq = s_gt + (geo.Pmax + 31) / 32;
+
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+  const bool vec = (geo.Pmax & 3) == 0;                     // rows of scores are 16-byte aligned
+#pragma unroll 4
+  for (int i = 4 * tid; i < P; i += 4 * THREADS) {
+    uint4 k4;
+    if (vec) {                                              // (pages past P inside the row: never looked at)
+      const float4 v = __ldcg(reinterpret_cast<const float4*>(s + i));   // written by a kernel that may still run: not through L1
+      k4 = make_uint4(score_key(v.x), score_key(v.y), score_key(v.z), score_key(v.w));
+    } else {
+      k4 = make_uint4(score_key(__ldcg(s + i)), i + 1 < P ? score_key(__ldcg(s + i + 1)) : 0u, i + 2 < P ? score_key(__ldcg(s + i + 2)) : 0u,
+                      i + 3 < P ? score_key(__ldcg(s + i + 3)) : 0u);
+    }
+    skeys4[i / 4] = k4;
+    if (i + 4 <= Pw) {
+      lo = min(min(lo, min(k4.x, k4.y)), min(k4.z, k4.w));
+      hi = max(max(hi, max(k4.x, k4.y)), max(k4.z, k4.w));
+    } else {
+      if (i < Pw) { lo = min(lo, k4.x); hi = max(hi, k4.x); }
+      if (i + 1 < Pw) { lo = min(lo, k4.y); hi = max(hi, k4.y); }
+      if (i + 2 < Pw) { lo = min(lo, k4.z); hi = max(hi, k4.z); }
+    }
+  }
+  SWARM_STAMP(status, 2);
+  uint32_t T = 0u;
+  int need_eq = P;
+  if (k_sel == 0) {
+    T = 0xFFFFFFFFu;
+    need_eq = 0;
+  } else if (k_sel < Pw) {
+    block_minmax<THREADS>(st, tid, lo, hi);
+    SWARM_STAMP(status, 3);
+    // f(key) for every key of this thread's scored pages
+    auto for_keys = [&](auto f) {
+#pragma unroll 2
+      for (int i = 4 * tid; i < Pw; i += 4 * THREADS) {
+        const uint4 k4 = skeys4[i / 4];
+        f(k4.x);
+        if (i + 4 <= Pw) { f(k4.y); f(k4.z); f(k4.w); }
+        else {
+          if (i + 1 < Pw) f(k4.y);
+          if (i + 2 < Pw) f(k4.z);
+        }
+      }
+    };
+    uint32_t base = lo;
+    int bits = 32 - __clz(hi - lo), remaining = k_sel;
+    for (int level = 0; level < kLevels && bits > 0; ++level) {
+      const int shift = max(bits - kDigitBits<THREADS>, 0);
+      const uint32_t width_m1 = bits >= 32 ? 0xFFFFFFFFu : ((1u << bits) - 1u);
+      if (level == 0) {                                     // every key is a candidate
+        for_keys([&](uint32_t key) { atomicAdd(&st.hist[hist_slot<THREADS>((key - base) >> shift)], 1); });
+      } else {
+        for_keys([&](uint32_t key) {
+          const uint32_t rel = key - base;
+          if (rel <= width_m1) atomicAdd(&st.hist[hist_slot<THREADS>(rel >> shift)], 1);
+        });
+      }
+      __syncthreads();
+      SWARM_STAMP(status, 4 + 2 * level);
+      narrow<THREADS>(st, tid, shift, base, remaining);
+      SWARM_STAMP(status, 5 + 2 * level);
+      base = st.base;
+      bits = st.bits;
+      remaining = st.remaining;
+      const int n_cand = st.n_cand;
+      if (bits > 0 && n_cand <= kRankMax) {
+        const uint32_t cwidth_m1 = (1u << bits) - 1u;
+        for_keys([&](uint32_t key) { if (key - base <= cwidth_m1) st.cand[atomicAdd(&st.n_fill, 1)] = key; });
+        finish_by_ranking<THREADS>(st, tid, n_cand, remaining);
+        base = st.base;
+        bits = 0;
+        remaining = st.remaining;
+      }
+    }
+    T = base;
+    need_eq = remaining;
+  }
+  __syncthreads();                                          // all keys are stored (where nothing above was a barrier)
+  SWARM_STAMP(status, 12);
+
+  const int words = (P + 31) / 32;
+#pragma unroll 4
+  for (int w = warp; w < words; w += THREADS / 32) {
+    const int i = 32 * w + lane;
+    const uint32_t key = i < P ? skeys[i] : 0u;
+    const unsigned gt = __ballot_sync(0xFFFFFFFFu, i < P && (key > T || i >= Pw)), eq = __ballot_sync(0xFFFFFFFFu, i < Pw && key == T);
+    if (lane == 0) { s_gt[w] = gt; s_eq[w] = eq; }
+  }
+  __syncthreads();
+  // thread t places the pages of words [w0, w1)
+  const int per = (words + THREADS - 1) / THREADS, w0 = min(words, tid * per), w1 = min(words, w0 + per);
+  int cnt = 0;
+  for (int w = w0; w < w1; ++w) cnt += __popc(s_gt[w]) | (__popc(s_eq[w]) << 16);
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) st.warp_out[warp] = incl;
+  __syncthreads();
+  const int before = incl - cnt + totals_before<THREADS>(st.warp_out, warp, lane);
+  // the bitmap first, then the announcement, then the list and the cluster marks (see topk_regs_body)
+  int eq_left = max(0, need_eq - (before >> 16));           // pages at the threshold this thread may still take
+  for (int w = w0; w < w1; ++w) {
+    unsigned eq = s_eq[w];
+    while (__popc(eq) > eq_left) eq &= ~(0x80000000u >> __clz(eq));   // the lowest ids win
+    eq_left -= __popc(eq);
+    s_gt[w] |= eq;                                          // (only this thread reads the word again)
+    if (x.selmap != nullptr && 4 * w + 4 <= x.selmap_pitch)
+      reinterpret_cast<uint32_t*>(x.selmap + (long long)bh * x.selmap_pitch)[w] = s_gt[w];
+  }
+  if (x.selmap != nullptr)                                  // words past the last page of the request
+    for (int w = words + tid; 4 * w + 4 <= x.selmap_pitch; w += THREADS)
+      reinterpret_cast<uint32_t*>(x.selmap + (long long)bh * x.selmap_pitch)[w] = 0u;
+  selection_announce(geo, x, b, kvh);
+  int place = (before & 0xFFFF) + min(before >> 16, need_eq);
+  for (int w = w0; w < w1; ++w) {
+    for (unsigned todo = s_gt[w]; todo != 0u;) {
+      // four pages at a time, their table reads in front of the flag stores (see topk_regs_body)
+      int page[4], c[4] = {0, 0, 0, 0};
+      unsigned have = 0u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (todo != 0u) {
+          page[i] = 32 * w + __ffs(todo) - 1;
+          have |= 1u << i;
+          if (x.flags != nullptr) c[i] = x.page2cluster[rb.pb + page[i]];
+        }
+        todo &= todo - 1u;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if ((have >> i) & 1u) {
+          out[place++] = page[i];
+          if (x.flags != nullptr) {
+            if (c[i] < 0 || c[i] >= rb.cn - rb.cb || rb.cb + c[i] >= geo.Cmax) atomicOr(x.status, SWARM_DEV_BAD_CLUSTER);
+            else x.flags[rb.cb + c[i]] = 1;
+          }
+        }
+      }
+    }
+  }
+  for (int j = k_eff + tid; j < geo.k; j += THREADS) out[j] = -1;
+  if (tid == 0) n_sel[bh] = k_eff;
+  SWARM_STAMP(status, 13);
+  selection_done(geo, x);
+  SWARM_KERNEL_END(status, 1);
+}
+
+// ---- generic variant: any list length, keys re-read from global memory ----------------------------
 constexpr int kGenericThreads = 1024;
 
-template <bool kKeysInSmem>
 __global__ void __launch_bounds__(kGenericThreads)
 topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
                     int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x) {
-  extern __shared__ uint32_t skeys[];
   __shared__ SelectState<kGenericThreads> st;
   __shared__ int warp_gt[32], warp_eq[32];
   __shared__ bool s_flag;
@@ -582,12 +770,11 @@ topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_
   const int k_eff = min(geo.k, P);
   const int Pw = P - min(geo.W, P);                         // see topk_regs_kernel
   const int k_sel = k_eff - (P - Pw);
-  auto key_at = [&](int i) -> uint32_t { return kKeysInSmem ? skeys[i] : score_key(__ldcg(s + i)); };
+  auto key_at = [&](int i) -> uint32_t { return score_key(__ldcg(s + i)); };
 
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
   for (int i = tid; i < P; i += kGenericThreads) {
     const uint32_t key = score_key(__ldcg(s + i));
-    if (kKeysInSmem) skeys[i] = key;
     if (i < Pw) {
       lo = min(lo, key);
       hi = max(hi, key);
@@ -672,11 +859,27 @@ topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_
   selection_done(geo, x);
 }
 
-constexpr size_t kSmemKeyBytes = 160 * 1024;
+// Bytes of dynamic shared memory of topk_smem_kernel: the keys and two bits per page.
+size_t smem_key_bytes(int Pmax) { return (size_t)((Pmax + 31) & ~31) * 4 + (size_t)((Pmax + 31) / 32) * 8; }
+constexpr size_t kSmemKeyBytes = 200 * 1024;               // 48 K pages
 
 }  // namespace
 
-int topk_threads(int Pmax) { return Pmax <= 1024 ? 128 : Pmax <= 2048 ? 256 : Pmax <= 4096 ? 512 : 1024; }
+// Which kernel selects: lists of up to 4096 pages, and few lists (the step then is a chain of latencies) of up to 16384,
+// in registers; many long lists and longer ones with their keys in shared memory.
+SelectKind select_kind(int Pmax, long long lists) {
+  if (Pmax <= 4096 || (Pmax <= 16384 && lists <= kLlScoreLists)) return kSelectRegs;
+  if (smem_key_bytes(Pmax) <= kSmemKeyBytes) return lists <= kLlScoreLists ? kSelectSmem1024 : kSelectSmem512;
+  return kSelectGeneric;
+}
+int select_per_sm(int Pmax, long long lists) {
+  const int threads = Pmax <= 1024 ? 128 : Pmax <= 2048 ? 256 : Pmax <= 4096 ? 512 : 1024;
+  switch (select_kind(Pmax, lists)) {
+    case kSelectRegs: return threads <= 512 ? 0 : 1;
+    case kSelectSmem512: return std::max(1, std::min(3, (int)(220 * 1024 / (smem_key_bytes(Pmax) + sizeof(SelectState<512>) + 1024))));
+    default: return 1;
+  }
+}
 
 // A CTA can only join an SM whose shared-memory carve-out is the one its kernel asks for: beside the scorer's CTAs
 // that is the largest.
@@ -686,11 +889,15 @@ static cudaError_t share_sm(K kernel) {
 }
 
 cudaError_t configure_topk() {
-  cudaError_t e = cudaFuncSetAttribute(topk_generic_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKeyBytes);
+  cudaError_t e = cudaFuncSetAttribute(topk_smem_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKeyBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_smem_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKeyBytes);
+  if (e == cudaSuccess) e = share_sm(topk_smem_kernel<512>);
   if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, false>);
   if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, true>);
   if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, false>);
   if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, true>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, true>);
   return e;
 }
 
@@ -728,18 +935,22 @@ cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t*
                             ctx_len, sel, n_sel, status, x)                                                         \
                : launch_pdl(topk_regs_kernel<THREADS, ITEMS, false>, grid, dim3(THREADS), 0, st, overlap, geo, scores, \
                             ctx_len, sel, n_sel, status, x)
-  if (geo.Pmax <= 1024) SWARM_TOPK_REGS(128, 8);
-  if (geo.Pmax <= 2048) SWARM_TOPK_REGS(256, 8);
-  if (geo.Pmax <= 4096) SWARM_TOPK_REGS(512, 8);
-  if (geo.Pmax <= 8192) SWARM_TOPK_REGS(1024, 8);
-  if (geo.Pmax <= 16384) SWARM_TOPK_REGS(1024, 16);
+  const SelectKind kind = select_kind(geo.Pmax, (long long)geo.B * geo.Hq);
+  if (kind == kSelectRegs) {
+    if (geo.Pmax <= 1024) SWARM_TOPK_REGS(128, 8);
+    if (geo.Pmax <= 2048) SWARM_TOPK_REGS(256, 8);
+    if (geo.Pmax <= 4096) SWARM_TOPK_REGS(512, 8);
+    if (geo.Pmax <= 8192) SWARM_TOPK_REGS(1024, 8);
+    SWARM_TOPK_REGS(1024, 16);
+  }
 #undef SWARM_TOPK_REGS
-  const size_t key_bytes = (size_t)geo.Pmax * sizeof(uint32_t);
-  if (key_bytes <= kSmemKeyBytes)
-    return launch_pdl(topk_generic_kernel<true>, grid, dim3(kGenericThreads), key_bytes, st, overlap, geo, scores,
-                      ctx_len, sel, n_sel, status, x);
-  return launch_pdl(topk_generic_kernel<false>, grid, dim3(kGenericThreads), 0, st, overlap, geo, scores, ctx_len,
-                    sel, n_sel, status, x);
+  if (kind == kSelectSmem512)
+    return launch_pdl(topk_smem_kernel<512>, grid, dim3(512), smem_key_bytes(geo.Pmax), st, overlap, geo, scores, ctx_len, sel, n_sel,
+                      status, x);
+  if (kind == kSelectSmem1024)
+    return launch_pdl(topk_smem_kernel<1024>, grid, dim3(1024), smem_key_bytes(geo.Pmax), st, overlap, geo, scores, ctx_len, sel, n_sel,
+                      status, x);
+  return launch_pdl(topk_generic_kernel, grid, dim3(kGenericThreads), 0, st, overlap, geo, scores, ctx_len, sel, n_sel, status, x);
 }
 
 }  // namespace swarm
