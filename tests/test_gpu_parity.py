@@ -736,6 +736,28 @@ def test_local_window_covering_all_of_k_and_longer_than_a_request():
 
 
 # ---- every list-length variant of the selection kernel, with and without a local window --------------------
+@pytest.mark.parametrize("pages,top_k,window", [(4097, 1, 0), (4999, 100, 3), (8192, 512, 0), (9001, 700, 9)])
+def test_selection_of_many_long_lists(pages, top_k, window):
+    """136 lists longer than a register-resident CTA takes when there are many: keys in shared memory, row lengths that
+    16-byte loads reach and do not, tied scores in one request, contexts that end anywhere (the last request has one page)."""
+    cfg = small("c5_skewed", batch=17, n_q_heads=8, n_kv_heads=1, ctx_range=None, ctx_len=16 * pages - 5, top_k=top_k, n_topics=8)
+    w = W.generate(cfg, seed=pages, device=DEV)
+    lens = torch.randint(1, 16 * pages - 4, (17,), generator=torch.Generator().manual_seed(pages), dtype=torch.int32)
+    lens[0], lens[-1] = 16 * pages - 5, 7
+    w.ctx_len.copy_(lens)
+    w.q[3].zero_()                                          # every score of request 3 is 0
+    sess = Session(w, keep_scores=True, local_window_pages=min(window, top_k))
+    sess.step()
+    torch.cuda.synchronize()
+    assert sess.status() == 0
+    sc, sel = sess.o.scores.cpu().numpy(), sess.o.sel.cpu().numpy()
+    want, n_want = oracle.topk(sc, lens.numpy(), cfg.page_size, top_k, min(window, top_k))
+    assert np.array_equal(sel, want) and np.array_equal(sess.o.n_sel.cpu().numpy(), n_want)
+    parity.check_resolve(w, parity.host_tables(w), sel, sess.o.n_sel.cpu().numpy(), sess.o.uniq.cpu().numpy(), sess.o.queue_of.cpu().numpy(),
+                         sess.o.n_uniq.cpu().numpy()[0], sess.o.queue_load.cpu().numpy())
+    sess.close()
+
+
 @pytest.mark.parametrize("pages", [900, 2000, 4000, 8000, 16000, 30000, 45000])
 @pytest.mark.parametrize("window", [0, 5])
 def test_selection_at_every_list_length(pages, window):
