@@ -555,6 +555,7 @@ topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
 // the SM to itself).  A thread reads four neighbouring pages at a time, the same ones in every pass; at the end a warp
 // turns 32 pages into two words of bits (above the threshold, at it) with two ballots, and a thread per word places
 // them.
+__host__ __device__ constexpr bool smem_words_in_hist(int Pmax, int threads) { return (Pmax + 31) / 32 * 2 <= 4 * threads; }
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 3 : 1)
 topk_smem_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
@@ -587,7 +588,8 @@ topk_smem_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
   const int Pw = P - min(geo.W, P);                         // see topk_regs_kernel
   const int k_sel = k_eff - (P - Pw);
   uint32_t* skeys = reinterpret_cast<uint32_t*>(skeys4);
-  uint32_t* s_gt = skeys + ((geo.Pmax + 31) & ~31);         // a bit per page: above the threshold, at it
+  // a bit per page: above the threshold, at it (in the histogram's place where they fit, see smem_key_bytes)
+  uint32_t* s_gt = smem_words_in_hist(geo.Pmax, THREADS) ? reinterpret_cast<uint32_t*>(st.hist) : skeys + ((geo.Pmax + 31) & ~31);
   uint32_t* s_eq = s_gt + (geo.Pmax + 31) / 32;
 
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
@@ -859,8 +861,11 @@ topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_
   selection_done(geo, x);
 }
 
-// Bytes of dynamic shared memory of topk_smem_kernel: the keys and two bits per page.
-size_t smem_key_bytes(int Pmax) { return (size_t)((Pmax + 31) & ~31) * 4 + (size_t)((Pmax + 31) / 32) * 8; }
+// Bytes of dynamic shared memory of topk_smem_kernel: the keys and, where the histogram is too small for them, two bits
+// per page.  (At 16384 pages this is what lets three CTAs share an SM instead of two.)
+size_t smem_key_bytes(int Pmax, int threads) {
+  return (size_t)((Pmax + 31) & ~31) * 4 + (smem_words_in_hist(Pmax, threads) ? 0 : (size_t)((Pmax + 31) / 32) * 8);
+}
 constexpr size_t kSmemKeyBytes = 200 * 1024;               // 48 K pages
 
 }  // namespace
@@ -869,14 +874,14 @@ constexpr size_t kSmemKeyBytes = 200 * 1024;               // 48 K pages
 // in registers; many long lists and longer ones with their keys in shared memory.
 SelectKind select_kind(int Pmax, long long lists) {
   if (Pmax <= 4096 || (Pmax <= 16384 && lists <= kLlScoreLists)) return kSelectRegs;
-  if (smem_key_bytes(Pmax) <= kSmemKeyBytes) return lists <= kLlScoreLists ? kSelectSmem1024 : kSelectSmem512;
+  if (smem_key_bytes(Pmax, 512) <= kSmemKeyBytes) return lists <= kLlScoreLists ? kSelectSmem1024 : kSelectSmem512;
   return kSelectGeneric;
 }
 int select_per_sm(int Pmax, long long lists) {
   const int threads = Pmax <= 1024 ? 128 : Pmax <= 2048 ? 256 : Pmax <= 4096 ? 512 : 1024;
   switch (select_kind(Pmax, lists)) {
     case kSelectRegs: return threads <= 512 ? 0 : 1;
-    case kSelectSmem512: return std::max(1, std::min(3, (int)(220 * 1024 / (smem_key_bytes(Pmax) + sizeof(SelectState<512>) + 1024))));
+    case kSelectSmem512: return std::max(1, std::min(3, (int)(228 * 1024 / (smem_key_bytes(Pmax, 512) + sizeof(SelectState<512>) + 1024 + 128))));
     default: return 1;
   }
 }
@@ -945,10 +950,10 @@ cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t*
   }
 #undef SWARM_TOPK_REGS
   if (kind == kSelectSmem512)
-    return launch_pdl(topk_smem_kernel<512>, grid, dim3(512), smem_key_bytes(geo.Pmax), st, overlap, geo, scores, ctx_len, sel, n_sel,
+    return launch_pdl(topk_smem_kernel<512>, grid, dim3(512), smem_key_bytes(geo.Pmax, 512), st, overlap, geo, scores, ctx_len, sel, n_sel,
                       status, x);
   if (kind == kSelectSmem1024)
-    return launch_pdl(topk_smem_kernel<1024>, grid, dim3(1024), smem_key_bytes(geo.Pmax), st, overlap, geo, scores, ctx_len, sel, n_sel,
+    return launch_pdl(topk_smem_kernel<1024>, grid, dim3(1024), smem_key_bytes(geo.Pmax, 1024), st, overlap, geo, scores, ctx_len, sel, n_sel,
                       status, x);
   return launch_pdl(topk_generic_kernel, grid, dim3(kGenericThreads), 0, st, overlap, geo, scores, ctx_len, sel, n_sel, status, x);
 }
