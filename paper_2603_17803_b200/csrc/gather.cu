@@ -18,6 +18,8 @@ gather_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int32_t*
               const int32_t* __restrict__ n_sel, const int64_t* __restrict__ page_base,
               const int32_t* __restrict__ ctx_len, uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out,
               int32_t* __restrict__ n_tok, uint32_t* __restrict__ status) {
+  pdl_launch_dependents();
+  pdl_wait();                                               // (its launch overlaps what precedes it in the stream)
   const int j = blockIdx.x % geo.k, bh = blockIdx.x / geo.k, b = bh / geo.Hq, h = bh % geo.Hq;
   const int S = geo.S;
   const int len = ctx_len[b];
@@ -151,8 +153,8 @@ cudaError_t launch_gather(const Geometry& geo, const uint16_t* kv_pool, const in
                           const int64_t* page_base, const int32_t* ctx_len, uint16_t* k_out, uint16_t* v_out,
                           int32_t* n_tok, uint32_t* status, cudaStream_t st) {
   const unsigned grid = (unsigned)geo.k * geo.B * geo.Hq;   // validated to fit at ctx creation
-  gather_kernel<<<grid, 256, 0, st>>>(geo, kv_pool, sel, n_sel, page_base, ctx_len, k_out, v_out, n_tok, status);
-  return cudaGetLastError();
+  return launch_pdl(gather_kernel, dim3(grid), dim3(256), 0, st, true, geo, kv_pool, sel, n_sel, page_base, ctx_len, k_out, v_out, n_tok,
+                    status);
 }
 
 cudaError_t launch_build_summaries(const Geometry& geo, const uint16_t* kv_pool, const int64_t* page_base,

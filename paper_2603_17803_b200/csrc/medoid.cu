@@ -64,7 +64,8 @@ expand_clusters_kernel(Geometry geo, int k_c, int pitch, const int32_t* __restri
                        const int64_t* __restrict__ page_base, const int32_t* __restrict__ page2cluster) {
   extern __shared__ uint32_t s_row[];
   const int bh = blockIdx.x, b = bh / geo.Hq;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
+  pdl_launch_dependents();                                  // the attention CTAs set themselves up meanwhile
   const int P = pages_of(ctx_len[b], geo.S);               // inputs: read before the wait
   const long long cb = cluster_base[b], cn = cluster_base[b + 1];
   for (int i = tid; i < pitch / 4; i += blockDim.x) s_row[i] = 0u;
@@ -72,14 +73,18 @@ expand_clusters_kernel(Geometry geo, int k_c, int pitch, const int32_t* __restri
   __syncthreads();
   const int n = min(n_sel_c[bh], k_c);
   unsigned err = 0u;
-  for (int j = warp; j < n; j += blockDim.x / 32) {         // one warp per selected cluster
+  // Eight lanes per selected cluster, 32 clusters at a time: every cluster costs three dependent trips to memory
+  // (its id, its member range, its members), and with a warp per cluster four clusters of a warp paid them one after
+  // another (the kernel 7 of the step's 60 us; 32 clusters per head).
+  const int sub = tid & 7;
+  for (int j = tid >> 3; j < n; j += blockDim.x / 8) {
     const int c = sel_c[(long long)bh * k_c + j];
     if (c < 0 || c >= cn - cb || cb + c >= geo.Cmax) { err |= SWARM_DEV_BAD_CLUSTER; continue; }
     const long long e0 = cluster_page_ptr[cb + c], e1 = cluster_page_ptr[cb + c + 1];
     if (e0 < 0 || e1 < e0 || e1 > n_member_entries) { err |= SWARM_DEV_BAD_CLUSTER; continue; }   // corrupt member offsets
     // what gets scheduled: the cluster as a whole, or (entry level) each of its pages on its own
-    if (lane == 0 && entry_base == nullptr) flags[cb + c] = 1;
-    for (long long e = e0 + lane; e < e1; e += 32) {
+    if (sub == 0 && entry_base == nullptr) flags[cb + c] = 1;
+    for (long long e = e0 + sub; e < e1; e += 8) {
       const int p = cluster_pages[e];
       if (p < 0 || p >= P || p >= pitch * 8) {
         err |= SWARM_DEV_BAD_PAGE;

@@ -386,7 +386,8 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();                               // the next kernel in the stream may be scheduled while this one runs
-  const long long c_all = cluster_base[geo.B];           // an input table: not written by the previous kernel
+  if (sel != nullptr) pdl_wait();                        // (on its own, any input may come from the previous kernel)
+  const long long c_all = cluster_base[geo.B];           // inside a step an input table: not written by the previous kernel
   const int C = (int)min((long long)geo.Cmax, c_all);
   unsigned err = 0u, step_no = 0u;
   // Every instruction below runs once per step, on an SM that has not fetched it since the step before, and while the
