@@ -24,6 +24,7 @@
 #include "swarm_internal.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace swarm {
 namespace {
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(256) density_kernel(ClusterArgs a) {
 }
 
 // ---- rounds ----------------------------------------------------------------------------------------------------
-constexpr int kRoundThreads = 512, kRoundWarps = kRoundThreads / 32;
+constexpr int kRoundThreads = 384, kRoundWarps = kRoundThreads / 32;
 constexpr int kCountedCand = 1024;                        // up to here candidates are sorted by counting
 constexpr unsigned kGridWaitLimit = 1u << 23;
 
@@ -99,7 +100,7 @@ struct RoundShared {
   uint32_t holds[kMaxPicks][kNoteWords];
   uint32_t taken[kNoteWords];                             // the medoids among them
   uint32_t joined[1024];                                  // bit k of word b: candidate 32 b + k is a member
-  uint32_t likely[kRoundWarps];                           // candidates of the first 512 whose rows are worth loading ahead
+  uint32_t likely[kRoundWarps];                           // candidates of the first 384 whose rows are worth loading ahead
 };
 
 // Exclusive prefix of v over the CTA and the total (two barriers).
@@ -124,13 +125,14 @@ __device__ __forceinline__ int block_prefix(RoundShared& sh, int v, int& total) 
   return before + incl - v;
 }
 
-// Every CTA of the (cooperative) grid has arrived for the nth time; false when that wait, or one inside a CTA, ran out.
-__device__ __forceinline__ bool grid_barrier(const ClusterArgs& a, RoundShared& sh, unsigned nth) {
+// Every CTA of the (cooperative) grid has arrived for the nth time; false when that wait ran out.
+__device__ __forceinline__ void grid_arrive(const ClusterArgs& a) {
   __syncthreads();
+  if (threadIdx.x == 0) red_release_add(a.ctl + kCtlArrived, 1u);
+}
+__device__ __forceinline__ bool grid_wait(const ClusterArgs& a, RoundShared& sh, unsigned nth) {
   if (threadIdx.x == 0) {
     unsigned* p = a.ctl + kCtlArrived;
-    if (sh.failed) atomicExch(a.ctl + kCtlFailed, 1u);
-    red_release_add(p, 1u);
     const unsigned target = nth * gridDim.x;
     unsigned polls = 0, v = 0;
     do {
@@ -177,9 +179,9 @@ __device__ __forceinline__ void load_block(const ClusterArgs& a, const uint16_t*
   }
 }
 
-// Grows the cluster of medoid m (all threads of the CTA).  Returns its size; member i >= 1 is (*members)[i] (shared
-// memory).  `smem`: the CTA's dynamic shared memory.
-__device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, int cap, int m, const uint16_t** members) {
+// Grows the cluster of medoid m (all threads of the CTA).  Returns its size; its members behind the medoid are the
+// candidates whose bits are set in sh.joined, and a bit each in `mark`.  `smem`: the CTA's dynamic shared memory.
+__device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, int cap, int m, uint32_t* mark) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = a.n;
   const float* row_m = a.dist + (long long)m * n;
@@ -187,58 +189,89 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
   const bool counted = n_cand <= kCountedCand;
   uint32_t* key = reinterpret_cast<uint32_t*>(smem);      // [cap] distance keys; then the running sums; then the members
   uint16_t* idx = reinterpret_cast<uint16_t*>(smem + cap * 4);           // [cap] entries
-  uint64_t* raw = reinterpret_cast<uint64_t*>(smem + cap * 6);           // (key << 32 | entry) as collected, if counted
+  uint32_t* raw_key = reinterpret_cast<uint32_t*>(smem + cap * 6);       // as collected, if counted
+  uint32_t* raw_entry = raw_key + kCountedCand;
+  static_assert(kCountedCand >= 1024, "32 x 32 operands take its place, the marks of 32768 entries the keys'");
 
   // ---- candidates in any order ----
   if (tid == 0) sh.n_cand = 0;
   __syncthreads();
-  auto append = [&](bool is, int e, float d) {            // (whole warps)
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, is);
-    if (bal == 0u) return;
+  // (whole warps; each thread's are counted first, so that a warp asks for room once)
+  auto append = [&](uint32_t mask, auto entry_of, auto dist_of, auto count) {
+    int before = __popc(mask);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xFFFFFFFFu, before, o);
+      if (lane >= o) before += t;
+    }
     int at = 0;
-    if (lane == 0) at = atomicAdd(&sh.n_cand, __popc(bal));
-    at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
-    if (is && at < n_cand) {
-      if (counted) raw[at] = ((uint64_t)dist_key(d) << 32) | (uint32_t)e;
-      else { key[at] = dist_key(d); idx[at] = (uint16_t)e; }
+    if (lane == 31 && before > 0) at = atomicAdd(&sh.n_cand, before);
+    at = __shfl_sync(0xFFFFFFFFu, at, 31) + before - __popc(mask);
+    if (mask == 0u) return;
+#pragma unroll
+    for (int u = 0; u < decltype(count)::value; ++u) {
+      if (((mask >> u) & 1u) && at < n_cand) {
+        const uint32_t k = dist_key(dist_of(u));
+        if (counted) { raw_key[at] = k; raw_entry[at] = (uint32_t)entry_of(u); }
+        else { key[at] = k; idx[at] = (uint16_t)entry_of(u); }
+        ++at;
+      }
     }
   };
   if ((n & 3) == 0) {
-    for (int j0 = warp * 128; j0 < n; j0 += kRoundThreads * 16) {
-      float4 v[4];
+    for (int j0 = 4 * tid; j0 < (n + 127 & ~127); j0 += kRoundThreads * 24) {   // (a warp's 32 threads together)
+      float v[24];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {                       // four loads in flight
-        const int j = j0 + u * kRoundThreads * 4 + lane * 4;
-        if (j < n) v[u] = __ldg(reinterpret_cast<const float4*>(row_m + j));
+      for (int u = 0; u < 6; ++u) {                       // six loads in flight
+        const int j = j0 + u * kRoundThreads * 4;
+        const float4 f = j < n ? __ldg(reinterpret_cast<const float4*>(row_m + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[4 * u] = f.x; v[4 * u + 1] = f.y; v[4 * u + 2] = f.z; v[4 * u + 3] = f.w;
       }
+      auto entry_of = [&](int u) { return j0 + (u >> 2) * kRoundThreads * 4 + (u & 3); };
+      uint32_t mask = 0u;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = j0 + u * kRoundThreads * 4 + lane * 4;
-        append(j < n && v[u].x <= a.tau && j != m, j, v[u].x);
-        append(j < n && v[u].y <= a.tau && j + 1 != m, j + 1, v[u].y);
-        append(j < n && v[u].z <= a.tau && j + 2 != m, j + 2, v[u].z);
-        append(j < n && v[u].w <= a.tau && j + 3 != m, j + 3, v[u].w);
-      }
+      for (int u = 0; u < 24; ++u) mask |= (v[u] <= a.tau && entry_of(u) < n && entry_of(u) != m ? 1u : 0u) << u;
+      append(mask, entry_of, [&](int u) { return v[u]; }, std::integral_constant<int, 24>());
     }
   } else {
-    for (int j0 = warp * 32; j0 < n; j0 += kRoundThreads) {
-      const int j = j0 + lane;
-      const float v = j < n ? __ldg(row_m + j) : 0.f;
-      append(j < n && v <= a.tau && j != m, j, v);
+    for (int j0 = tid; j0 < (n + 31 & ~31); j0 += kRoundThreads) {
+      const float v = j0 < n ? __ldg(row_m + j0) : 0.f;
+      append(j0 < n && v <= a.tau && j0 != m ? 1u : 0u, [&](int) { return j0; }, [&](int) { return v; }, std::integral_constant<int, 1>());
     }
   }
   __syncthreads();
   // ---- sorted by (distance, index) ----
-  if (counted) {                                          // each candidate's place by counting the ones in front of it
-    for (int i = tid; i < n_cand; i += kRoundThreads) {
-      const uint64_t mine = raw[i];
-      int at = 0;
-#pragma unroll 8
-      for (int j = 0; j < n_cand; ++j) at += raw[j] < mine;
-      key[at] = (uint32_t)(mine >> 32);
-      idx[at] = (uint16_t)mine;
-    }
+  if (counted) {
+    // Each candidate's place by counting the keys up to its own, four lanes per candidate.  Equal keys land on one place
+    // and leave another unfilled; then the count is repeated with the entries in it.
+    const int padded = (n_cand + 15) & ~15;
+    for (int i = n_cand + tid; i < padded; i += kRoundThreads) raw_key[i] = 0xFFFFFFFFu;
+    for (int i = tid; i < n_cand; i += kRoundThreads) idx[i] = 0xFFFFu;
     __syncthreads();
+    auto place = [&](bool ties) {
+      for (int t0 = 0; t0 < 4 * n_cand; t0 += kRoundThreads) {
+        const int i = (t0 + tid) >> 2, part = tid & 3;
+        const uint32_t mine = i < n_cand ? raw_key[i] : 0u, e = i < n_cand ? raw_entry[i] : 0u;
+        int at = 0;
+#pragma unroll 4
+        for (int j = 4 * part; j < padded; j += 16) {
+          const uint4 k = *reinterpret_cast<const uint4*>(raw_key + j);
+          at += (k.x <= mine) + (k.y <= mine) + (k.z <= mine) + (k.w <= mine);
+          if (ties) {
+            const uint4 o = *reinterpret_cast<const uint4*>(raw_entry + j);
+            at -= (k.x == mine && o.x > e) + (k.y == mine && o.y > e) + (k.z == mine && o.z > e) + (k.w == mine && o.w > e);
+          }
+        }
+        at += __shfl_xor_sync(0xFFFFFFFFu, at, 1);
+        at += __shfl_xor_sync(0xFFFFFFFFu, at, 2);
+        if (part == 0 && i < n_cand) { key[at - 1] = mine; idx[at - 1] = (uint16_t)e; }
+      }
+      __syncthreads();
+    };
+    place(false);
+    bool open = false;
+    for (int i = tid; i < n_cand; i += kRoundThreads) open = open || idx[i] == 0xFFFFu;
+    if (__syncthreads_or(open)) place(true);
   } else {
     int m2 = 1;
     while (m2 < n_cand) m2 <<= 1;
@@ -254,40 +287,47 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
     else { sum[i] = __int_as_float(0x7FFFFFFF); idx[i] = (uint16_t)m; }   // no candidate: NaN passes no bound
   }
   if (tid < kRoundWarps) sh.likely[tid] = 0xFFFFFFFFu;
+  for (int w = tid; w < bit_words(n); w += kRoundThreads) mark[w] = 0u;   // (where the collected candidates were)
   __syncthreads();
   // thread t holds candidate t's sum in a register; candidates from kRoundThreads on have theirs in shared memory
   const bool have = tid < 32 * blocks;
   float s = have ? sum[tid] : 0.f;
   const int c0 = have ? idx[tid] : m;
+  float* tile = reinterpret_cast<float*>(raw_entry);      // the operands of the block being decided
   int size = 1;
   float cur[32], nxt[32];
   uint32_t cur_have = 0u, nxt_have = 0u;                  // rows loaded (a row is left out while its candidate looks hopeless)
   auto fetch = [&](int b, float (&val)[32], uint32_t& loaded) {
     loaded = 0u;
     if (b < blocks && b < kRoundWarps && warp >= b && warp < blocks) {
-      loaded = *reinterpret_cast<volatile uint32_t*>(&sh.likely[b]);
+      loaded = warp == b ? 0xFFFFFFFFu : *reinterpret_cast<volatile uint32_t*>(&sh.likely[b]);
       load_block(a, idx, b, loaded, tid, c0, val);
     }
   };
   auto step = [&](int b, float (&val)[32], uint32_t loaded) {
-    const int owner = b & (kRoundWarps - 1);
+    const int owner = b % kRoundWarps;
     if (warp == owner) {
       const int i = 32 * b + lane;                        // this lane's candidate
       float x = b < kRoundWarps ? s : sum[i];
-      if (b >= kRoundWarps) { load_block(a, idx, b, 0xFFFFFFFFu, i, idx[i], val); loaded = 0xFFFFFFFFu; }
-      uint32_t joined = 0u;
-      int sz = size;
+      if (b >= kRoundWarps) load_block(a, idx, b, 0xFFFFFFFFu, i, idx[i], val);
+      // A link of the chain is a load from shared memory, an add, a compare and a ballot, and there is one per member:
+      // candidates that no join lets in are passed over on the ballot of the last one.  (Unrolled over the 32 registers
+      // the warp waited for instructions: 2900 cycles per 32 candidates.)
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const unsigned pass = __ballot_sync(0xFFFFFFFFu, x <= a.tau * (float)sz) >> k;
-        if (pass == 0u) break;                            // nobody left in this block joins
-        if (pass & 1u) {
-          joined |= 1u << k;
-          ++sz;
-          float v = val[k];
-          if (!((loaded >> k) & 1u) && lane > k) v = __ldg(a.dist + (long long)idx[32 * b + k] * n + idx[i]);
-          if (lane > k) x += v;
-        }
+      for (int k = 0; k < 32; ++k) tile[32 * k + lane] = val[k];
+      uint32_t joined = 0u, above = 0xFFFFFFFFu;
+      float members = (float)size + 1.f, bound = a.tau * (float)size, next = a.tau * members;
+      for (;;) {
+        const uint32_t pass = __ballot_sync(0xFFFFFFFFu, x <= bound) & above;
+        if (pass == 0u) break;
+        const int k = __ffs(pass) - 1;
+        const float v = tile[32 * k + lane];              // (written by this lane)
+        joined |= 1u << k;
+        above = 0xFFFFFFFEu << k;
+        x += v;                                           // (of no account for the lanes up to k)
+        bound = next;
+        members += 1.f;
+        next = a.tau * members;
       }
       if (lane == 0) sh.joined[b] = joined;
     }
@@ -326,12 +366,21 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
     fetch(b + 2, cur, cur_have);
     step(b + 1, nxt, nxt_have);
   }
-  // ---- its members, in the sums' place ----
   __syncthreads();
-  uint16_t* list = reinterpret_cast<uint16_t*>(key);
+  for (int i = tid; i < n_cand; i += kRoundThreads)
+    if ((sh.joined[i >> 5] >> (i & 31)) & 1u) atomicOr(&mark[idx[i] >> 5], 1u << (idx[i] & 31));
+  __syncthreads();
+  return size;
+}
+
+// The members of the cluster grown last behind its medoid: member i >= 1 is list[i] (shared memory, the sums' place).
+__device__ const uint16_t* list_members(RoundShared& sh, unsigned char* smem, int cap, int n_cand) {
+  uint16_t* list = reinterpret_cast<uint16_t*>(smem);
+  const uint16_t* idx = reinterpret_cast<const uint16_t*>(smem + cap * 4);
+  const int blocks = (n_cand + 31) / 32;
   int at = 1;
-  for (int b0 = 0; b0 < blocks; b0 += kRoundThreads) {    // (at most two turns)
-    const int b = b0 + tid;
+  for (int b0 = 0; b0 < blocks; b0 += kRoundThreads) {    // (at most three turns)
+    const int b = b0 + threadIdx.x;
     uint32_t j = b < blocks ? sh.joined[b] : 0u;
     int total;
     int p = at + block_prefix(sh, __popc(j), total);
@@ -339,8 +388,7 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
     at += total;
   }
   __syncthreads();
-  *members = list;
-  return size;
+  return list;
 }
 
 __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a, int cap) {
@@ -351,31 +399,43 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
   if (tid == 0) sh.failed = 0;
   if (me == 0 && tid == 0) a.ptr[0] = 0;
 
-  // ---- the order of the walk: the densities in shared memory, a warp counts the entries in front of four entries ----
-  int* s_rho = reinterpret_cast<int*>(dyn);
+  // ---- the order of the walk: a warp counts the entries in front of kPer entries, from keys in shared memory ----
+  // (density << 15 | 32767 - entry: in front means a larger key, one compare)
+  constexpr int kPer = 5;                                  // (8192 entries on 148 SMs: one turn)
+  int* s_key = reinterpret_cast<int*>(dyn);
   const int n4 = (n + 3) & ~3;
-  for (int i = tid; i < n4; i += kRoundThreads) s_rho[i] = i < n ? a.rho[i] : -1;
+#pragma unroll 6
+  for (int i = 4 * tid; i < n4; i += 4 * kRoundThreads) {
+    int r[4] = {-1, -1, -1, -1};
+    if (i + 4 <= n) {
+      const int4 v = *reinterpret_cast<const int4*>(a.rho + i);
+      r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
+    } else {
+      for (int j = 0; i + j < n; ++j) r[j] = a.rho[i + j];
+    }
+    *reinterpret_cast<int4*>(s_key + i) = make_int4(r[0] << 15 | (32767 - i), r[1] < 0 ? -1 : r[1] << 15 | (32766 - i),
+                                                    r[2] < 0 ? -1 : r[2] << 15 | (32765 - i), r[3] < 0 ? -1 : r[3] << 15 | (32764 - i));
+  }
   __syncthreads();
-  for (int e0 = (me * kRoundWarps + warp) * 4; e0 < n; e0 += G * kRoundWarps * 4) {
-    int mine[4], at[4] = {0, 0, 0, 0};
+  for (int e0 = (me * kRoundWarps + warp) * kPer; e0 < n; e0 += G * kRoundWarps * kPer) {
+    int mine[kPer], at[kPer] = {};
 #pragma unroll
-    for (int u = 0; u < 4; ++u) mine[u] = e0 + u < n ? s_rho[e0 + u] : 0;
+    for (int u = 0; u < kPer; ++u) mine[u] = e0 + u < n ? s_key[e0 + u] : 0;
+#pragma unroll 2
     for (int o = lane * 4; o < n4; o += 128) {
-      const int4 r = *reinterpret_cast<const int4*>(s_rho + o);
+      const int4 r = *reinterpret_cast<const int4*>(s_key + o);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {                       // (an entry in front of e0 + u wins a tie)
-        const int m = mine[u], e = e0 + u;
-        at[u] += (r.x >= m + (o >= e)) + (r.y >= m + (o + 1 >= e)) + (r.z >= m + (o + 2 >= e)) + (r.w >= m + (o + 3 >= e));
-      }
+      for (int u = 0; u < kPer; ++u) at[u] += (r.x > mine[u]) + (r.y > mine[u]) + (r.z > mine[u]) + (r.w > mine[u]);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kPer; ++u) {
       const int p = __reduce_add_sync(0xFFFFFFFFu, at[u]);
       if (lane == 0 && e0 + u < n) { a.queue[p] = e0 + u; a.place[e0 + u] = p; }
     }
   }
   unsigned nth = 0;
-  bool fine = grid_barrier(a, sh, ++nth);
+  grid_arrive(a);
+  bool fine = grid_wait(a, sh, ++nth);
   int n_clu = 0, from = 0, status = 0;                     // clusters written; bitmap words before `from` are all covered
   long long fill = 0;
 
@@ -388,12 +448,11 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
       if (w < bwords) b = (w * 32 + 32 <= n ? 0xFFFFFFFFu : (1u << (n - w * 32)) - 1u) & ~__ldcg(a.covered + w);
       int total;
       int rank = n_picks + block_prefix(sh, __popc(b), total);
-      for (; b && rank < G; b &= b - 1u, ++rank) {
-        const int p = w * 32 + __ffs(b) - 1;
-        sh.pick[rank] = __ldcg(a.queue + p);
-      }
+      for (; b && rank < G; b &= b - 1u, ++rank) sh.pick[rank] = w * 32 + __ffs(b) - 1;
       n_picks = min(G, n_picks + total);
     }
+    __syncthreads();
+    if (tid < n_picks) sh.pick[tid] = __ldcg(a.queue + sh.pick[tid]);   // (places first: their entries in one trip)
     __syncthreads();
     if (n_picks == 0) break;                               // (uniform over the grid: nobody covers before the next barrier)
     // ---- every CTA grows one and notes which of the others its cluster holds ----
@@ -401,12 +460,8 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
     const uint16_t* members = nullptr;
     if (me < n_picks) {
       const int m = sh.pick[me];
-      size = grow(a, sh, dyn, cap, m, &members);
       uint32_t* mark = reinterpret_cast<uint32_t*>(dyn + cap * 6);
-      for (int w = tid; w < bwords; w += kRoundThreads) mark[w] = 0u;
-      __syncthreads();
-      for (int i = 1 + tid; i < size; i += kRoundThreads) atomicOr(&mark[members[i] >> 5], 1u << (members[i] & 31));
-      __syncthreads();
+      size = grow(a, sh, dyn, cap, m, mark);
       if (tid < kMaxPicks) {
         const int e = tid < n_picks ? sh.pick[tid] : m;
         const uint32_t w = __ballot_sync(0xFFFFFFFFu, tid < n_picks && ((mark[e >> 5] >> (e & 31)) & 1u));
@@ -414,7 +469,9 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
       }
       if (tid == 0) a.size[me] = size;
     }
-    if (!(fine = grid_barrier(a, sh, ++nth))) break;
+    grid_arrive(a);
+    if (me < n_picks) members = list_members(sh, dyn, cap, a.rho[sh.pick[me]]);
+    if (!(fine = grid_wait(a, sh, ++nth))) break;
     // ---- the walk over them ----
     for (int i = tid; i < n_picks * kNoteWords; i += kRoundThreads) (&sh.holds[0][0])[i] = __ldcg(a.holds + i);
     if (tid < n_picks) sh.pick_size[tid] = __ldcg(a.size + tid);
@@ -460,7 +517,8 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
       }
     }
     if (status != 0) break;                                // (uniform over the grid)
-    fine = grid_barrier(a, sh, ++nth);
+    grid_arrive(a);
+    fine = grid_wait(a, sh, ++nth);
     from = __ldcg(a.place + sh.pick[0]) >> 5;              // everything in front of this round's first entry is covered
   }
   if (me == 0 && tid == 0) {

@@ -8,19 +8,22 @@
 //            Idempotent byte stores: concurrent writers store the same value, so the dedup needs no
 //            atomics.  Four independent slots per thread keep the dependent loads overlapped.
 //   tail     (the CTA that finishes marking last, found with one ticket counter)
-//     compact  ordered compaction of the flags -> uniq[] ascending by id: each lane takes 4 flags
-//              with one load (the replica masks and sizes of those clusters are requested in the same
-//              round trip), a warp scan places them; the flags are cleared on the way so the next call
-//              starts from zeros.  The clusters that need the serial pass are packed, with their output
-//              slots, into per-warp segments of an item list (shared memory when it fits).
+//     compact  ordered compaction of the flags -> uniq[] ascending by id: rows of 1024 clusters (flags, replica
+//              masks, sizes) travel through a cp.async ring in shared memory, one scan over the CTA places a
+//              row's ids; the flags are cleared on the way so the next call starts from zeros.  The clusters
+//              that need the serial pass are packed, with their output slots, into one dense list (shared
+//              memory; longer ones in global memory).
 //              With cache state attached (swarm_set_cache) the same pass drops the activated clusters
 //              that are resident (Eq. 8) and updates the activation frequencies and Eq. 6 scores.
 //     route    single-replica clusters go to their queue (integer histogram, order-free).  Clusters
-//              with R >= 2 replicas are visited by (R ascending, id ascending) by one warp: lane j
-//              keeps (load[j] << 5 | j); one redux.min over the lanes named by the replica mask
-//              picks the least-loaded replica with ties to the lowest queue id, and only the lane
-//              whose value equals the minimum adds the cluster's weight.
-//              Under SWARM_ORDER_BY_ID the same warp visits every cluster in id order instead.
+//              with R >= 2 replicas are visited by (R ascending, id ascending), each going to its
+//              least-loaded replica, ties to the lowest queue id: a chain, because every choice depends on
+//              the loads left by the one before it.  It bounds the serial step.  Three forms of it, all
+//              bit-identical: lanes_pass (two replicas, equal weights, up to 8 queues), levels_pass (two
+//              replicas, any weights, up to 16 queues), and for everything else one warp with a link per
+//              cluster -- lane j keeps (load[j] << 5 | j), one redux.min over the lanes named by the
+//              replica mask picks the queue.  Under SWARM_ORDER_BY_ID that warp visits every cluster in
+//              id order instead.
 //     submit   (optional output) the batched submission order of Sec. 5.1, see the end of the body.
 #pragma once
 #include "swarm_internal.cuh"
