@@ -81,6 +81,8 @@ def load_library() -> ctypes.CDLL:
         lib.swarm_workspace_bytes.restype = ctypes.c_int64
         lib.swarm_build_clusters_workspace_bytes.restype = ctypes.c_int64
         lib.swarm_cache_admit_workspace_bytes.restype = ctypes.c_int64
+        v, i32, i64 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
+        lib.swarm_build_clusters.argtypes = [v, i32, ctypes.c_float, v, i64, v, v, v, i64, v, v, v, v]
         _lib = lib
     return _lib
 
@@ -241,22 +243,29 @@ def swarm_build_clusters(dist: torch.Tensor, tau: float, members_cap: Optional[i
     n = int(dist.shape[0])
     if dist.dtype != torch.float32 or dist.dim() != 2 or dist.shape[1] != n:
         raise ValueError("dist must be a float32 [n][n] tensor")
-    lib = load_library()
+    if not (dist.is_cuda and dist.is_contiguous()):
+        raise ValueError("dist must be a contiguous CUDA tensor")
     ws_bytes = swarm_build_clusters_workspace_bytes(n)
     dev = dist.device
     cap = int(members_cap if members_cap is not None else 16 * n)
-    i32 = dict(dtype=torch.int32, device=dev)
+    # The calls' host time lies between two runs of the GPU (each ends in a copy to the host), so it is kept short: one
+    # allocation for the outputs, addresses by arithmetic, views made while the GPU works.
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
-    density, medoid, members = torch.empty(n, **i32), torch.empty(n, **i32), torch.empty(max(cap, 4), **i32)
-    head = torch.empty(n + 12, **i32)                # [0] clusters, [4] status, [8:] cluster_ptr: one copy to the host
-    ptr = head[8:]
-    _check(lib.swarm_build_clusters(_ptr(dist, "dist"), ctypes.c_int32(n), ctypes.c_float(tau), _ptr(ws),
-                                    ctypes.c_int64(ws_bytes), _ptr(density), _ptr(ptr), _ptr(members),
-                                    ctypes.c_int64(cap), _ptr(medoid), _ptr(head), _ptr(head[4:]),
-                                    _stream(stream)), "swarm_build_clusters")
+    row = (n + 3) & ~3
+    at_medoid, at_head, at_members = row, 2 * row, 3 * row + 12
+    out = torch.empty(at_members + max(cap, 4), dtype=torch.int32, device=dev)
+    base = out.data_ptr()
+    head = base + 4 * at_head                        # [0] clusters, [4] status, [8:] cluster_ptr: one copy to the host
+    _check(load_library().swarm_build_clusters(dist.data_ptr(), n, tau, ws.data_ptr(), ws_bytes, base, head + 32,
+                                               base + 4 * at_members, cap, base + 4 * at_medoid, head, head + 16,
+                                               _stream(stream)), "swarm_build_clusters")
     if stream is not None and stream != torch.cuda.current_stream(dev):   # the copy waits for the caller's stream
         torch.cuda.current_stream(dev).wait_stream(stream)
-    host = head.cpu()
+    density, medoid, ptr, members = out[:n], out[at_medoid:], out[at_head + 8:], out[at_members:]
+    host = torch.empty(at_members - at_head, dtype=torch.int32, pin_memory=True)
+    host.copy_(out[at_head:at_members], non_blocking=True)
+    torch.cuda.current_stream(dev).synchronize()
+    host = host.numpy()
     n_clusters, status = int(host[0]), int(host[4])
     if status == 2:
         raise SwarmError(ERR_CUDA, "swarm_build_clusters (a bounded wait ran out)")

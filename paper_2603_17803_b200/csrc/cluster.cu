@@ -717,16 +717,16 @@ cudaError_t launch_build_clusters(const float* dist, int n, float tau, void* wor
   a.ptr = ptr; a.members = members; a.members_cap = members_cap; a.medoid = medoid; a.n_clusters = n_clusters;
   a.dev_status = dev_status;
 
+  density_kernel<<<dim3((n + 7) / 8), dim3(256), 0, st>>>(a);   // (first: the rest of the host's work runs beside it)
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   int cap = 1024;                                          // power of two >= n: the candidates of one cluster
   while (cap < n) cap <<= 1;
   const int smem = cap * 6 + std::max(kCountedCand * 8, bit_words(n) * 4);
   int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  density_kernel<<<dim3((n + 7) / 8), dim3(256), 0, st>>>(a);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::max(1, std::min({sms, n, kMaxPicks})));   // one CTA per SM, each grows one cluster per round
