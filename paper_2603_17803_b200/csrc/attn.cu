@@ -105,6 +105,8 @@ attn_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
     bh0 = b * geo.Hq + kvh * geo.g + tile * 8;
     G = min(8, geo.g - tile * 8);
   } else {
+    // the last heads first: their buffers were written last and may still be in L2
+    grp = n_groups - 1 - grp;
     bh0 = grp;
     b = grp / geo.Hq;
     G = 1;

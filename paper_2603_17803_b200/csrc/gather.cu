@@ -13,11 +13,13 @@ namespace {
 // One warp per (b, h, slot j): copies the K block and the V block (adjacent in the pool) of page sel[b][h][j] for head
 // kv(h) into rows [j*S, (j+1)*S) of the head's gathered buffers.  Rows of padding tokens and whole
 // unused slots are written as zeros.
-// Bound by HBM (copies written, distinct pages read).  A warp keeps sixteen 512-byte loads in flight behind one trip for
-// the indices, sixteen warps per SM.  (A CTA of 256 threads per slot, two loads per thread behind three dependent trips, was
-// bound by the turn-over of its CTAs: 157 MB written from 79 MB 49 -> 43 us, 5.5 TB/s.)
-constexpr int kGatherThreads = 128, kGatherBatch = 16;
-__global__ void __launch_bounds__(kGatherThreads, 4)
+// Bound by HBM (copies written, distinct pages read).  A warp keeps four 512-byte loads in flight behind one trip for
+// the indices, 48 warps per SM.  (A CTA of 256 threads per slot, two loads per thread behind three dependent trips, was
+// bound by the turn-over of its CTAs.  157 MB written from 79 MB, behind the selection and the resolution: 55 -> 50 us;
+// 645 MB: 187 -> 187 us.  More bytes in flight help a gather that runs by itself, 45 -> 43 us at sixteen loads per lane, and
+// hurt one that starts on all SMs at once behind another kernel, 187 -> 197 us.)
+constexpr int kGatherThreads = 128, kGatherBatch = 4;
+__global__ void __launch_bounds__(kGatherThreads, 12)
 gather_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int32_t* __restrict__ sel,
               const int32_t* __restrict__ n_sel, const int64_t* __restrict__ page_base,
               const int32_t* __restrict__ ctx_len, uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out,
