@@ -922,6 +922,22 @@ def test_submit_order_full_size_and_bad_masks():
     sess.close()
 
 
+@pytest.mark.parametrize("batch,topics", [(1, 4), (11, 4)])
+def test_submit_order_at_the_ends_of_its_range(batch, topics):
+    """A list shorter than the warps that rank it (20 clusters), and one whose keys (45056) come to shared memory in two parts."""
+    pages = 40 if batch == 1 else 8192
+    cfg = small("c3_batched", batch=batch, ctx_len=16 * pages, top_k=pages, n_q_heads=1, n_kv_heads=1, n_topics=topics, cluster_pages=2,
+                replication="two", n_queues=12)
+    w = W.generate(cfg, seed=batch, device=DEV)
+    sess = Session(w)
+    sess.enable_submit_order()
+    sess.step()
+    torch.cuda.synchronize()
+    assert sess.status() == 0
+    assert check_submit_order(w, sess) == w.n_clusters
+    sess.close()
+
+
 # ---- Algorithm 1 (offline co-activation clustering) ---------------------------------------------------------
 def check_clusters(dist, tau, cap=None):
     density, ptr, members, medoid = B.swarm_build_clusters(dist, tau, members_cap=cap)
