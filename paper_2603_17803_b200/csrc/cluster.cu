@@ -555,7 +555,9 @@ admit_kernel(const float* __restrict__ score, const uint16_t* __restrict__ size,
     if (u == 0x80000000u) u = 0u;
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   };
+  pdl_launch_dependents();                                  // (its launch, and that of the kernel behind it, overlap)
   for (int i = tid; i < kAdmitBins; i += kAdmitThreads) hist[i] = 0u;
+  pdl_wait();
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll 4
   for (int c = tid; c < n; c += kAdmitThreads) {
@@ -688,8 +690,7 @@ long long cache_admit_workspace_bytes(int n) { return ((long long)n * 4 + 255) /
 cudaError_t launch_cache_admit(const float* score, const uint16_t* size, int n, long long capacity, void* workspace,
                                uint8_t* resident, int32_t* info, cudaStream_t st) {
   (void)workspace;                                         // nothing is sorted any more
-  admit_kernel<<<dim3(1), dim3(kAdmitThreads), 0, st>>>(score, size, n, capacity, resident, info);
-  return cudaGetLastError();
+  return launch_pdl(admit_kernel, dim3(1), dim3(kAdmitThreads), 0, st, true, score, size, n, capacity, resident, info);
 }
 
 namespace {
