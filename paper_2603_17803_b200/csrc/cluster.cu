@@ -15,7 +15,7 @@
 //
 // Growing one cluster: the candidates are sorted by (distance, index) in shared memory and visited in that order; one
 // joins when its running sum is within tau * |C|.  A CTA does this 32 candidates at a time, a thread per candidate: the
-// warp that owns the 32 decides them one after the other (a ballot and an add per join, operands in registers), the
+// warp that owns the 32 decides them one after the other (a ballot and an add per join, operands in a tile in shared memory), the
 // others then add the rows of those that joined.  The matrix entries a thread will need for the next 32 are loaded while
 // the present ones are decided.  Bound by those gathers: n_c^2 / 2 scattered words per cluster of n_c candidates, about
 // one 32-byte sector per two cycles and SM.  (As a walk that went to memory for every join it took 1.3 us per join.)
@@ -78,6 +78,8 @@ __global__ void __launch_bounds__(256) density_kernel(ClusterArgs a) {
 }
 
 // ---- rounds ----------------------------------------------------------------------------------------------------
+// 384 threads: with 512 the two blocks of operands that a thread holds spill (36 against 32 us for the largest clusters of
+// 8192 entries in 64 topics); more candidates than threads are rare and kept in shared memory.
 constexpr int kRoundThreads = 384, kRoundWarps = kRoundThreads / 32;
 constexpr int kCountedCand = 1024;                        // up to here candidates are sorted by counting
 constexpr unsigned kGridWaitLimit = 1u << 23;

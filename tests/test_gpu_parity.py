@@ -996,6 +996,20 @@ def test_algorithm1_on_unstructured_distances(n, frac, symmetric):
             B.swarm_build_clusters(dist, tau, members_cap=max(n, len(members_ref) - 1))
 
 
+@pytest.mark.parametrize("n", [2, 32, 34, 384, 385, 386, 1025, 1026])
+def test_algorithm1_at_the_ends_of_its_candidate_lists(n):
+    """Nearly every entry a candidate of every other: lists that end at a block of 32, at the 384 candidates that threads
+    hold and at the 1024 that are sorted by counting.  Distances in general position (few ties)."""
+    g = torch.Generator(device=DEV).manual_seed(n)
+    dist = torch.rand((n, n), generator=g, device=DEV)
+    dist.fill_diagonal_(0.0)
+    check = [oracle.build_clusters(dist.cpu().numpy(), tau, members_cap=400 * n) for tau in (0.999, 0.55)]
+    for tau, (rho, ptr_ref, members_ref, medoid_ref) in zip((0.999, 0.55), check):
+        density, ptr, members, medoid = B.swarm_build_clusters(dist, tau, members_cap=400 * n)
+        assert np.array_equal(density.cpu().numpy(), rho) and np.array_equal(medoid.cpu().numpy(), medoid_ref)
+        assert np.array_equal(ptr.cpu().numpy(), ptr_ref) and np.array_equal(members.cpu().numpy(), members_ref)
+
+
 def test_algorithm1_with_more_members_than_the_scratch_holds():
     """40 entries sit within reach of all 600, the others only of those: about 555 clusters of 41 members, more than the
     scratch list's 16 per entry, so most clusters are grown a second time for the output."""
