@@ -344,12 +344,18 @@ __device__ __forceinline__ unsigned levels_pass(uint32_t* mask, uint32_t* wgt, i
   return key;
 }
 
-// Dynamic shared memory, in words: the tables of the two passes above, then `cap` words each of what the serial pass works
-// on -- replica masks, weight << 5 (the chosen queue joins it in the low bits), output slots -- and, if a submission order
-// is wanted, of its keys and ranks.
+// Dynamic shared memory, in words: the tables of the two passes above, then what the serial pass works on, `cap` words
+// each -- replica masks and weight << 5 (the chosen queue joins it in the low bits), both with kBlanks words of room behind
+// them, output slots -- and, if a submission order is wanted, its keys and ranks.
+constexpr int kBlanks = 16;                              // blank clusters that follow the list: the flat loop fetches that far ahead
 __host__ __device__ constexpr int serial_cap(bool submit) {
-  return (((int)(kResolveSmemBytes / 4) - kPassWords) / (submit ? 5 : 3) - 24) & ~7;   // (16 blank ones behind the list)
+  return (((int)(kResolveSmemBytes / 4) - kPassWords) / (submit ? 5 : 3) - 24) & ~7;
 }
+__host__ __device__ constexpr int serial_words(bool submit) {
+  return kPassWords + 2 * (serial_cap(submit) + kBlanks) + (submit ? 3 : 1) * serial_cap(submit);
+}
+static_assert(serial_words(false) * 4 <= (int)kResolveSmemBytes && serial_words(true) * 4 <= (int)kResolveSmemBytes,
+              "the lists and their blanks fit behind the tables");
 
 // `cta` of `n_ctas` CTAs of kThreads threads run the body with kResolveSmemBytes of dynamic shared memory.
 template <bool kCached>
@@ -376,8 +382,8 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   const int cap = serial_cap(r.submit_order != nullptr);
   uint32_t* s_pass = reinterpret_cast<uint32_t*>(s_dyn);
   uint32_t* s_mask = s_pass + kPassWords;
-  uint32_t* s_wgt = s_mask + cap;
-  uint32_t* s_slot = s_wgt + cap;
+  uint32_t* s_wgt = s_mask + cap + kBlanks;
+  uint32_t* s_slot = s_wgt + cap + kBlanks;
   __shared__ int s_tot[2][kWarps];                       // clusters to fetch | those for the serial pass << 16, per warp, of two rows
   __shared__ int s_rows[kBuilders];
   __shared__ bool s_even;
@@ -650,7 +656,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   }
   if (err && !dry) atomicOr(status, err);
   err = 0u;
-  if (staged && tid < 16) s_mask[n_serial + tid] = s_wgt[n_serial + tid] = 0u;
+  if (staged && tid < kBlanks) s_mask[n_serial + tid] = s_wgt[n_serial + tid] = 0u;
   __syncthreads();
   SWARM_STAMP_ANY_CTA(status, 3);
 
@@ -698,6 +704,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     // of the next eight clusters are fetched while eight are decided, lane u keeps the queue of the u-th.
     if (flat && n_serial > 0) {
       constexpr int kAhead = 8;
+      static_assert(2 * kAhead <= kBlanks, "a turn that starts in the list fetches up to two turns' clusters");
       const uint32_t m_at = shared_addr(s_mask), w_at = shared_addr(s_wgt);
       unsigned m[kAhead], w[kAhead];
 #pragma unroll

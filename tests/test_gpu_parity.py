@@ -333,6 +333,40 @@ def test_schedules_longer_than_the_shared_list(batch, replication, sizes):
         sess.close()
 
 
+@pytest.mark.parametrize("order", [False, True])
+@pytest.mark.parametrize("over", [-16, -15, 0, 1])
+def test_schedules_at_the_capacity_of_the_shared_list(over, order):
+    """The serial pass keeps lists of up to 9928 clusters in shared memory, 5944 with a submission order, and lets blank
+    clusters follow them: lists that end 16 and 15 places short of the capacity, at it and behind it.  A cluster per
+    page, every page selected."""
+    n = (5944 if order else 9928) + over
+    cfg = small("c1_tiny", ctx_len=16 * n, top_k=n, n_q_heads=1, n_kv_heads=1, cluster_pages=1, n_queues=12)
+    w = W.generate(cfg, seed=n, device=DEV)
+    two = w.cluster_replica_mask.clone()
+    rng = np.random.default_rng(n)
+    third = torch.from_numpy(1 << rng.integers(0, 12, size=n).astype(np.int32)).to(DEV)
+    every_third = torch.arange(n, device=DEV) % 3 == 0
+    # all of two replicas, equal and unequal weights; two or three replicas; in id order with single replicas among them
+    for masks, sizes, flags in ((two, (8,), 0), (two, (1, 2, 7), 0), (torch.where(every_third, two | third, two), (3, 5), 0),
+                                (torch.where(every_third, third, two), (4, 9), B.ORDER_BY_ID)):
+        w.cluster_replica_mask = masks.contiguous()
+        w.cluster_size.copy_(torch.from_numpy(rng.choice(sizes, size=n).astype(np.uint16).view(np.int16)))
+        sess = Session(w, flags=flags)
+        if order:
+            sess.enable_submit_order()
+        sess.o.queue_of.fill_(255)
+        sess.step()
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        o = sess.o
+        uniq, _, _ = parity.check_resolve(w, parity.host_tables(w), o.sel.cpu().numpy(), o.n_sel.cpu().numpy(), o.uniq.cpu().numpy(),
+                                          o.queue_of.cpu().numpy(), o.n_uniq.cpu().numpy()[0], o.queue_load.cpu().numpy(), flags)
+        assert len(uniq) == n
+        if order:
+            assert check_submit_order(w, sess, flags) == n
+        sess.close()
+
+
 def test_all_equal_scores_pick_lowest_ids_and_signed_zero_ties():
     cfg = small("c1_tiny", ctx_len=16 * 300, top_k=20)
     w = W.generate(cfg, seed=8, device=DEV)
