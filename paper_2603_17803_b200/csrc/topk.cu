@@ -176,7 +176,8 @@ __device__ __forceinline__ void mark_cluster(const Geometry& geo, const TopkExtr
 template <int THREADS>
 struct SelectState {
   alignas(16) int hist[kBins<THREADS>];
-  int warp_tot[32], warp_out[32];
+  int warp_tot[32];
+  unsigned warp_out[32];   // pages above the threshold | pages at it << 16
   uint32_t red_min[32], red_max[32];
   uint32_t cand[kRankMax]; // candidate keys of the chosen bin, when few enough to finish by direct ranking
   int n_fill;          // fill counter of cand[]; zero at the start
@@ -192,9 +193,9 @@ __device__ __forceinline__ int hist_slot(uint32_t bin) { return (int)((uint32_t)
 
 // Sum of the totals of the warps before `warp` (THREADS / 32 <= 32 totals in shared memory): every warp reduces
 // the masked totals with shuffles instead of each thread adding them up one by one.
-template <int THREADS>
-__device__ __forceinline__ int totals_before(const int* warp_tot, int warp, int lane) {
-  int v = (lane < THREADS / 32 && lane < warp) ? warp_tot[lane] : 0;
+template <int THREADS, class T>
+__device__ __forceinline__ T totals_before(const T* warp_tot, int warp, int lane) {
+  T v = (lane < THREADS / 32 && lane < warp) ? warp_tot[lane] : 0;
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
   return v;
@@ -415,17 +416,17 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
     gt_mask = (gt_mask | win) & exist;
   }
   gt_mask &= ~eq_mask;
-  const int cnt = __popc(gt_mask) | (__popc(eq_mask) << 16);
-  int incl = cnt;
+  const unsigned cnt = (unsigned)__popc(gt_mask) | ((unsigned)__popc(eq_mask) << 16);
+  unsigned incl = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    const unsigned t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += t;
   }
   if (lane == 31) st.warp_out[warp] = incl;
   __syncthreads();
-  const int before = incl - cnt + totals_before<THREADS>(st.warp_out, warp, lane);
-  const int gt_before = before & 0xFFFF, eq_before = before >> 16;
+  const unsigned before = incl - cnt + totals_before<THREADS>(st.warp_out, warp, lane);
+  const int gt_before = (int)(before & 0xFFFFu), eq_before = (int)(before >> 16);
   // The page bitmap goes out first and the head is announced to the attention CTAs right behind it: a release
   // waits for every store issued before it to be acknowledged, so the selection list, the cluster marks and the
   // rest (which the attention does not read) are stored after the announcement, not before.
@@ -683,19 +684,20 @@ topk_smem_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
   __syncthreads();
   // thread t places the pages of words [w0, w1)
   const int per = (words + THREADS - 1) / THREADS, w0 = min(words, tid * per), w1 = min(words, w0 + per);
-  int cnt = 0;
-  for (int w = w0; w < w1; ++w) cnt += __popc(s_gt[w]) | (__popc(s_eq[w]) << 16);
-  int incl = cnt;
+  unsigned cnt = 0u;                                        // (unsigned: more than 32767 pages may be at the threshold)
+  for (int w = w0; w < w1; ++w) cnt += (unsigned)__popc(s_gt[w]) | ((unsigned)__popc(s_eq[w]) << 16);
+  unsigned incl = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    const unsigned t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += t;
   }
   if (lane == 31) st.warp_out[warp] = incl;
   __syncthreads();
-  const int before = incl - cnt + totals_before<THREADS>(st.warp_out, warp, lane);
+  const unsigned before = incl - cnt + totals_before<THREADS>(st.warp_out, warp, lane);
+  const int gt_before = (int)(before & 0xFFFFu), eq_before = (int)(before >> 16);
   // the bitmap first, then the announcement, then the list and the cluster marks (see topk_regs_body)
-  int eq_left = max(0, need_eq - (before >> 16));           // pages at the threshold this thread may still take
+  int eq_left = max(0, need_eq - eq_before);           // pages at the threshold this thread may still take
   for (int w = w0; w < w1; ++w) {
     unsigned eq = s_eq[w];
     while (__popc(eq) > eq_left) eq &= ~(0x80000000u >> __clz(eq));   // the lowest ids win
@@ -708,7 +710,7 @@ topk_smem_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
     for (int w = words + tid; 4 * w + 4 <= x.selmap_pitch; w += THREADS)
       reinterpret_cast<uint32_t*>(x.selmap + (long long)bh * x.selmap_pitch)[w] = 0u;
   selection_announce(geo, x, b, kvh);
-  int place = (before & 0xFFFF) + min(before >> 16, need_eq);
+  int place = gt_before + min(eq_before, need_eq);
   for (int w = w0; w < w1; ++w) {
     for (unsigned todo = s_gt[w]; todo != 0u;) {
       // four pages at a time, their table reads in front of the flag stores (see topk_regs_body)
@@ -866,7 +868,8 @@ topk_generic_kernel(Geometry geo, const float* __restrict__ scores, const int32_
 size_t smem_key_bytes(int Pmax, int threads) {
   return (size_t)((Pmax + 31) & ~31) * 4 + (smem_words_in_hist(Pmax, threads) ? 0 : (size_t)((Pmax + 31) / 32) * 8);
 }
-constexpr size_t kSmemKeyBytes = 200 * 1024;               // 48 K pages
+constexpr size_t kSmemKeyBytes = 200 * 1024;               // 48160 pages
+static_assert(kSmemKeyBytes / 4 < 65536, "a list's counts are packed two to a word");
 
 }  // namespace
 

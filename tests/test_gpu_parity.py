@@ -792,6 +792,41 @@ def test_selection_of_many_long_lists(pages, top_k, window):
     sess.close()
 
 
+@pytest.mark.parametrize("heads", [4, 136])
+@pytest.mark.parametrize("pages,top_k,window", [(32769, 150, 0), (40000, 64, 0), (40000, 39000, 7), (48160, 150, 5), (48160, 48000, 0), (48161, 150, 0)])
+def test_selection_where_more_pages_tie_than_a_signed_half_word_holds(pages, top_k, window, heads):
+    """Long lists with nearly all scores equal, as few lists and as many, up to the longest one with its keys in shared
+    memory (48160 pages) and one page more.  The keys of all but 100 pages are zero, so those tie at score 0 behind
+    the 100; for the first head the query is zero and every page ties."""
+    cfg = small("c1_tiny", ctx_len=16 * pages - 3, top_k=top_k, n_q_heads=heads, n_kv_heads=1)
+    w = W.generate(cfg, seed=pages, device=DEV)
+    keep = torch.randperm(pages, generator=torch.Generator().manual_seed(pages))[:100].to(DEV)
+    some = w.kv_pool[keep, :, 0].clone()
+    w.kv_pool[:, :, 0] = 0
+    w.kv_pool[keep, :, 0] = some
+    w.q[0, 0] = 0
+    sess = Session(w, keep_scores=True, local_window_pages=window)
+    lens = w.ctx_len.cpu().numpy()
+
+    def check():
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        sc, sel, n_sel = (t.cpu().numpy() for t in (sess.o.scores, sess.o.sel, sess.o.n_sel))
+        assert (sc == 0).sum(axis=-1).min() >= pages - 100
+        want, n_want = oracle.topk(sc, lens, cfg.page_size, top_k, window)
+        assert np.array_equal(sel, want) and np.array_equal(n_sel, n_want)
+        return sel, n_sel
+
+    sess.select()
+    check()
+    if heads == 4:                                          # inside the step it marks the selected pages' clusters too
+        sess.step()
+        sel, n_sel = check()
+        parity.check_resolve(w, parity.host_tables(w), sel, n_sel, sess.o.uniq.cpu().numpy(), sess.o.queue_of.cpu().numpy(),
+                             sess.o.n_uniq.cpu().numpy()[0], sess.o.queue_load.cpu().numpy())
+    sess.close()
+
+
 @pytest.mark.parametrize("pages", [900, 2000, 4000, 8000, 16000, 30000, 45000])
 @pytest.mark.parametrize("window", [0, 5])
 def test_selection_at_every_list_length(pages, window):
