@@ -557,9 +557,9 @@ admit_kernel(const float* __restrict__ score, const uint16_t* __restrict__ size,
     if (u == 0x80000000u) u = 0u;
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   };
-  pdl_launch_dependents();                                  // (its launch, and that of the kernel behind it, overlap)
   for (int i = tid; i < kAdmitBins; i += kAdmitThreads) hist[i] = 0u;
-  pdl_wait();
+  pdl_wait();                                               // (its launch, and that of the kernel behind it, overlap)
+  pdl_launch_dependents();
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll 4
   for (int c = tid; c < n; c += kAdmitThreads) {

@@ -24,8 +24,8 @@ gather_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int32_t*
               const int32_t* __restrict__ n_sel, const int64_t* __restrict__ page_base,
               const int32_t* __restrict__ ctx_len, uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out,
               int32_t* __restrict__ n_tok, uint32_t* __restrict__ status) {
-  pdl_launch_dependents();
   pdl_wait();                                               // (its launch overlaps what precedes it in the stream)
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const long long u = (long long)blockIdx.x * (kGatherThreads / 32) + (threadIdx.x >> 5);
   if (u >= (long long)geo.B * geo.Hq * geo.k) return;
@@ -100,8 +100,8 @@ constexpr int kSummaryThreads = 256;
 __global__ void __launch_bounds__(kSummaryThreads, 4)
 summaries_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int64_t* __restrict__ page_base,
                  const int32_t* __restrict__ ctx_len, uint16_t* __restrict__ ksum, uint32_t* __restrict__ status) {
-  pdl_launch_dependents();
   pdl_wait();                                               // (its launch overlaps what precedes it in the stream)
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const int S = geo.S;
   if (blockIdx.x == 0) {                                    // lengths that do not fit their pages

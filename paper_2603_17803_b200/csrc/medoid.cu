@@ -22,8 +22,8 @@ __global__ void __launch_bounds__(kRowThreads)
 medoid_rows_kernel(Geometry geo, const uint16_t* __restrict__ ksum, const int64_t* __restrict__ page_base,
                    const int64_t* __restrict__ cluster_base, const int32_t* __restrict__ medoid_page,
                    uint16_t* __restrict__ medoid_ksum, int32_t* __restrict__ len, uint32_t* __restrict__ status) {
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();                                  // (behind the wait: the pseudo lengths are read ahead of one)
   if (blockIdx.x == 0)
     for (int b = threadIdx.x; b < geo.B; b += kRowThreads)
       len[b] = (int32_t)min((long long)(cluster_base[b + 1] - cluster_base[b]) * geo.S, 0x7FFFFFFFLL);

@@ -394,8 +394,8 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   __shared__ int s_hits;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  pdl_launch_dependents();                               // the next kernel in the stream may be scheduled while this one runs
   if (sel != nullptr) pdl_wait();                        // (on its own, any input may come from the previous kernel)
+  pdl_launch_dependents();                               // the next kernel in the stream may be scheduled while this one runs
   const long long c_all = cluster_base[geo.B];           // inside a step an input table: not written by the previous kernel
   const int C = (int)min((long long)geo.Cmax, c_all);
   unsigned err = 0u, step_no = 0u;

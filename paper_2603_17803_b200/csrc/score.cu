@@ -80,8 +80,8 @@ page_score_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
   constexpr int NV = G * R;
   constexpr int LOG_NV = ilog2(NV), LOG_G = ilog2(G);
   static_assert(NV <= 32 && (1 << LOG_NV) == NV && (1 << LOG_G) == G, "R and G must be powers of two, R*G <= 32");
-  pdl_launch_dependents();   // the next kernel may be scheduled as soon as every CTA of this one runs
   pdl_wait();                // launched behind whatever precedes it in the stream (see launch_mma)
+  pdl_launch_dependents();   // behind the wait: the selection reads its lengths ahead of its own
   SWARM_STAMP(status, 0);
   SWARM_KERNEL_BEGIN(status, 0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

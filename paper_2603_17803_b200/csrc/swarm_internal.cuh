@@ -324,6 +324,11 @@ __device__ __forceinline__ int pages_of(int ctx_len, int S) { return (ctx_len + 
 // Programmatic dependent launch: a kernel launched with the programmatic-serialization attribute may
 // start while its predecessor in the stream is still running; it must call pdl_wait() before it
 // touches anything the predecessor writes.  Both are no-ops for ordinary launches.
+// A kernel lets its dependents go only BEHIND its own wait.  Then everything in front of a kernel's direct predecessor has
+// finished by the time the kernel starts, and what it reads ahead of its wait (lengths, table bases, with the index
+// prefetch the first summaries) may have been written by any operation but the one directly before.  The selection and the
+// expansion of clusters, which trigger first thing, stand behind a kernel of the same call that keeps the rule and
+// writes none of that.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 

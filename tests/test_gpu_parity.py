@@ -657,6 +657,70 @@ def test_index_prefetch_changes_no_result(name, tail):
     ref.close()
 
 
+@pytest.mark.parametrize("between", ["medoid_rows", "admission", "gathered_attention"])
+@pytest.mark.parametrize("name", ["c2_small", "c3_small"])
+def test_index_update_one_operation_ahead_of_a_prefetching_step(name, between):
+    """The contract of the index prefetch: the operation directly before the step writes none of the index, one further up
+    may.  The pool is rewritten between turns, its summaries are built again, one other call follows, then the step."""
+    w = W.generate(CASES[name], seed=18, device=DEV)
+    pools = [w.kv_pool.clone(), W.generate(CASES[name], seed=19, device=DEV).kv_pool]
+    want = []
+    for pool in pools:
+        w.kv_pool.copy_(pool)
+        ref = Session(w)
+        torch.cuda.synchronize()
+        ref.step()
+        parity.check_step(w, ref)
+        want.append({k: getattr(ref.o, k).clone() for k in ("sel", "n_sel", "out", "lse")})
+        ref.close()
+    sess = Session(w, keep_gathered=True, index_prefetch=True)
+    sess.enable_medoid_index(5)
+    sess.outputs = B.make_outputs(**{k: None if k in ("k_out", "v_out", "n_tok") else getattr(sess.o, k) for k in sess.o.__dataclass_fields__})
+    sess.select()
+    sess.gather()
+    score = torch.rand(w.n_clusters, device=DEV)
+    resident = torch.zeros(w.n_clusters, dtype=torch.uint8, device=DEV)
+    for turn in range(6):
+        w.kv_pool.copy_(pools[turn % 2])
+        B.swarm_build_summaries(sess.ctx, sess.inputs, sess.ksum)
+        if between == "medoid_rows":
+            B.swarm_build_medoid_index(sess.ctx, sess.inputs, sess.medoid_page, sess.medoid_ksum, sess.cluster_ctx_len)
+        elif between == "admission":
+            B.swarm_cache_admit(score, w.cluster_size, w.n_pool_pages // 4, resident)
+        else:
+            sess.sparse_attn()
+        sess.step()
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        for k, v in want[turn % 2].items():
+            assert torch.equal(getattr(sess.o, k), v), (turn, k)
+    sess.close()
+
+
+@pytest.mark.parametrize("scorer", [B.SCORER_AUTO, B.SCORER_FP32])
+def test_medoid_step_directly_behind_its_index_build(scorer):
+    """The pseudo lengths and the rows are rewritten right in front of the step that reads them, with either scorer."""
+    w = W.generate(CASES["c5_small"], seed=20, device=DEV)
+    sess = Session(w, scorer=scorer)
+    sess.enable_medoid_index(7, keep_scores=True)
+    torch.cuda.synchronize()
+    sess.step_medoid()
+    check_medoid_step(w, sess, 7)
+    keys = ("sel_clusters", "n_sel_clusters", "cluster_scores")
+    want = {k: getattr(sess, k).clone() for k in keys}
+    out = sess.o.out.clone()
+    for _ in range(6):
+        sess.medoid_ksum.zero_()
+        sess.cluster_ctx_len.fill_(1)
+        B.swarm_build_medoid_index(sess.ctx, sess.inputs, sess.medoid_page, sess.medoid_ksum, sess.cluster_ctx_len)
+        sess.step_medoid()
+        torch.cuda.synchronize()
+        assert sess.status() == 0 and torch.equal(sess.o.out, out)
+        for k, v in want.items():
+            assert torch.equal(getattr(sess, k), v), k
+    sess.close()
+
+
 @pytest.mark.parametrize("name", ["c3_small", "c5_small"])
 def test_resident_filter_and_cache_counters(name):
     """Eq. 8 with the resident term, activation frequencies and Eq. 6 scores, against the oracle on the GPU's
