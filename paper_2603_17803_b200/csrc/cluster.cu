@@ -18,7 +18,8 @@
 // warp that owns the 32 decides them one after the other (a ballot and an add per join, operands in a tile in shared memory), the
 // others then add the rows of those that joined.  The matrix entries a thread will need for the next 32 are loaded while
 // the present ones are decided.  Bound by those gathers: n_c^2 / 2 scattered words per cluster of n_c candidates, about
-// one 32-byte sector per two cycles and SM.  (As a walk that went to memory for every join it took 1.3 us per join.)
+// one 32-byte sector per two cycles and SM.  (As a walk that went to memory for every join it took 1.3 us per join.)  Lists
+// that hold much of the matrix take whole rows instead.
 // A candidate's sum is a plain fp32 accumulation in joining order over D[member][candidate], so every decision is the
 // one a sequential fp32 walk takes.
 #include "swarm_internal.cuh"
@@ -283,60 +284,55 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
 
   // ---- the walk over the candidates, 32 at a time ----
   const int blocks = (n_cand + 31) / 32;
-  float* sum = reinterpret_cast<float*>(key);
-  for (int i = tid; i < 32 * blocks; i += kRoundThreads) {
-    if (i < n_cand) sum[i] = key_dist(key[i]);
-    else { sum[i] = __int_as_float(0x7FFFFFFF); idx[i] = (uint16_t)m; }   // no candidate: NaN passes no bound
-  }
+  // Candidate t's sum lies in a register of thread t; candidates from kRoundThreads on have theirs in shared memory.
+  const float kNever = __int_as_float(0x7FFFFFFF);        // no candidate: NaN passes no bound
+  for (int i = n_cand + tid; i < 32 * blocks; i += kRoundThreads) idx[i] = (uint16_t)m;
+  float s = tid < n_cand ? key_dist(key[tid]) : kNever;
   if (tid < kRoundWarps) sh.likely[tid] = 0xFFFFFFFFu;
   for (int w = tid; w < bit_words(n); w += kRoundThreads) mark[w] = 0u;   // (where the collected candidates were)
   __syncthreads();
-  // thread t holds candidate t's sum in a register; candidates from kRoundThreads on have theirs in shared memory
-  const bool have = tid < 32 * blocks;
-  float s = have ? sum[tid] : 0.f;
-  const int c0 = have ? idx[tid] : m;
+  const int c0 = tid < 32 * blocks ? idx[tid] : m;
   float* tile = reinterpret_cast<float*>(raw_entry);      // the operands of the block being decided
   int size = 1;
+  // Block b's members, by the warp that holds the sums x of its candidates and their operands val.
+  auto decide = [&](int b, float x, float (&val)[32]) {
+    // A link of the chain is a load from shared memory, an add, a compare and a ballot, and there is one per member:
+    // candidates that no join lets in are passed over on the ballot of the last one.  (Unrolled over the 32 registers
+    // the warp waited for instructions: 2900 cycles per 32 candidates.)
+#pragma unroll
+    for (int k = 0; k < 32; ++k) tile[32 * k + lane] = val[k];
+    uint32_t joined = 0u, above = 0xFFFFFFFFu;
+    float members = (float)size + 1.f, bound = a.tau * (float)size, next = a.tau * members;
+    for (;;) {
+      const uint32_t pass = __ballot_sync(0xFFFFFFFFu, x <= bound) & above;
+      if (pass == 0u) break;
+      const int k = __ffs(pass) - 1;
+      const float v = tile[32 * k + lane];                // (written by this lane)
+      joined |= 1u << k;
+      above = 0xFFFFFFFEu << k;
+      x += v;                                             // (of no account for the lanes up to k)
+      bound = next;
+      members += 1.f;
+      next = a.tau * members;
+    }
+    if (lane == 0) sh.joined[b] = joined;
+  };
   float cur[32], nxt[32];
   uint32_t cur_have = 0u, nxt_have = 0u;                  // rows loaded (a row is left out while its candidate looks hopeless)
+  const int first = min(blocks, kRoundWarps);             // blocks in registers
   auto fetch = [&](int b, float (&val)[32], uint32_t& loaded) {
     loaded = 0u;
-    if (b < blocks && b < kRoundWarps && warp >= b && warp < blocks) {
+    if (b < first && warp >= b && warp < first) {
       loaded = warp == b ? 0xFFFFFFFFu : *reinterpret_cast<volatile uint32_t*>(&sh.likely[b]);
       load_block(a, idx, b, loaded, tid, c0, val);
     }
   };
   auto step = [&](int b, float (&val)[32], uint32_t loaded) {
-    const int owner = b % kRoundWarps;
-    if (warp == owner) {
-      const int i = 32 * b + lane;                        // this lane's candidate
-      float x = b < kRoundWarps ? s : sum[i];
-      if (b >= kRoundWarps) load_block(a, idx, b, 0xFFFFFFFFu, i, idx[i], val);
-      // A link of the chain is a load from shared memory, an add, a compare and a ballot, and there is one per member:
-      // candidates that no join lets in are passed over on the ballot of the last one.  (Unrolled over the 32 registers
-      // the warp waited for instructions: 2900 cycles per 32 candidates.)
-#pragma unroll
-      for (int k = 0; k < 32; ++k) tile[32 * k + lane] = val[k];
-      uint32_t joined = 0u, above = 0xFFFFFFFFu;
-      float members = (float)size + 1.f, bound = a.tau * (float)size, next = a.tau * members;
-      for (;;) {
-        const uint32_t pass = __ballot_sync(0xFFFFFFFFu, x <= bound) & above;
-        if (pass == 0u) break;
-        const int k = __ffs(pass) - 1;
-        const float v = tile[32 * k + lane];              // (written by this lane)
-        joined |= 1u << k;
-        above = 0xFFFFFFFEu << k;
-        x += v;                                           // (of no account for the lanes up to k)
-        bound = next;
-        members += 1.f;
-        next = a.tau * members;
-      }
-      if (lane == 0) sh.joined[b] = joined;
-    }
+    if (warp == b) decide(b, s, val);
     __syncthreads();
     const uint32_t joined = sh.joined[b];
     size += __popc(joined);
-    if (b < kRoundWarps && warp > b && warp < blocks) {   // the sums of the candidates behind the block
+    if (warp > b && warp < first) {                       // the sums of the candidates behind the block
       uint32_t late = joined & ~loaded;
       while (late) {                                      // (joined against expectation: loaded now)
         const int k = __ffs(late) - 1;
@@ -350,23 +346,90 @@ __device__ int grow(const ClusterArgs& a, RoundShared& sh, unsigned char* smem, 
       const unsigned hint = __ballot_sync(0xFFFFFFFFu, s <= 1.25f * a.tau * (float)size);
       if (lane == 0) sh.likely[warp] = hint;              // an average a quarter above the radius is not about to join
     }
-    for (int i = tid + kRoundThreads; i < n_cand; i += kRoundThreads) {
-      if (i < 32 * (b + 1)) continue;
-      const int c = idx[i];
-      float v[32], x = sum[i];
-      load_block(a, idx, b, joined, i, c, v);
+  };
+
+  // ---- the candidates behind those ----
+  // A member costs the remaining candidates a gather of a 32-byte sector each, or all entries its whole row, n / 8 sectors
+  // in order: rows while more than an eighth of the matrix remains, on sums that lie by entry then.  (Gathers alone against
+  // this: one cluster of 8192 entries 22.9 and 7.4 ms, of 16384 entries 259 and 29, 8192 entries in 8 topics 3.05 and
+  // 3.13.  A quarter as the line: 24000 entries in 8 topics 62 -> 129 ms; a sixteenth: 8192 in 16 topics 0.93 -> 1.14.)
+  float* sum = reinterpret_cast<float*>(key);
+  const bool more = n_cand > kRoundThreads;
+  auto rows_pay = [&](int b) { return 8 * (n_cand - max(32 * (b + 1), kRoundThreads)) > n; };
+  const bool by_entry = more && rows_pay(0);
+  if (by_entry) {                                         // (all keys that are still wanted have been read)
+    for (int e = tid; e < n; e += kRoundThreads) sum[e] = __ldg(row_m + e);
+  } else {
+    for (int i = tid + kRoundThreads; i < n_cand; i += kRoundThreads) sum[i] = key_dist(key[i]);   // (thread i mod 384, as below)
+  }
+  auto fetch_tile = [&](int b) {                          // by the warp that decides block b, a block ahead
+    if (b < blocks && warp == b % kRoundWarps) load_block(a, idx, b, 0xFFFFFFFFu, 32 * b + lane, idx[32 * b + lane], cur);
+  };
+  // block b's members join the sums
+  auto add = [&](int b) {
+    const uint32_t joined = sh.joined[b];
+    if (joined == 0u) return;
+    if (rows_pay(b)) {
+      for (int e0 = tid; e0 < n; e0 += 4 * kRoundThreads) {
+        float x[4];
 #pragma unroll
-      for (int k = 0; k < 32; ++k) if ((joined >> k) & 1u) x += v[k];
-      sum[i] = x;
+        for (int u = 0; u < 4; ++u) x[u] = e0 + u * kRoundThreads < n ? sum[e0 + u * kRoundThreads] : 0.f;
+        for (uint32_t todo = joined; todo != 0u;) {
+          float v[8][4];                                  // eight rows by four entries in flight, added in joining order
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const bool has = todo != 0u;
+            const float* row = a.dist + (long long)idx[32 * b + (has ? __ffs(todo) - 1 : 0)] * n;
+            todo &= todo - 1u;                            // 0 stays 0
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              v[r][u] = has && e0 + u * kRoundThreads < n ? __ldg(row + e0 + u * kRoundThreads) : 0.f;
+          }
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] += v[r][u];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (e0 + u * kRoundThreads < n) sum[e0 + u * kRoundThreads] = x[u];
+      }
+    } else {
+      for (int i = tid + kRoundThreads; i < n_cand; i += kRoundThreads) {
+        if (i < 32 * (b + 1)) continue;
+        const int c = idx[i], at = by_entry ? c : i;
+        float v[32], x = sum[at];
+        load_block(a, idx, b, joined, i, c, v);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) if ((joined >> k) & 1u) x += v[k];
+        sum[at] = x;
+      }
     }
   };
+
   fetch(0, cur, cur_have);
-  for (int b = 0; b < blocks; b += 2) {
+  for (int b = 0; b < first; b += 2) {
     fetch(b + 1, nxt, nxt_have);
     step(b, cur, cur_have);
-    if (b + 1 >= blocks) break;
+    if (b + 1 >= first) break;
     fetch(b + 2, cur, cur_have);
     step(b + 1, nxt, nxt_have);
+    if (more) {                                           // (fills the wait for the next block's operands)
+      for (int q = b; q < b + 2; ++q) add(q);
+    }
+  }
+  if (more) {
+    fetch_tile(kRoundWarps);
+    for (int b = kRoundWarps; b < blocks; ++b) {
+      if (by_entry) __syncthreads();                      // (rows leave an entry's sum with another thread than gathers and decisions)
+      if (warp == b % kRoundWarps) {
+        const int i = 32 * b + lane;                      // this lane's candidate
+        decide(b, i < n_cand ? sum[by_entry ? idx[i] : i] : kNever, cur);
+      }
+      __syncthreads();
+      size += __popc(sh.joined[b]);
+      fetch_tile(b + 1);
+      add(b);
+    }
   }
   __syncthreads();
   for (int i = tid; i < n_cand; i += kRoundThreads)

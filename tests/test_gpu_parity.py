@@ -1143,6 +1143,26 @@ def test_algorithm1_at_the_ends_of_its_candidate_lists(n):
         assert np.array_equal(ptr.cpu().numpy(), ptr_ref) and np.array_equal(members.cpu().numpy(), members_ref)
 
 
+@pytest.mark.parametrize("n,reach", [(1024, 513), (1024, 514), (3075, 769), (3075, 770), (2050, 2050), (8193, 8193)])
+def test_algorithm1_on_lists_whose_sums_are_kept_by_entry(n, reach):
+    """Eight entries within the radius of the first `reach`, which lie at random from one another, about half of them within
+    it: lists of reach - 1 and about half as many candidates of which some join.  The lengths are those at which the sums of
+    candidates behind the first 384 move from the candidates' order to the entries' (8 (reach - 1 - 384) > n), and lists of
+    all entries."""
+    g = torch.Generator(device=DEV).manual_seed(n + reach)
+    dist = torch.rand((n, n), generator=g, device=DEV)
+    dist[reach:] = 2.0
+    dist[:, reach:] = 2.0
+    dist[:8, :reach] = 0.25 + dist[:8, :reach] / 16
+    dist[:reach, :8] = dist[:8, :reach].T
+    dist.fill_diagonal_(0.0)
+    rho, ptr_ref, members_ref, medoid_ref = oracle.build_clusters(dist.cpu().numpy(), 0.5, members_cap=400 * n)
+    assert rho.max() == reach - 1 and len(medoid_ref) > n - reach
+    density, ptr, members, medoid = B.swarm_build_clusters(dist, 0.5, members_cap=400 * n)
+    assert np.array_equal(density.cpu().numpy(), rho) and np.array_equal(medoid.cpu().numpy(), medoid_ref)
+    assert np.array_equal(ptr.cpu().numpy(), ptr_ref) and np.array_equal(members.cpu().numpy(), members_ref)
+
+
 def test_algorithm1_with_more_members_than_the_scratch_holds():
     """40 entries sit within reach of all 600, the others only of those: about 555 clusters of 41 members, more than the
     scratch list's 16 per entry, so most clusters are grown a second time for the output."""
