@@ -254,12 +254,15 @@ def swarm_build_clusters(dist: torch.Tensor, tau: float, members_cap: Optional[i
     row = (n + 3) & ~3
     at_medoid, at_head, at_members = row, 2 * row, 3 * row + 12
     out = torch.empty(at_members + max(cap, 4), dtype=torch.int32, device=dev)
+    other = stream is not None and stream != torch.cuda.current_stream(dev)
+    if other:                                        # the memory just taken may still be in use on the current stream
+        stream.wait_stream(torch.cuda.current_stream(dev))
     base = out.data_ptr()
     head = base + 4 * at_head                        # [0] clusters, [4] status, [8:] cluster_ptr: one copy to the host
     _check(load_library().swarm_build_clusters(dist.data_ptr(), n, tau, ws.data_ptr(), ws_bytes, base, head + 32,
                                                base + 4 * at_members, cap, base + 4 * at_medoid, head, head + 16,
                                                _stream(stream)), "swarm_build_clusters")
-    if stream is not None and stream != torch.cuda.current_stream(dev):   # the copy waits for the caller's stream
+    if other:                                        # the copy waits for the caller's stream
         torch.cuda.current_stream(dev).wait_stream(stream)
     density, medoid, ptr, members = out[:n], out[at_medoid:], out[at_head + 8:], out[at_members:]
     host = torch.empty(at_members - at_head, dtype=torch.int32, pin_memory=True)

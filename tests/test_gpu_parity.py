@@ -1,4 +1,6 @@
 """GPU parity tests: every call goes through the C-ABI library and is compared with the CPU oracle."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -1187,6 +1189,56 @@ def test_algorithm1_hand_case_and_capacity():
         B.swarm_build_clusters(dist, 0.5, members_cap=5)
     with pytest.raises(B.SwarmError):
         B.swarm_build_clusters(dist, -1.0)
+
+
+def test_algorithm1_on_a_stream_beside_pending_work():
+    """The outputs may be memory that work still pending on the current stream is about to write: the call's stream waits
+    for it."""
+    n, cap = 64, 300000
+    dist = W.coactivation_distances(n, 4, seed=3, device=DEV)
+    want = B.swarm_build_clusters(dist, 0.4, members_cap=cap)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        blocks = [torch.empty(words, dtype=torch.int32, device=DEV) for words in (cap + 4 * n, cap + 3 * n + 12)]
+        torch.cuda._sleep(20_000_000)                       # about 10 ms in front of the writes
+        for t in blocks:
+            t.fill_(7)
+        del blocks, t
+        got = B.swarm_build_clusters(dist, 0.4, members_cap=cap, stream=side)
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
+
+
+def test_algorithm1_from_two_threads_on_streams_of_their_own():
+    """Two threads cluster different matrices at the same time, one of them beside decode steps of a third stream."""
+    dists = [W.coactivation_distances(n, n // 32, seed=n, device=DEV) for n in (2048, 1500)]
+    want = [B.swarm_build_clusters(d, 0.4) for d in dists]
+    w = W.generate(CASES["c2_small"], seed=21, device=DEV)
+    sess = Session(w)
+    sess.step()
+    torch.cuda.synchronize()
+    out = sess.o.out.clone()
+    wrong = []
+
+    def work(i):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(25):
+                got = B.swarm_build_clusters(dists[i], 0.4)
+                if not all(torch.equal(a, b) for a, b in zip(got, want[i])):
+                    wrong.append(i)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for _ in range(200):
+        sess.step()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not wrong and sess.status() == 0 and torch.equal(sess.o.out, out)
+    sess.close()
 
 
 def test_algorithm1_clusters_drive_the_medoid_step():
