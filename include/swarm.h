@@ -376,7 +376,7 @@ int32_t swarm_step_medoid(swarm_ctx* ctx, const swarm_inputs* inputs, const swar
  * (cluster_size, pages) still fit into capacity_pages; the first cluster that does not fit ends the admission.
  * Writes resident[c] = 1 or 0 for every cluster -- the table swarm_set_cache reads -- and, if info is not NULL,
  * info[0] = clusters admitted, info[1] = pages used.  Device pointers, 16-byte aligned; n_clusters <= 65536;
- * workspace: swarm_cache_admit_workspace_bytes(n_clusters) bytes (< 0: minus an error code). */
+ * workspace: swarm_cache_admit_workspace_bytes(n_clusters) bytes (< 0: minus an error code); checked, but not used at present. */
 int64_t swarm_cache_admit_workspace_bytes(int32_t n_clusters);
 int32_t swarm_cache_admit(const float* score, const uint16_t* cluster_size, int32_t n_clusters, int64_t capacity_pages,
                           void* workspace, int64_t workspace_bytes, uint8_t* resident, int32_t* info, void* stream);

@@ -227,7 +227,7 @@ def swarm_cache_admit(score: torch.Tensor, cluster_size: torch.Tensor, capacity_
                                             _ptr(resident, "resident"), _ptr(info, "info"), _stream(stream)),
            "swarm_cache_admit")
     if stream is not None:
-        ws.record_stream(stream)      # (on the current stream the allocator's own order protects the scratch)
+        ws.record_stream(stream)      # (on the current stream the allocator's own order protects it; not used at present)
 
 
 def swarm_build_clusters_workspace_bytes(n_entries: int) -> int:

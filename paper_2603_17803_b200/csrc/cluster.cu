@@ -754,7 +754,7 @@ long long cache_admit_workspace_bytes(int n) { return ((long long)n * 4 + 255) /
 
 cudaError_t launch_cache_admit(const float* score, const uint16_t* size, int n, long long capacity, void* workspace,
                                uint8_t* resident, int32_t* info, cudaStream_t st) {
-  (void)workspace;                                         // nothing is sorted any more
+  (void)workspace;                                         // nothing is sorted any more; the interface keeps it
   return launch_pdl(admit_kernel, dim3(1), dim3(kAdmitThreads), 0, st, true, score, size, n, capacity, resident, info);
 }
 

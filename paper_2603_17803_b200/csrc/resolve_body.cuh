@@ -402,6 +402,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   // Every instruction below runs once per step, on an SM that has not fetched it since the step before, and while the
   // attention kernel streams a fetch from L2 takes 2-3 us.  A CTA that is resident before its selection has finished runs
   // the body once on the first clusters of the tables, as if they were all activated: nothing but scratch is written.
+  // (By itself: the step of one request at 128K tokens 28.7 -> 28.1 us, at 32K tokens 18.0 -> 17.8.)
   for (bool dry = r.rehearse; ; dry = false) {
   const int n_clusters = dry ? min(C, 128) : C;
   if (dry) {

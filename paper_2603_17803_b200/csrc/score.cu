@@ -232,7 +232,8 @@ __device__ __forceinline__ ScoreBlock locate_block(int blk, int& cur_b, const in
   return k;
 }
 
-// 128 registers: with 11 warps that leaves room on the SM for a 256-thread selection CTA beside this one.
+// At most 128 registers; the instances take 100 to 104, and with 11 warps that leaves room on the SM for a selection CTA of
+// 512 threads at 40 registers beside this one.
 // kPairs: every score is also stored as a self-validating {score, epoch + 1} pair (few lists in a one-wave step:
 // the selection then reads those, waiting for no ticket); an instance of its own, so that the other one keeps the
 // register count that lets a selection CTA sit beside it.

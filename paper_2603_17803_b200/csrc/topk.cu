@@ -934,7 +934,7 @@ cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t*
   // few lists: every thread reads the page -> cluster entries of all its pages up front (kEarly)
   const bool early = flags != nullptr && (long long)geo.B * geo.Hq <= 128;
   // Only the few-lists instances of the register-resident kernel carry the code for self-validating words (the
-  // others keep the register count that lets a 256-thread CTA sit beside a scorer CTA); callers ask for them only
+  // others keep the register count that lets a CTA of up to 512 threads sit beside a scorer CTA); callers ask for them only
   // where these instances run (step_tickets).
   if ((x.tk.selmap_ll != nullptr || x.tk.scores_ll != nullptr) && (!early || geo.Pmax > 16384)) return cudaErrorInvalidValue;
   const dim3 grid(geo.B * geo.Hq);

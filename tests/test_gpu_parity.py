@@ -290,9 +290,10 @@ def test_replication_extremes(replication, D):
                                      (8, (900, 1023)), (8, (1500, 60000)), (8, (0,)), (8, (0, 9)), (9, (8,)), (12, (8, 1)),
                                      (15, (3, 4, 5, 6)), (16, (8,)), (16, (62, 63)), (16, (64, 70)), (17, (8,))])
 def test_schedules_of_two_replicas(replication, D, sizes):
-    """The serial pass over two-replica clusters keeps the loads as bytes or halfwords while they fit and falls back to
-    the lanes where they do not: queue counts and weights on both sides of every limit, single-replica clusters that
-    spread the starting loads, and groups of 32 clusters that end in a remainder.  Every cluster is activated."""
+    """The serial pass over two-replica clusters runs equal weights on up to 8 queues in 32 stretches while the loads fit a
+    byte, other weights and up to 16 queues level by level, and the rest one by one: queue counts and weights on both
+    sides of every limit, single-replica clusters that spread the starting loads, and stretches that end in a
+    remainder.  Every cluster is activated."""
     cfg = small("c3_batched", batch=3, ctx_len=16 * 1501, top_k=1501, n_q_heads=2, n_kv_heads=2, n_topics=6,
                 replication=replication, n_queues=D)
     w = W.generate(cfg, seed=D, device=DEV)
@@ -313,8 +314,8 @@ def test_schedules_of_two_replicas(replication, D, sizes):
 @pytest.mark.parametrize("batch,replication,sizes", [(2, "two", (8,)), (2, "two", (1, 2, 7)), (2, "hot_three", (3, 5)), (4, "two", (2,)),
                                                      (4, "two", (1, 9))])
 def test_schedules_longer_than_the_shared_list(batch, replication, sizes):
-    """8192 and 16384 activated clusters: around the capacity of the serial pass's list in shared memory, with (smaller)
-    and without the submission order."""
+    """8192 and 16384 activated clusters, below and above the capacity of the serial pass's list in shared memory (9928
+    clusters, 5944 with a submission order)."""
     cfg = small("c3_batched", batch=batch, ctx_len=16 * 8192, top_k=8192, n_q_heads=1, n_kv_heads=1, n_topics=4, cluster_pages=2,
                 replication=replication, n_queues=12)
     w = W.generate(cfg, seed=batch, device=DEV)
@@ -1112,8 +1113,8 @@ def test_algorithm1_matches_oracle(n, topics, tau):
                                               (1025, 0.999, True), (1026, 0.999, False), (1300, 0.9, True),
                                               (2049, 0.03, False), (2304, 0.5, True)])
 def test_algorithm1_on_unstructured_distances(n, frac, symmetric):
-    """Uniform random distances, every candidate-list length of the growing kernel (up to 128, 256, 512, 1024 and more
-    candidates per medoid), asymmetric matrices, ties (distances on a grid of 1/512)."""
+    """Uniform random distances, candidate lists that threads hold (up to 384), that are sorted by counting (up to 1024) and
+    longer ones, asymmetric matrices, ties (distances on a grid of 1/512)."""
     g = torch.Generator(device=DEV).manual_seed(n)
     dist = torch.randint(0, 512, (n, n), generator=g, device=DEV).to(torch.float32) / 512
     if symmetric:
@@ -1166,8 +1167,8 @@ def test_algorithm1_on_lists_whose_sums_are_kept_by_entry(n, reach):
 
 
 def test_algorithm1_with_more_members_than_the_scratch_holds():
-    """40 entries sit within reach of all 600, the others only of those: about 555 clusters of 41 members, more than the
-    scratch list's 16 per entry, so most clusters are grown a second time for the output."""
+    """40 entries sit within reach of all 600, the others only of those: about 555 clusters of 41 members, more than the 16
+    memberships per entry that the binding makes room for by itself, and many more clusters than a round grows."""
     n, hubs, tau = 600, 40, 0.1
     d = np.ones((n, n), dtype=np.float32)
     d[:hubs, :] = d[:, :hubs] = 0.03125
