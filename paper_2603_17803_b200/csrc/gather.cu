@@ -83,17 +83,26 @@ gather_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int32_t*
 // each over 8 coordinates; the halves are merged with one shuffle and lanes 0-15 write the 256-byte
 // minima row, lanes 16-31 the maxima row.
 // Bound by HBM.  The warps of a grid that fills the device once walk the pool in its own order (page, then head), so
-// that neighbours read neighbouring blocks, and every warp has eight 512-byte loads in flight.  (A grid of one CTA per
-// eight pages of the longest request, head and request left half of the CTAs of a ragged batch empty and took the loads one
-// after the other: the index build of 16 requests of up to 60000 tokens took 214 us, now 193; these summaries 181 us of
-// them, 5.85 TB/s, 0.89 of the measured copy bandwidth.)  Four CTAs per SM cap a thread at 64 registers: 16 bytes spill.
-__device__ __forceinline__ void min_max8(const uint4& v, float (&lo)[8], float (&hi)[8]) {
+// that neighbours read neighbouring blocks, and every warp has eight 512-byte loads in flight.  The minima and maxima are
+// taken on pairs of bf16: a block costs a warp about 100 instructions instead of 250, and no registers spill at four CTAs per
+// SM.  Summaries and medoid rows of 16 requests of up to 60000 tokens (1061 and 31 MB): 191 us with the values widened to fp32,
+// 182 in pairs (the summaries alone at 0.95 of the measured copy bandwidth); five and six CTAs per SM spill, 194 and 258.
+__device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ void min_max8(const uint4& v, uint32_t (&lo)[4], uint32_t (&hi)[4]) {
   const uint32_t words[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const float a = bf16_lo(words[e]), d2 = bf16_hi(words[e]);
-    lo[2 * e] = fminf(lo[2 * e], a);         hi[2 * e] = fmaxf(hi[2 * e], a);
-    lo[2 * e + 1] = fminf(lo[2 * e + 1], d2); hi[2 * e + 1] = fmaxf(hi[2 * e + 1], d2);
+    lo[e] = min2(lo[e], words[e]);
+    hi[e] = max2(hi[e], words[e]);
   }
 }
 
@@ -135,9 +144,9 @@ summaries_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int64
     if (len < 1 || P > owned || p >= P) continue;
     const int valid = p == P - 1 ? len - S * (P - 1) : S;
     const uint16_t* K = kv_pool + ((page * geo.Hkv + kvh) * 2) * (long long)S * kHeadDim + half * kHeadDim + c * 8;
-    float lo[8], hi[8];
+    uint32_t lo[4], hi[4];                                   // pairs of bf16
 #pragma unroll
-    for (int e = 0; e < 8; ++e) { lo[e] = INFINITY; hi[e] = -INFINITY; }
+    for (int e = 0; e < 4; ++e) { lo[e] = 0x7F807F80u; hi[e] = 0xFF80FF80u; }   // +inf, -inf
     for (int t0 = 0; t0 < valid; t0 += 16) {
       uint4 v[8];
       if (t0 + 16 <= valid) {
@@ -150,19 +159,13 @@ summaries_kernel(Geometry geo, const uint16_t* __restrict__ kv_pool, const int64
 #pragma unroll
       for (int i = 0; i < 8; ++i) min_max8(v[i], lo, hi);
     }
-    uint32_t packed[4];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      lo[e] = fminf(lo[e], __shfl_xor_sync(0xFFFFFFFFu, lo[e], 16));
-      hi[e] = fmaxf(hi[e], __shfl_xor_sync(0xFFFFFFFFu, hi[e], 16));
-    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float a = half ? hi[2 * e] : lo[2 * e], d2 = half ? hi[2 * e + 1] : lo[2 * e + 1];
-      packed[e] = (__float_as_uint(a) >> 16) | (__float_as_uint(d2) & 0xFFFF0000u);   // values are bf16 already
+      lo[e] = min2(lo[e], __shfl_xor_sync(0xFFFFFFFFu, lo[e], 16));
+      hi[e] = max2(hi[e], __shfl_xor_sync(0xFFFFFFFFu, hi[e], 16));
     }
     uint4* dst = reinterpret_cast<uint4*>(ksum + ((page * geo.Hkv + kvh) * 2 + half) * (long long)kHeadDim + c * 8);
-    *dst = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+    *dst = half ? make_uint4(hi[0], hi[1], hi[2], hi[3]) : make_uint4(lo[0], lo[1], lo[2], lo[3]);
   }
 }
 

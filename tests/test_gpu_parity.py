@@ -1560,3 +1560,32 @@ def test_head_sharded_step_on_one_device(name, world):
     for s in sess:
         s.close()
     full.close()
+
+
+@pytest.mark.parametrize("page,ctx_len", [(16, [16 * 37 + 1, 5, 16 * 3]), (32, [32 * 9 + 31, 1, 33])])
+def test_summaries_of_special_values(page, ctx_len):
+    """Minima and maxima are whole values: denormals are kept, -0 lies below +0, infinities count, NaN does not."""
+    cfg = W.scaled(W.CONFIGS["c5_skewed"], batch=len(ctx_len), ctx_range=(1, max(ctx_len)), page_size=page, top_k=2, n_topics=2)
+    w = W.generate(cfg, seed=5, device=DEV)
+    assert int((w.page_base[1:] - w.page_base[:-1]).min()) >= 1
+    lens = [min(n, int(w.page_base[b + 1] - w.page_base[b]) * page) for b, n in enumerate(ctx_len)]
+    w.ctx_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    values = np.array([0x0000, 0x8000, 0x0001, 0x8001, 0x007F, 0x807F, 0x3F80, 0xBF80, 0x7F7F, 0xFF7F, 0x7F80, 0xFF80, 0x7FC0, 0xFFC1], dtype=np.uint16)
+    bits = np.random.default_rng(7).choice(values, size=w.kv_pool.shape, p=[.3, .3] + [.4 / 12] * 12)
+    w.kv_pool.copy_(torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16))
+    sess = Session(w)
+    torch.cuda.synchronize()
+    got = sess.ksum.view(torch.int16).cpu().numpy().view(np.uint16)
+    key = np.where(bits & 0x8000, 0x7FFF - (bits & 0x7FFF).astype(np.int32), 0x8000 + bits.astype(np.int32))   # sign-magnitude order
+    nan = (bits & 0x7FFF) > 0x7F80
+    for b, n in enumerate(lens):
+        base = int(w.page_base[b])
+        for p in range(-(-n // page)):
+            tok = slice(0, min(page, n - p * page))
+            for part, empty, reduce in ((0, 0x7F80, np.argmin), (1, 0xFF80, np.argmax)):
+                k = np.where(nan[base + p, :, 0, tok], 1 << 20 if part == 0 else -1, key[base + p, :, 0, tok])
+                at = reduce(k, axis=1)
+                want = np.take_along_axis(bits[base + p, :, 0, tok], at[:, None], axis=1)[:, 0]
+                want = np.where(nan[base + p, :, 0, tok].all(axis=1), empty, want)
+                assert np.array_equal(got[base + p, :, part], want), (b, p, part)
+    sess.close()
