@@ -1589,3 +1589,35 @@ def test_summaries_of_special_values(page, ctx_len):
                 want = np.where(nan[base + p, :, 0, tok].all(axis=1), empty, want)
                 assert np.array_equal(got[base + p, :, part], want), (b, p, part)
     sess.close()
+
+
+@pytest.mark.parametrize("own_stream", [True, False])
+@pytest.mark.parametrize("name", ["c2_small", "c3_small", "c5_small"])
+def test_step_host_directly_behind_an_index_build(name, own_stream):
+    """The host step's scorer asks for its first summaries while the queries travel: still after whatever precedes the call in its
+    stream, here the summaries of a pool rewritten every turn (the recorded graph on a stream of its own; plain launches)."""
+    w = W.generate(CASES[name], seed=23, device=DEV)
+    pools = [w.kv_pool.clone(), w.kv_pool.flip(1)]          # (the KV heads in the other order)
+    q_host = w.q.cpu().pin_memory()
+    out_host = torch.empty((w.cfg.batch, w.cfg.n_q_heads, w.cfg.head_dim), dtype=torch.float32).pin_memory()
+    want = []
+    for pool in pools:
+        w.kv_pool.copy_(pool)
+        ref = Session(w)
+        torch.cuda.synchronize()
+        ref.step()
+        torch.cuda.synchronize()
+        want.append((ref.o.sel.clone(), ref.o.out.cpu()))
+        ref.close()
+    sess = Session(w)
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream() if own_stream else None
+    for turn in range(8):
+        with torch.cuda.stream(stream or torch.cuda.current_stream()):
+            w.kv_pool.copy_(pools[turn % 2])
+            B.swarm_build_summaries(sess.ctx, sess.inputs, sess.ksum)
+            sess.step_host(q_host, out_host, stream=stream)
+        assert torch.equal(out_host, want[turn % 2][1]), turn
+        torch.cuda.synchronize()
+        assert sess.status() == 0 and torch.equal(sess.o.sel, want[turn % 2][0])
+    sess.close()
