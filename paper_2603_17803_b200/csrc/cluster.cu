@@ -464,38 +464,46 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
   if (tid == 0) sh.failed = 0;
   if (me == 0 && tid == 0) a.ptr[0] = 0;
 
-  // ---- the order of the walk: a warp counts the entries in front of kPer entries, from keys in shared memory ----
-  // (density << 15 | 32767 - entry: in front means a larger key, one compare)
-  constexpr int kPer = 5;                                  // (8192 entries on 148 SMs: one turn)
-  int* s_key = reinterpret_cast<int*>(dyn);
-  const int n4 = (n + 3) & ~3;
+  // ---- the order of the walk: places by counting ----
+  // Every CTA counts the entries of each density, those in front of its own stretch of entries apart (two counts to a word), and
+  // adds up the denser ones; an entry's place is what is denser, what is as dense in front of the stretch, and what is as dense
+  // in front of it inside the stretch.  Bound by barriers and the atomics on a few popular counts.  (8192 entries: 7 us; comparing every
+  // entry with every other, 12 us.  The whole call 299.7 -> 292.7, 3911 entries 211 -> 205.)
+  {
+    uint32_t* hist = reinterpret_cast<uint32_t*>(dyn);     // [n] by n - 1 - density: all entries << 16 | those in front of the stretch
+    const int stretch = (n + G - 1) / G, first = min(n, me * stretch), last = min(n, first + stretch);
+    for (int i = tid; i < n; i += kRoundThreads) hist[i] = 0u;
+    __syncthreads();
 #pragma unroll 6
-  for (int i = 4 * tid; i < n4; i += 4 * kRoundThreads) {
-    int r[4] = {-1, -1, -1, -1};
-    if (i + 4 <= n) {
-      const int4 v = *reinterpret_cast<const int4*>(a.rho + i);
-      r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
-    } else {
-      for (int j = 0; i + j < n; ++j) r[j] = a.rho[i + j];
+    for (int i = 4 * tid; i < n; i += 4 * kRoundThreads) {
+      int r[4];
+      if (i + 4 <= n) {
+        const int4 v = *reinterpret_cast<const int4*>(a.rho + i);
+        r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
+      } else {
+        for (int j = 0; j < 4; ++j) r[j] = i + j < n ? a.rho[i + j] : -1;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (r[j] >= 0) atomicAdd(&hist[n - 1 - r[j]], i + j < first ? 0x10001u : 0x10000u);
     }
-    *reinterpret_cast<int4*>(s_key + i) = make_int4(r[0] << 15 | (32767 - i), r[1] < 0 ? -1 : r[1] << 15 | (32766 - i),
-                                                    r[2] < 0 ? -1 : r[2] << 15 | (32765 - i), r[3] < 0 ? -1 : r[3] << 15 | (32764 - i));
-  }
-  __syncthreads();
-  for (int e0 = (me * kRoundWarps + warp) * kPer; e0 < n; e0 += G * kRoundWarps * kPer) {
-    int mine[kPer], at[kPer] = {};
-#pragma unroll
-    for (int u = 0; u < kPer; ++u) mine[u] = e0 + u < n ? s_key[e0 + u] : 0;
-#pragma unroll 2
-    for (int o = lane * 4; o < n4; o += 128) {
-      const int4 r = *reinterpret_cast<const int4*>(s_key + o);
-#pragma unroll
-      for (int u = 0; u < kPer; ++u) at[u] += (r.x > mine[u]) + (r.y > mine[u]) + (r.z > mine[u]) + (r.w > mine[u]);
+    __syncthreads();
+    const int per = (n + kRoundThreads - 1) / kRoundThreads, b0 = min(n, tid * per), b1 = min(n, b0 + per);
+    int sum = 0, total;
+    for (int i = b0; i < b1; ++i) sum += (int)(hist[i] >> 16);
+    int run = block_prefix(sh, sum, total);
+    for (int i = b0; i < b1; ++i) {
+      const uint32_t h = hist[i];
+      hist[i] = (uint32_t)run + (h & 0xFFFFu);
+      run += (int)(h >> 16);
     }
-#pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int p = __reduce_add_sync(0xFFFFFFFFu, at[u]);
-      if (lane == 0 && e0 + u < n) { a.queue[p] = e0 + u; a.place[e0 + u] = p; }
+    __syncthreads();
+    for (int e = first + tid; e < last; e += kRoundThreads) {
+      const int r = a.rho[e];
+      int p = (int)hist[n - 1 - r];
+      for (int j = first; j < e; ++j) p += a.rho[j] == r;
+      a.queue[p] = e;
+      a.place[e] = p;
     }
   }
   unsigned nth = 0;

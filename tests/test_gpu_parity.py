@@ -1621,3 +1621,20 @@ def test_step_host_directly_behind_an_index_build(name, own_stream):
         torch.cuda.synchronize()
         assert sess.status() == 0 and torch.equal(sess.o.sel, want[turn % 2][0])
     sess.close()
+
+
+@pytest.mark.parametrize("n", [3, 146, 147, 148, 149, 297, 1483])
+def test_algorithm1_order_of_equal_densities(n):
+    """The walk starts with the densest entries, ties with the lower index first: a few densities shared by many entries, entries
+    around multiples of the CTAs that count them (each its own stretch)."""
+    rng = np.random.default_rng(n)
+    kind = rng.integers(0, 5, size=n)                     # five blocks of near entries, far from the others
+    dist = np.where(kind[:, None] == kind[None, :], 0.125, 0.875).astype(np.float32)
+    np.fill_diagonal(dist, 0.0)
+    dist[rng.integers(0, n, size=n // 3), rng.integers(0, n, size=n // 3)] = 0.375   # some rows of other densities
+    np.fill_diagonal(dist, 0.0)
+    for tau in (0.0625, 0.25, 0.5):                       # nobody near, the blocks, the blocks and the odd ones
+        rho, ptr_ref, members_ref, medoid_ref = oracle.build_clusters(dist, tau, members_cap=64 * n)
+        density, ptr, members, medoid = B.swarm_build_clusters(torch.from_numpy(dist).to(DEV), tau, members_cap=64 * n)
+        assert np.array_equal(density.cpu().numpy(), rho) and np.array_equal(medoid.cpu().numpy(), medoid_ref)
+        assert np.array_equal(ptr.cpu().numpy(), ptr_ref) and np.array_equal(members.cpu().numpy(), members_ref)
