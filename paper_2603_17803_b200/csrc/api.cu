@@ -525,7 +525,9 @@ int32_t swarm_resolve_clusters(swarm_ctx* ctx, const swarm_inputs* in, const int
   if (!resolve_inputs_ok(in) || bad(sel) || bad(n_sel) || bad(uniq) || bad(queue_of) || bad(n_uniq) ||
       bad(queue_load))
     return SWARM_ERR_INVALID_ARG;
-  SWARM_TRY(launch_resolve(step_resolve_args(ctx, in, sel, n_sel, uniq, queue_of, n_uniq, queue_load), static_cast<cudaStream_t>(stream), true));
+  ResolveArgs rs = step_resolve_args(ctx, in, sel, n_sel, uniq, queue_of, n_uniq, queue_load);
+  rs.rehearse = true;
+  SWARM_TRY(launch_resolve(rs, static_cast<cudaStream_t>(stream), true));
   return SWARM_OK;
 }
 
@@ -708,7 +710,7 @@ int32_t step_impl(swarm_ctx* ctx, const swarm_inputs* in, const swarm_outputs* o
   // serial pass is the longest item of the step).
   a.n_splits = pick_splits(ctx, true, /*fused=*/true);
   a.n_more = pick_more(ctx, true, a.n_splits, /*fused=*/true);
-  rs.rehearse = links.tk.selmap_ll != nullptr;
+  rs.rehearse = links.tk.selmap_ll != nullptr || rs.has_cache;   // where the resolution ends the step (figures: resolve_body)
   SWARM_TRY(launch_attention(ctx->geo, a, status, st, /*overlap=*/true, &rs));
   return SWARM_OK;
 }

@@ -351,12 +351,13 @@ __host__ __device__ constexpr int serial_words(bool submit) {
 static_assert(serial_words(false) * 4 <= (int)kResolveSmemBytes && serial_words(true) * 4 <= (int)kResolveSmemBytes,
               "the lists and their blanks fit behind the tables");
 
-// `cta` of `n_ctas` CTAs of kThreads threads run the body with kResolveSmemBytes of dynamic shared memory.
-template <bool kCached>
+// `cta` of `n_ctas` CTAs of kThreads threads run the body with kResolveSmemBytes of dynamic shared memory.  kAlone: in a kernel of
+// its own, which may be given a selection to mark (inside the attention kernel that code would only be more to fetch).
+template <bool kCached, bool kAlone>
 __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int n_ctas) {
   const Geometry& geo = r.geo;
   const swarm_cache& cache = r.cache;
-  const int32_t* __restrict__ sel = r.sel;
+  const int32_t* __restrict__ sel = kAlone ? r.sel : nullptr;
   const int32_t* __restrict__ n_sel = r.n_sel;
   const int64_t* __restrict__ page_base = r.page_base;
   const int32_t* __restrict__ page2cluster = r.page2cluster;
@@ -385,27 +386,43 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   __shared__ unsigned s_classes, s_wmin, s_wmax;         // of the serial pass: replica classes, smallest and largest weight
   __shared__ unsigned s_item_m[32], s_item_w[32];
   __shared__ bool s_last;
+  constexpr int kDryClusters = 128;
+  __shared__ struct { int32_t uniq[kDryClusters], freq[kDryClusters]; float score[kDryClusters]; uint8_t queue_of[kDryClusters]; } s_dry;
   __shared__ int s_hits;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (sel != nullptr) pdl_wait();                        // (on its own, any input may come from the previous kernel)
-  pdl_launch_dependents();                               // the next kernel in the stream may be scheduled while this one runs
-  const long long c_all = cluster_base[geo.B];           // inside a step an input table: not written by the previous kernel
-  const int C = (int)min((long long)geo.Cmax, c_all);
+  // On its own any input may come from the previous kernel: nothing is read before the wait.
+  long long c_all = sel == nullptr ? cluster_base[geo.B] : 0;   // inside a step an input table: not written by the previous kernel
+  int C = (int)min((long long)geo.Cmax, c_all);
   unsigned err = 0u, step_no = 0u;
   // Every instruction below runs once per step, on an SM that has not fetched it since the step before, and while the
   // attention kernel streams a fetch from L2 takes 2-3 us.  A CTA that is resident before its selection has finished runs
-  // the body once on the first clusters of the tables, as if they were all activated: nothing but scratch is written.
-  // (By itself: the step of one request at 128K tokens 28.7 -> 28.1 us, at 32K tokens 18.0 -> 17.8.)
+  // the body once on the first clusters of the tables, as if they were all activated, or in a kernel of its own on made-up ones:
+  // nothing but shared memory is written, and in a kernel of its own nothing is read.  A rehearsal takes about 10 us.  It pays where
+  // the CTA waits as long anyway and the resolution ends the step: one request at 128K tokens 28.7 -> 28.1 us, at 32K tokens 18.0 -> 17.8;
+  // with cache state, together with the stores of four words below, 16 ragged requests of up to 128K tokens 130.3 -> 125.1, 37 of 55K
+  // 190.5 -> 178.7, 12 of 33K 45.8 -> 43.0; four separate calls 115.6 -> 115.1.  Steps of several waves without cache state: 36.6 -> 36.9 (the
+  // attention ends them); the medoid step, which has 4 us to wait: 10 us longer.
   for (bool dry = r.rehearse; ; dry = false) {
-  const int n_clusters = dry ? min(C, 128) : C;
+  const bool made_up = dry && sel != nullptr;
+  int n_clusters = made_up ? kDryClusters : min(C, kDryClusters);
+  int32_t* freq_out = cache.freq;
+  float* score_out = cache.score;
   if (dry) {
-    uniq = reinterpret_cast<int32_t*>(items);
-    queue_of = reinterpret_cast<uint8_t*>(uniq + n_clusters);   // (16 bytes of scratch per cluster)
+    uniq = s_dry.uniq;
+    queue_of = s_dry.queue_of;
+    freq_out = s_dry.freq;
+    score_out = s_dry.score;
   } else {
   uniq = r.uniq;
   queue_of = r.queue_of;
   pdl_wait();                                            // the flags / the selection come from the previous kernel
+  pdl_launch_dependents();                               // the next kernel in the stream may be scheduled while this one runs
+  if (sel != nullptr) {
+    c_all = __ldcg(cluster_base + geo.B);
+    C = (int)min((long long)geo.Cmax, c_all);
+  }
+  n_clusters = C;
   err = (c_all > geo.Cmax) ? SWARM_DEV_BAD_CLUSTER : 0u;
   // Overlapped tail: nothing after this kernel in the step waits for it, so it runs beside the next step's
   // scoring and selection.  That selection marks the other one of two flag arrays (the selection kernel counts
@@ -492,13 +509,14 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   const bool unit = (geo.flags & SWARM_UNIT_LOAD) != 0;
   // vector loads of the cache state need its arrays aligned like the library's own tables
   const bool cache_vec = kCached && (reinterpret_cast<uintptr_t>(cache.resident) & 3u) == 0 &&
-                         (reinterpret_cast<uintptr_t>(cache.freq) & 15u) == 0;
-  const bool need_sz = !unit || (kCached && cache.score != nullptr);   // unit loads need no size table, Eq. 6 does
+                         (reinterpret_cast<uintptr_t>(cache.freq) & 15u) == 0 && (reinterpret_cast<uintptr_t>(cache.score) & 15u) == 0;
+  const bool need_score = kCached && cache.score != nullptr;
+  const bool need_sz = !unit || need_score;   // unit loads need no size table, Eq. 6 does
   const int rows = (n_clusters + kRow - 1) / kRow;
   const uint32_t ring = shared_addr(s_pass);
   auto request = [&](int row) {                            // (entries beyond the tables arrive as zeros)
     const int c = row * kRow + 4 * tid, have = min(4, n_clusters - c);
-    if (row < rows && have > 0) {
+    if (row < rows && have > 0 && !made_up) {
       const uint32_t at = ring + (row % kDepth) * kRowBytes;
       copy_async<16>(at + 16 * tid, replica_mask + c, 4 * have);
       if (need_sz) copy_async<8>(at + kThreads * 16 + 8 * tid, cluster_size + c, 2 * have);
@@ -511,6 +529,12 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   for (int row = 0; row < kDepth; ++row) request(row);
+  if (made_up && tid < kDryClusters / 4) {                 // clusters of two replicas and two weights
+    uint32_t* at = s_pass;
+    *reinterpret_cast<uint4*>(at + 4 * tid) = make_uint4(3u, 3u, 3u, 3u);
+    at[kThreads * 4 + 2 * tid] = at[kThreads * 4 + 2 * tid + 1] = 0x00070008u;
+    if (kCached) at[kThreads * 11 + tid] = 0u;
+  }
   int n = 0, n_serial = 0;                                 // clusters to fetch so far, and those for the serial pass
   const bool spill = n_clusters > cap;                     // the list may outgrow shared memory: it is written to global memory as well
   // submission order (optional): (replica class, queue) keys, kept in shared memory so that the ordering pass at the
@@ -518,6 +542,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   uint32_t* order_key = s_slot + cap;
   const bool order_keys = r.submit_order != nullptr;
   unsigned classes = 0u, wmin = 0xFFFFFFFFu, wmax = 0u;
+  int hits = 0;                                            // activated clusters that are resident
   for (int row = 0; row < rows; ++row) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kDepth - 1) : "memory");
     __syncthreads();
@@ -551,19 +576,30 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
         }
       }
     }
-    if (kCached && !dry) {
-      // cache bookkeeping of Sec. 5.2 for every cluster, activated or not
+    if (kCached && c0 < n_clusters) {
+      // cache bookkeeping of Sec. 5.2 for every cluster, activated or not; four clusters' words in one store where the
+      // arrays allow it (before: eight stores of a word per thread and row)
+      float score[4];
+      bool moved = false;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (c0 + j < n_clusters) {
-          const bool on = ((f >> (8 * j)) & 0xFFu) != 0u, is_res = ((res >> (8 * j)) & 0xFFu) != 0u;
-          if (on) ++fr[j]; else if (is_res) --fr[j];
-          if (on || is_res) cache.freq[c0 + j] = fr[j];
-          if (cache.score != nullptr) {
-            const float size_f = (float)((sz[j >> 1] >> (16 * (j & 1))) & 0xFFFFu);
-            cache.score[c0 + j] = (float)fr[j] * (cache.t_base + size_f * cache.t_transfer) / size_f;
+        const bool on = ((f >> (8 * j)) & 0xFFu) != 0u, is_res = ((res >> (8 * j)) & 0xFFu) != 0u;
+        fr[j] += on ? 1 : is_res ? -1 : 0;
+        moved = moved || on || is_res;
+        hits += on && is_res ? 1 : 0;
+        const float size_f = (float)((sz[j >> 1] >> (16 * (j & 1))) & 0xFFFFu);
+        score[j] = need_score ? (float)fr[j] * (cache.t_base + size_f * cache.t_transfer) / size_f : 0.f;
+      }
+      if (cache_vec && !dry && c0 + 4 <= n_clusters) {
+        if (moved) *reinterpret_cast<int4*>(freq_out + c0) = make_int4(fr[0], fr[1], fr[2], fr[3]);
+        if (need_score) *reinterpret_cast<float4*>(score_out + c0) = make_float4(score[0], score[1], score[2], score[3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (c0 + j < n_clusters) {
+            if (moved) freq_out[c0 + j] = fr[j];
+            if (need_score) score_out[c0 + j] = score[j];
           }
-          if (on && is_res) atomicAdd(&s_hits, 1);
         }
       }
     }
@@ -649,6 +685,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     atomicMin(&s_wmin, wmin);
     atomicMax(&s_wmax, wmax);
   }
+  if (kCached && hits) atomicAdd(&s_hits, hits);
   if (err && !dry) atomicOr(status, err);
   err = 0u;
   if (staged && tid < kBlanks) s_mask[n_serial + tid] = s_wgt[n_serial + tid] = 0u;

@@ -222,7 +222,7 @@ struct ResolveArgs {
   // StepTickets, and the distance between the two flag arrays that alternate steps mark.  Null / 0 otherwise.
   unsigned* tail_ctl = nullptr;
   long long flags_alt = 0;
-  bool rehearse = false;   // one CTA inside a step that is one chain: run the body once on made-up flags while the selection runs
+  bool rehearse = false;   // run the body once for nothing while the selection runs, so that its instructions are fetched (see resolve_body)
 };
 ResolveArgs make_resolve_args(const Geometry& geo, const int32_t* sel, const int32_t* n_sel, const int64_t* page_base,
                               const int32_t* page2cluster, const int64_t* cluster_base, const uint32_t* replica_mask,

@@ -1638,3 +1638,65 @@ def test_algorithm1_order_of_equal_densities(n):
         density, ptr, members, medoid = B.swarm_build_clusters(torch.from_numpy(dist).to(DEV), tau, members_cap=64 * n)
         assert np.array_equal(density.cpu().numpy(), rho) and np.array_equal(medoid.cpu().numpy(), medoid_ref)
         assert np.array_equal(ptr.cpu().numpy(), ptr_ref) and np.array_equal(members.cpu().numpy(), members_ref)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 4])
+@pytest.mark.parametrize("pages", [5, 16 * 8, 16 * 128 + 3, 2 * 1024 + 1])
+def test_cache_bookkeeping_at_row_ends_and_unaligned_arrays(pages, shift):
+    """Counters and scores of four clusters at a time where the arrays allow it, one by one otherwise: cluster counts around
+    multiples of 4 and of a row of 1024, arrays that start off a 16-byte boundary.  A cluster per page, a third of them selected."""
+    cfg = small("c1_tiny", ctx_len=16 * pages, top_k=max(1, pages // 3), n_q_heads=1, n_kv_heads=1, cluster_pages=1, n_queues=6)
+    w = W.generate(cfg, seed=pages, device=DEV)
+    C = w.n_clusters
+    rng = np.random.default_rng(pages + shift)
+    w.cluster_size.copy_(torch.from_numpy(rng.integers(1, 12, size=C).astype(np.uint16).view(np.int16)))
+    resident0, freq0 = (rng.random(C) < 0.4).astype(np.uint8), rng.integers(-2, 9, size=C).astype(np.int32)
+    guard = 77
+    resident, freq = torch.full((C + 32,), guard, dtype=torch.uint8, device=DEV), torch.full((C + 32,), guard, dtype=torch.int32, device=DEV)
+    score = torch.full((C + 32,), float(guard), device=DEV)
+    resident[shift:shift + C], freq[shift:shift + C] = torch.from_numpy(resident0).to(DEV), torch.from_numpy(freq0).to(DEV)
+    n_hit = torch.zeros(4, dtype=torch.int32, device=DEV)
+    sess = Session(w)
+    B.swarm_set_cache(sess.ctx, resident=resident[shift:], freq=freq[shift:], score=score[shift:], n_hit=n_hit, t_base=80.0, t_transfer=2.5)
+    tabs = parity.host_tables(w)
+    for turn in range(2):
+        if turn == 0:
+            sess.step()
+        else:
+            sess.resolve()                                # the separate call takes the same path
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        uniq, qof, load, hits, freq0, score0 = oracle.resolve_cached(
+            sess.o.sel.cpu().numpy(), sess.o.n_sel.cpu().numpy(), tabs["page_base"], tabs["page2cluster"], tabs["cluster_base"],
+            tabs["replica_mask"], tabs["cluster_size"], resident0, freq0, cfg.n_queues, 80.0, 2.5)
+        n = int(sess.o.n_uniq[0])
+        assert n == len(uniq) and int(n_hit[0]) == hits
+        assert np.array_equal(sess.o.uniq[:n].cpu().numpy(), uniq) and np.array_equal(sess.o.queue_of[:n].cpu().numpy(), qof)
+        assert np.array_equal(freq[shift:shift + C].cpu().numpy(), freq0)
+        assert np.allclose(score[shift:shift + C].cpu().numpy(), score0, rtol=1e-6, atol=1e-6)
+        for t in (freq, score):                           # nothing beside the arrays is touched
+            assert bool((t[:shift] == guard).all()) and bool((t[shift + C:] == guard).all())
+    B.swarm_set_cache(sess.ctx)
+    sess.close()
+
+
+def test_resolution_directly_behind_an_update_of_its_tables():
+    """The separate call runs its code once on made-up clusters while the kernel before it is still running, and reads none of its
+    tables until that has finished."""
+    w = W.generate(CASES["c3_small"], seed=29, device=DEV)
+    sess = Session(w)
+    sess.step()
+    torch.cuda.synchronize()
+    big = torch.empty(64 << 20, device=DEV)
+    masks, sizes = w.cluster_replica_mask.clone(), w.cluster_size.clone()
+    for turn in range(4):
+        big.fill_(float(turn))                            # (a while of work in front)
+        w.cluster_size.copy_(sizes + turn)
+        w.cluster_replica_mask.mul_(0).add_(masks.roll(turn))
+        sess.resolve()
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        o = sess.o
+        parity.check_resolve(w, parity.host_tables(w), o.sel.cpu().numpy(), o.n_sel.cpu().numpy(), o.uniq.cpu().numpy(), o.queue_of.cpu().numpy(),
+                             o.n_uniq.cpu().numpy()[0], o.queue_load.cpu().numpy())
+    sess.close()
