@@ -833,13 +833,15 @@ int32_t swarm_step_medoid(swarm_ctx* ctx, const swarm_inputs* in, const swarm_me
   links.req_base = in->cluster_base;
   SWARM_TRY(launch_page_score(gc, static_cast<const uint16_t*>(in->q), static_cast<const uint16_t*>(idx->medoid_ksum),
                               in->cluster_base, len_c, sc, status, st, links.tk.ready, reserved_sms(ctx, gc, false)));
-  SWARM_TRY(launch_topk(gc, sc, len_c, o->sel, o->n_sel, status, st, true, links));
   // selected clusters -> page bitmaps per head (for attention) and cluster flags (for the resolve kernel)
-  SWARM_TRY(launch_expand_clusters(ctx->geo, idx->top_k_clusters, o->sel, o->n_sel, in->cluster_base,
-                                   idx->cluster_page_ptr, idx->cluster_pages, in->ctx_len,
-                                   ws_ptr<uint8_t>(ctx, ctx->lay.selmap), ws_ptr<uint8_t>(ctx, ctx->lay.flags), status, st,
-                                   true, idx->entry_replica_mask != nullptr ? in->page_base : nullptr,
-                                   idx->n_member_entries, in->page_base, in->page2cluster));
+  const ExpandArgs ex{in->cluster_base, idx->cluster_page_ptr, idx->cluster_pages, in->ctx_len, ws_ptr<uint8_t>(ctx, ctx->lay.selmap),
+                      ws_ptr<uint8_t>(ctx, ctx->lay.flags), idx->entry_replica_mask != nullptr ? in->page_base : nullptr,
+                      idx->n_member_entries, in->page_base, in->page2cluster, selmap_pitch_bytes(ctx->geo.Pmax), ctx->geo.S, ctx->geo.W,
+                      ctx->geo.Cmax};
+  const bool expands = select_expands(gc, ex.pitch);
+  SWARM_TRY(launch_topk(gc, sc, len_c, o->sel, o->n_sel, status, st, true, links, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+                        expands ? &ex : nullptr));
+  if (!expands) SWARM_TRY(launch_expand_clusters(ex, ctx->geo, idx->top_k_clusters, o->sel, o->n_sel, status, st, true));
   AttnArgs a = paged_args(ctx, in, o->out, o->lse);
   a.n_splits = pick_splits(ctx, true, /*fused=*/true);
   a.n_more = pick_more(ctx, true, a.n_splits, /*fused=*/true);

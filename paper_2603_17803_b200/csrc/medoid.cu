@@ -7,9 +7,10 @@
 // exactly like cluster_base.  What this file adds is the glue around them:
 //   medoid_rows_kernel     index build: copy the summary rows of the medoid pages into the index, and the pseudo
 //                          context lengths (clusters of the request x page size) for the page kernels
-//   expand_clusters_kernel selected clusters -> per-head bitmap of their member pages plus the local window (what
+//   expand_clusters_kernel (where the selection kernel does not do it itself, see medoid_expand.cuh)
+//                          selected clusters -> per-head bitmap of their member pages plus the local window (what
 //                          the attention kernel reads) and the cluster flags (what the resolve kernel reads)
-#include "swarm_internal.cuh"
+#include "medoid_expand.cuh"
 
 namespace swarm {
 namespace {
@@ -53,69 +54,21 @@ medoid_rows_kernel(Geometry geo, const uint16_t* __restrict__ ksum, const int64_
   }
 }
 
-// One CTA per (request, query head).  The head's bitmap row is assembled in shared memory (bit p % 8 of byte
-// p / 8, the layout the selection kernel writes) and stored whole, so rows need no clearing between steps.
+// One CTA per (request, query head), behind a selection kernel that does not expand its clusters itself.  The head's bitmap row is
+// assembled in shared memory (bit p % 8 of byte p / 8, the layout the selection kernel writes) and stored whole, so rows need no
+// clearing between steps.
 __global__ void __launch_bounds__(256)
-expand_clusters_kernel(Geometry geo, int k_c, int pitch, const int32_t* __restrict__ sel_c,
-                       const int32_t* __restrict__ n_sel_c, const int64_t* __restrict__ cluster_base,
-                       const int64_t* __restrict__ cluster_page_ptr, const int32_t* __restrict__ cluster_pages,
-                       const int32_t* __restrict__ ctx_len, uint8_t* __restrict__ selmap, uint8_t* __restrict__ flags,
-                       uint32_t* __restrict__ status, const int64_t* __restrict__ entry_base, long long n_member_entries,
-                       const int64_t* __restrict__ page_base, const int32_t* __restrict__ page2cluster) {
+expand_clusters_kernel(const ExpandArgs ex, int Hq, int k_c, const int32_t* __restrict__ sel_c, const int32_t* __restrict__ n_sel_c,
+                       uint32_t* __restrict__ status) {
   extern __shared__ uint32_t s_row[];
-  const int bh = blockIdx.x, b = bh / geo.Hq;
-  const int tid = threadIdx.x;
+  const int bh = blockIdx.x, b = bh / Hq;
   pdl_launch_dependents();                                  // the attention CTAs set themselves up meanwhile
-  const int P = pages_of(ctx_len[b], geo.S);               // inputs: read before the wait
-  const long long cb = cluster_base[b], cn = cluster_base[b + 1];
-  for (int i = tid; i < pitch / 4; i += blockDim.x) s_row[i] = 0u;
+  const ExpandRequest rq = expand_request(ex, b);          // inputs: read before the wait
+  for (int i = threadIdx.x; i < ex.pitch / 4; i += blockDim.x) s_row[i] = 0u;
   pdl_wait();                                               // the cluster selection comes from the previous kernel
   __syncthreads();
-  const int n = min(n_sel_c[bh], k_c);
-  unsigned err = 0u;
-  // Eight lanes per selected cluster, 32 clusters at a time: every cluster costs three dependent trips to memory
-  // (its id, its member range, its members), and with a warp per cluster four clusters of a warp paid them one after
-  // another (the kernel 7 of the step's 60 us; 32 clusters per head).
-  const int sub = tid & 7;
-  for (int j = tid >> 3; j < n; j += blockDim.x / 8) {
-    const int c = sel_c[(long long)bh * k_c + j];
-    if (c < 0 || c >= cn - cb || cb + c >= geo.Cmax) { err |= SWARM_DEV_BAD_CLUSTER; continue; }
-    const long long e0 = cluster_page_ptr[cb + c], e1 = cluster_page_ptr[cb + c + 1];
-    if (e0 < 0 || e1 < e0 || e1 > n_member_entries) { err |= SWARM_DEV_BAD_CLUSTER; continue; }   // corrupt member offsets
-    // what gets scheduled: the cluster as a whole, or (entry level) each of its pages on its own
-    if (sub == 0 && entry_base == nullptr) flags[cb + c] = 1;
-    for (long long e = e0 + sub; e < e1; e += 8) {
-      const int p = cluster_pages[e];
-      if (p < 0 || p >= P || p >= pitch * 8) {
-        err |= SWARM_DEV_BAD_PAGE;
-      } else {
-        atomicOr(&s_row[p >> 5], 1u << (p & 31));
-        if (entry_base != nullptr) {
-          const long long unit = entry_base[b] + p;
-          if (unit < geo.Cmax) flags[unit] = 1;
-          else err |= SWARM_DEV_BAD_CLUSTER;
-        }
-      }
-    }
-  }
-  // the local window (Sec. 4.2, Tier 1 (2)): the last W pages of the request join every head's set and are
-  // scheduled like the members of the selected clusters
-  for (int p = max(0, P - geo.W) + tid; p < P && p < pitch * 8; p += blockDim.x) {
-    atomicOr(&s_row[p >> 5], 1u << (p & 31));
-    if (entry_base != nullptr) {
-      const long long unit = entry_base[b] + p;
-      if (unit < geo.Cmax) flags[unit] = 1;
-      else err |= SWARM_DEV_BAD_CLUSTER;
-    } else {
-      const int c = page2cluster[page_base[b] + p];
-      if (c < 0 || c >= cn - cb || cb + c >= geo.Cmax) err |= SWARM_DEV_BAD_CLUSTER;
-      else flags[cb + c] = 1;
-    }
-  }
-  if (err) atomicOr(status, err);
-  __syncthreads();
-  uint32_t* row = reinterpret_cast<uint32_t*>(selmap + (long long)bh * pitch);
-  for (int i = tid; i < pitch / 4; i += blockDim.x) row[i] = s_row[i];
+  const int32_t* mine = sel_c + (long long)bh * k_c;
+  expand_clusters<8>(ex, rq, bh, b, min(n_sel_c[bh], k_c), [&](int j) { return mine[j]; }, s_row, status);
 }
 
 }  // namespace
@@ -131,15 +84,10 @@ cudaError_t launch_medoid_rows(const Geometry& geo, const uint16_t* ksum, const 
                     ksum, page_base, cluster_base, medoid_page, medoid_ksum, len, status);
 }
 
-cudaError_t launch_expand_clusters(const Geometry& geo, int k_c, const int32_t* sel_c, const int32_t* n_sel_c,
-                                   const int64_t* cluster_base, const int64_t* cluster_page_ptr,
-                                   const int32_t* cluster_pages, const int32_t* ctx_len, uint8_t* selmap, uint8_t* flags,
-                                   uint32_t* status, cudaStream_t st, bool overlap, const int64_t* entry_base,
-                                   long long n_member_entries, const int64_t* page_base, const int32_t* page2cluster) {
-  const int pitch = selmap_pitch_bytes(geo.Pmax);
-  return launch_pdl(expand_clusters_kernel, dim3((unsigned)(geo.B * geo.Hq)), dim3(256), (size_t)pitch, st, overlap, geo,
-                    k_c, pitch, sel_c, n_sel_c, cluster_base, cluster_page_ptr, cluster_pages, ctx_len, selmap, flags,
-                    status, entry_base, n_member_entries, page_base, page2cluster);
+cudaError_t launch_expand_clusters(const ExpandArgs& ex, const Geometry& geo, int k_c, const int32_t* sel_c, const int32_t* n_sel_c, uint32_t* status,
+                                   cudaStream_t st, bool overlap) {
+  return launch_pdl(expand_clusters_kernel, dim3((unsigned)(geo.B * geo.Hq)), dim3(256), (size_t)ex.pitch, st, overlap, ex, geo.Hq, k_c, sel_c,
+                    n_sel_c, status);
 }
 
 }  // namespace swarm

@@ -165,6 +165,20 @@ cudaError_t launch_page_score(const Geometry& geo, const uint16_t* q, const uint
                               const int64_t* page_base, const int32_t* ctx_len, float* scores, uint32_t* status,
                               cudaStream_t st, unsigned* ready = nullptr, int reserve_sms = 0, uint2* scores_ll = nullptr,
                               const unsigned* ctl = nullptr, bool index_early = false);
+// What the expansion of a head's selected clusters needs (see medoid_expand.cuh).
+struct ExpandArgs {
+  const int64_t* cluster_base;
+  const int64_t* cluster_page_ptr;
+  const int32_t* cluster_pages;
+  const int32_t* ctx_len;
+  uint8_t* selmap;               // rows of `pitch` bytes
+  uint8_t* flags;
+  const int64_t* entry_base;     // entry level: the pages are scheduled one by one, else null
+  long long n_member_entries;
+  const int64_t* page_base;
+  const int32_t* page2cluster;
+  int pitch, S, W, Cmax;
+};
 // `overlap`: launch with programmatic dependent launch after the previous kernel of the stream.
 // `selmap` (optional): per (request, head) bitmap of the selected pages, rows of selmap_pitch_bytes(Pmax).
 // `flags` with the three tables (optional): also mark the selected pages' clusters (see launch_resolve).
@@ -180,7 +194,9 @@ cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t*
                         uint8_t* selmap = nullptr, const int64_t* page_base = nullptr,
                         const int32_t* page2cluster = nullptr, const int64_t* cluster_base = nullptr,
                         uint8_t* flags = nullptr, const uint32_t* replica_mask = nullptr,
-                        const uint16_t* cluster_size = nullptr);
+                        const uint16_t* cluster_size = nullptr, const ExpandArgs* expand = nullptr);
+// Whether the selection kernel for these lists can expand its clusters itself (launch_topk's `expand`; no launch_expand_clusters then).
+bool select_expands(const Geometry& geo, int pitch);
 // Everything the cluster-resolution body needs (see resolve_body.cuh).  sel == nullptr: the flags are already
 // set (by the selection or the expansion kernel) and a single CTA runs the tail.
 // Host-step extension of the fused attention + resolution kernel: the step's small results are also stored
@@ -277,11 +293,8 @@ constexpr int kMaxExpandRowBytes = 160 * 1024;            // longest per-head pa
 cudaError_t launch_medoid_rows(const Geometry& geo, const uint16_t* ksum, const int64_t* page_base,
                                const int64_t* cluster_base, const int32_t* medoid_page, uint16_t* medoid_ksum,
                                int32_t* len, uint32_t* status, cudaStream_t st);
-cudaError_t launch_expand_clusters(const Geometry& geo, int k_c, const int32_t* sel_c, const int32_t* n_sel_c,
-                                   const int64_t* cluster_base, const int64_t* cluster_page_ptr,
-                                   const int32_t* cluster_pages, const int32_t* ctx_len, uint8_t* selmap, uint8_t* flags,
-                                   uint32_t* status, cudaStream_t st, bool overlap, const int64_t* entry_base,
-                                   long long n_member_entries, const int64_t* page_base, const int32_t* page2cluster);
+cudaError_t launch_expand_clusters(const ExpandArgs& ex, const Geometry& geo, int k_c, const int32_t* sel_c, const int32_t* n_sel_c, uint32_t* status,
+                                   cudaStream_t st, bool overlap);
 
 // Algorithm 1 (offline co-activation clustering): see cluster.cu.
 long long build_clusters_workspace_bytes(int n);

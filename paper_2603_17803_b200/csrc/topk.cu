@@ -18,7 +18,7 @@
 #include <algorithm>
 
 #define SWARM_TRACE_FILE 1
-#include "swarm_internal.cuh"
+#include "medoid_expand.cuh"
 
 namespace swarm {
 namespace {
@@ -277,12 +277,12 @@ __device__ __forceinline__ void finish_by_ranking(SelectState<THREADS>& st, int 
 // ---- register-resident variant -------------------------------------------------------------------
 // The selection of one list with ITEMS consecutive pages per thread (the kernel was launched for lists of up to
 // THREADS * MAX_ITEMS pages; rows of the page bitmap are that long).
-template <int THREADS, int ITEMS, int MAX_ITEMS, bool kEarly>
+template <int THREADS, int ITEMS, int MAX_ITEMS, bool kEarly, bool kExpand>
 __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const Geometry& geo, const TopkExtras& x,
                                                const RequestBases& rb, const float* __restrict__ s,
                                                int32_t* __restrict__ out, int32_t* __restrict__ n_sel,
                                                uint32_t* __restrict__ status, int bh, int b, int kvh, int len_b, bool* s_flag,
-                                               int P, int Pw, int k_eff, int k_sel) {
+                                               int P, int Pw, int k_eff, int k_sel, int32_t* s_list) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // thread t owns pages [t*ITEMS, (t+1)*ITEMS); keys of pages that do not exist are never used
   uint32_t key[ITEMS];
@@ -479,7 +479,9 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
   for (unsigned todo = picked; todo != 0u; todo &= todo - 1u) {
     const unsigned bit = todo & (0u - todo), below = bit - 1u;
     const int eq_b = eq_before + __popc(eq_mask & below);
-    out[gt_before + __popc(gt_mask & below) + min(eq_b, need_eq)] = p0 + (__ffs(bit) - 1);
+    const int place = gt_before + __popc(gt_mask & below) + min(eq_b, need_eq);
+    out[place] = p0 + (__ffs(bit) - 1);
+    if (kExpand) s_list[place] = p0 + (__ffs(bit) - 1);
   }
   if (kEarly && x.flags != nullptr) {
 #pragma unroll
@@ -510,10 +512,17 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
 }
 
 // (up to 512 threads: 40 registers, which is what a scorer CTA leaves of each quarter of an SM's registers)
-template <int THREADS, int ITEMS, bool kEarly>
+// kExpand: the list is one of clusters, and the CTA goes on to turn the selected ones into the head's page bitmap and the cluster
+// flags.  Bound by two dependent trips to memory; as a kernel of its own behind this one it paid for the boundary between the kernels
+// as well (5 ragged requests of up to 100K tokens: the step 54.0 -> 51.2 us, 2 of 12K 20.5 -> 18.7, 4 of up to 375K 31.3 -> 30.1).  The heads
+// announced one by one to the attention on top of that: 51.6, 19.5 and 28.4, a release more per head; not kept.
+template <int THREADS, int ITEMS, bool kEarly, bool kExpand>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1536 / THREADS)
 topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
-                 int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x) {
+                 int32_t* __restrict__ sel, int32_t* __restrict__ n_sel, uint32_t* __restrict__ status, TopkExtras x,
+                 const __grid_constant__ ExpandArgs ex) {
+  extern __shared__ uint32_t s_expand[];                  // kExpand: the bitmap row, then the selected clusters
+  int32_t* s_list = reinterpret_cast<int32_t*>(s_expand + (kExpand ? ex.pitch / 4 : 0));
   __shared__ SelectState<THREADS> st;
   __shared__ bool s_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -526,6 +535,11 @@ topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
   prefetch_tables(geo, x);
   const RequestBases rb = load_bases(x, b);
   const int len_b = ctx_len[b];
+  ExpandRequest rq{0, 0, 0};
+  if (kExpand) {
+    rq = expand_request(ex, b);
+    for (int i = tid; i < ex.pitch / 4; i += THREADS) s_expand[i] = 0u;
+  }
   const float* s = scores + (long long)bh * geo.Pmax;
   int32_t* out = sel + (long long)bh * geo.k;
   if (x.flags_alt > 0) x.flags += (x.tk.ctl[kCtlMarked] & 1u) * x.flags_alt;   // stable: the previous step's selection has finished
@@ -539,12 +553,16 @@ topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* 
   // phase is per page held, and the lists of one launch differ in length (ragged batches).
   bool ok;
   if (ITEMS == 16 && P <= THREADS * 8)
-    ok = topk_regs_body<THREADS, 8, ITEMS, kEarly>(st, geo, x, rb, s, out, n_sel, status, bh, b, kvh, len_b, &s_flag, P, Pw, k_eff, k_sel);
+    ok = topk_regs_body<THREADS, 8, ITEMS, kEarly, kExpand>(st, geo, x, rb, s, out, n_sel, status, bh, b, kvh, len_b, &s_flag, P, Pw, k_eff, k_sel, s_list);
   else
-    ok = topk_regs_body<THREADS, ITEMS, ITEMS, kEarly>(st, geo, x, rb, s, out, n_sel, status, bh, b, kvh, len_b, &s_flag, P, Pw, k_eff, k_sel);
+    ok = topk_regs_body<THREADS, ITEMS, ITEMS, kEarly, kExpand>(st, geo, x, rb, s, out, n_sel, status, bh, b, kvh, len_b, &s_flag, P, Pw, k_eff, k_sel, s_list);
   if (!ok) {
     write_empty_selection(geo, x, bh, out, n_sel, THREADS);
     selection_announce(geo, x, b, kvh);
+  }
+  if (kExpand) {
+    __syncthreads();                                        // the list is complete
+    expand_clusters<THREADS == 128 ? 4 : 8>(ex, rq, bh, b, ok ? k_eff : 0, [&](int j) { return s_list[j]; }, s_expand, status);
   }
   selection_done(geo, x);
   SWARM_KERNEL_END(status, 1);
@@ -880,6 +898,14 @@ SelectKind select_kind(int Pmax, long long lists) {
   if (smem_key_bytes(Pmax, 512) <= kSmemKeyBytes) return lists <= kLlScoreLists ? kSelectSmem1024 : kSelectSmem512;
   return kSelectGeneric;
 }
+// Selections in registers expand their clusters themselves while the bitmap row and the list take no more than this: beside the
+// selection's own state it stays below the 48 KiB that need no opt-in, and in all but the longest contexts (100000 tokens and 32
+// clusters: 912 bytes) a CTA still fits beside a scorer CTA.
+constexpr size_t kExpandSmem = 16 * 1024;
+static size_t expand_smem(int k, int pitch) { return (size_t)pitch + 4 * (size_t)k; }
+bool select_expands(const Geometry& geo, int pitch) {
+  return select_kind(geo.Pmax, (long long)geo.B * geo.Hq) == kSelectRegs && expand_smem(geo.k, pitch) <= kExpandSmem;
+}
 int select_per_sm(int Pmax, long long lists) {
   const int threads = Pmax <= 1024 ? 128 : Pmax <= 2048 ? 256 : Pmax <= 4096 ? 512 : 1024;
   switch (select_kind(Pmax, lists)) {
@@ -900,12 +926,15 @@ cudaError_t configure_topk() {
   cudaError_t e = cudaFuncSetAttribute(topk_smem_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKeyBytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_smem_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemKeyBytes);
   if (e == cudaSuccess) e = share_sm(topk_smem_kernel<512>);
-  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, false>);
-  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, true>);
-  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, false>);
-  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, true>);
-  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, false>);
-  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, true>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, false, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, true, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<128, 8, false, true>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, false, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, true, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<256, 8, false, true>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, false, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, true, false>);
+  if (e == cudaSuccess) e = share_sm(topk_regs_kernel<512, 8, false, true>);
   return e;
 }
 
@@ -913,7 +942,7 @@ cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t*
                         int32_t* n_sel, uint32_t* status, cudaStream_t st, bool overlap, const TopkLinks& links,
                         uint8_t* selmap, const int64_t* page_base, const int32_t* page2cluster,
                         const int64_t* cluster_base, uint8_t* flags, const uint32_t* replica_mask,
-                        const uint16_t* cluster_size) {
+                        const uint16_t* cluster_size, const ExpandArgs* expand) {
   TopkExtras x;
   x.selmap = selmap;
   x.selmap_pitch = selmap_pitch_bytes(geo.Pmax);
@@ -939,10 +968,13 @@ cudaError_t launch_topk(const Geometry& geo, const float* scores, const int32_t*
   if ((x.tk.selmap_ll != nullptr || x.tk.scores_ll != nullptr) && (!early || geo.Pmax > 16384)) return cudaErrorInvalidValue;
   const dim3 grid(geo.B * geo.Hq);
 #define SWARM_TOPK_REGS(THREADS, ITEMS)                                                                           \
-  return early ? launch_pdl(topk_regs_kernel<THREADS, ITEMS, true>, grid, dim3(THREADS), 0, st, overlap, geo, scores, \
-                            ctx_len, sel, n_sel, status, x)                                                         \
-               : launch_pdl(topk_regs_kernel<THREADS, ITEMS, false>, grid, dim3(THREADS), 0, st, overlap, geo, scores, \
-                            ctx_len, sel, n_sel, status, x)
+  return expand != nullptr                                                                                          \
+             ? launch_pdl(topk_regs_kernel<THREADS, ITEMS, false, true>, grid, dim3(THREADS), expand_smem(geo.k, expand->pitch), st, overlap, \
+                          geo, scores, ctx_len, sel, n_sel, status, x, *expand)                                     \
+         : early ? launch_pdl(topk_regs_kernel<THREADS, ITEMS, true, false>, grid, dim3(THREADS), 0, st, overlap, geo, \
+                              scores, ctx_len, sel, n_sel, status, x, ExpandArgs{})                                 \
+                 : launch_pdl(topk_regs_kernel<THREADS, ITEMS, false, false>, grid, dim3(THREADS), 0, st, overlap, geo, \
+                              scores, ctx_len, sel, n_sel, status, x, ExpandArgs{})
   const SelectKind kind = select_kind(geo.Pmax, (long long)geo.B * geo.Hq);
   if (kind == kSelectRegs) {
     if (geo.Pmax <= 1024) SWARM_TOPK_REGS(128, 8);

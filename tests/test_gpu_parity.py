@@ -1700,3 +1700,20 @@ def test_resolution_directly_behind_an_update_of_its_tables():
         parity.check_resolve(w, parity.host_tables(w), o.sel.cpu().numpy(), o.n_sel.cpu().numpy(), o.uniq.cpu().numpy(), o.queue_of.cpu().numpy(),
                              o.n_uniq.cpu().numpy()[0], o.queue_load.cpu().numpy())
     sess.close()
+
+
+@pytest.mark.parametrize("batch,hq,pages,cluster_pages,k_c,window", [(1, 4, 1023, 1, 70, 0), (2, 2, 1025, 1, 5, 3), (3, 2, 2049, 1, 300, 0), (1, 2, 4097, 1, 3964, 0),
+                                                                     (1, 2, 4097, 1, 3965, 0), (2, 66, 4500, 1, 40, 2), (2, 4, 1500, 41, 9, 0)])
+def test_medoid_step_at_the_limits_of_its_selection(batch, hq, pages, cluster_pages, k_c, window):
+    """The selection expands its clusters itself while the bitmap row and the list fit 16 KiB (3964 clusters of 4097 pages, not 3965) and its
+    keys fit registers (not 132 lists of 4500 clusters); every CTA size, and clusters of more members than lanes look at in one turn."""
+    cfg = small("c3_batched", batch=batch, ctx_len=16 * pages - 3, n_q_heads=hq, n_kv_heads=2, top_k=8, n_topics=3, cluster_pages=cluster_pages)
+    w = W.generate(cfg, seed=pages + k_c, device=DEV)
+    sess = Session(w, local_window_pages=window)
+    sess.enable_medoid_index(k_c, keep_scores=True)
+    for _ in range(2):
+        sess.step_medoid()
+        check_medoid_step(w, sess, k_c, window=window)
+    sess.step()                                             # the page step on the same scratch
+    parity.check_step(w, sess)
+    sess.close()
