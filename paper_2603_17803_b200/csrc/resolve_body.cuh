@@ -533,7 +533,6 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     uint32_t* at = s_pass;
     *reinterpret_cast<uint4*>(at + 4 * tid) = make_uint4(3u, 3u, 3u, 3u);
     at[kThreads * 4 + 2 * tid] = at[kThreads * 4 + 2 * tid + 1] = 0x00070008u;
-    if (kCached) at[kThreads * 11 + tid] = 0u;
   }
   int n = 0, n_serial = 0;                                 // clusters to fetch so far, and those for the serial pass
   const bool spill = n_clusters > cap;                     // the list may outgrow shared memory: it is written to global memory as well
@@ -560,7 +559,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
       f = at[kThreads * 6 + tid];
       if (dry) f = c0 + 4 <= n_clusters ? 0x01010101u : 0u;
       else if (f) __stcg(reinterpret_cast<uint32_t*>(flags + c0), 0u);   // leave zeros for the next call
-      if (kCached) {
+      if (kCached && !made_up) {                           // (a made-up cluster has no cache state: nothing is resident, no counts)
         if (cache_vec) {
           const int4 f4 = *reinterpret_cast<const int4*>(at + kThreads * 7 + 4 * tid);
           fr[0] = f4.x; fr[1] = f4.y; fr[2] = f4.z; fr[3] = f4.w;

@@ -1680,6 +1680,56 @@ def test_cache_bookkeeping_at_row_ends_and_unaligned_arrays(pages, shift):
     sess.close()
 
 
+@pytest.mark.parametrize("shift", [0, 1, 4])
+@pytest.mark.parametrize("pages", [5, 16 * 8, 2 * 1024 + 1])
+def test_resolutions_in_a_row_with_cache_state(pages, shift):
+    """Separate resolutions and admissions directly behind one another, with nothing between them on the host: every kernel lets the next
+    one start early, and each still counts on what the one before it left in the caller's arrays, which end with the last cluster."""
+    cfg = small("c1_tiny", ctx_len=16 * pages, top_k=max(1, pages // 3), n_q_heads=2, n_kv_heads=1, cluster_pages=1, n_queues=6)
+    w = W.generate(cfg, seed=pages, device=DEV)
+    C, T_BASE, T_TR = w.n_clusters, 80.0, 2.5
+    rng = np.random.default_rng(pages + shift)
+    resident0, freq0 = (rng.random(C) < 0.4).astype(np.uint8), rng.integers(0, 4, size=C).astype(np.int32)
+    resident, freq = (torch.zeros(shift + C, dtype=t, device=DEV) for t in (torch.uint8, torch.int32))
+    score = torch.zeros(shift + C, device=DEV)
+    n_hit = torch.zeros(4, dtype=torch.int32, device=DEV)
+    sess = Session(w)
+    sess.select()
+    other = [torch.roll(sess.o.sel, 1, dims=1)] + [torch.flip((sess.o.sel + 1 + i) % pages, dims=[2]).contiguous() for i in range(2)]
+    sels = [sess.o.sel, *(o.contiguous() for o in other)]
+    kinds = ["resolve", "resolve", "admit", "resolve", "resolve", "resolve", "admit", "resolve", "admit", "resolve"]
+    if shift:                                               # an admission takes arrays on 16-byte boundaries only
+        kinds = [k for k in kinds if k == "resolve"]
+    capacity = max(1, int(w.cluster_size.sum()) // 3)
+    B.swarm_set_cache(sess.ctx, resident=resident[shift:], freq=freq[shift:], score=score[shift:], n_hit=n_hit, t_base=T_BASE, t_transfer=T_TR)
+    for _ in range(6):                                      # the races this would show do not occur every time
+        resident[shift:], freq[shift:] = torch.from_numpy(resident0).to(DEV), torch.from_numpy(freq0).to(DEV)
+        torch.cuda.synchronize()
+        for turn, kind in enumerate(kinds):
+            if kind == "resolve":
+                sess.resolve(sel=sels[turn % len(sels)])
+            else:
+                B.swarm_cache_admit(score[shift:], w.cluster_size, capacity, resident[shift:])
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        tabs = parity.host_tables(w)
+        want_res, want_freq, want_score = resident0, freq0, None
+        for turn, kind in enumerate(kinds):
+            if kind == "resolve":
+                uniq, qof, load, hits, want_freq, want_score = oracle.resolve_cached(
+                    sels[turn % len(sels)].cpu().numpy(), sess.o.n_sel.cpu().numpy(), tabs["page_base"], tabs["page2cluster"], tabs["cluster_base"],
+                    tabs["replica_mask"], tabs["cluster_size"], want_res, want_freq, cfg.n_queues, T_BASE, T_TR)
+            else:
+                want_res, _, _ = oracle.cache_admit(want_score, tabs["cluster_size"], capacity)
+        assert np.array_equal(freq[shift:].cpu().numpy(), want_freq) and np.array_equal(resident[shift:].cpu().numpy(), want_res)
+        n = int(sess.o.n_uniq[0])
+        assert n == len(uniq) and int(n_hit[0]) == hits
+        assert np.array_equal(sess.o.uniq[:n].cpu().numpy(), uniq) and np.array_equal(sess.o.queue_of[:n].cpu().numpy(), qof)
+        assert np.allclose(score[shift:].cpu().numpy(), want_score, rtol=1e-6, atol=1e-6)
+    B.swarm_set_cache(sess.ctx)
+    sess.close()
+
+
 def test_resolution_directly_behind_an_update_of_its_tables():
     """The separate call runs its code once on made-up clusters while the kernel before it is still running, and reads none of its
     tables until that has finished."""
