@@ -525,9 +525,7 @@ int32_t swarm_resolve_clusters(swarm_ctx* ctx, const swarm_inputs* in, const int
   if (!resolve_inputs_ok(in) || bad(sel) || bad(n_sel) || bad(uniq) || bad(queue_of) || bad(n_uniq) ||
       bad(queue_load))
     return SWARM_ERR_INVALID_ARG;
-  ResolveArgs rs = step_resolve_args(ctx, in, sel, n_sel, uniq, queue_of, n_uniq, queue_load);
-  rs.rehearse = true;
-  SWARM_TRY(launch_resolve(rs, static_cast<cudaStream_t>(stream), true));
+  SWARM_TRY(launch_resolve(step_resolve_args(ctx, in, sel, n_sel, uniq, queue_of, n_uniq, queue_load), static_cast<cudaStream_t>(stream), true));
   return SWARM_OK;
 }
 

@@ -391,21 +391,25 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   __shared__ int s_hits;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // On its own any input may come from the previous kernel: nothing is read before the wait.
-  long long c_all = sel == nullptr ? cluster_base[geo.B] : 0;   // inside a step an input table: not written by the previous kernel
-  int C = (int)min((long long)geo.Cmax, c_all);
+  if (sel != nullptr) {                                  // on its own any input may come from the previous kernel
+    pdl_wait();
+    pdl_launch_dependents();                             // the next kernel in the stream may be scheduled while this one runs
+  }
+  const long long c_all = cluster_base[geo.B];           // inside a step an input table: not written by the previous kernel
+  const int C = (int)min((long long)geo.Cmax, c_all);
   unsigned err = 0u, step_no = 0u;
   // Every instruction below runs once per step, on an SM that has not fetched it since the step before, and while the
   // attention kernel streams a fetch from L2 takes 2-3 us.  A CTA that is resident before its selection has finished runs
-  // the body once on the first clusters of the tables, as if they were all activated, or in a kernel of its own on made-up ones:
-  // nothing but shared memory is written, and in a kernel of its own nothing is read.  A rehearsal takes about 10 us.  It pays where
+  // the body once on the first clusters of the tables, as if they were all activated: nothing but shared memory is written.
+  // A rehearsal takes about 10 us.  It pays where
   // the CTA waits as long anyway and the resolution ends the step: one request at 128K tokens 28.7 -> 28.1 us, at 32K tokens 18.0 -> 17.8;
   // with cache state, together with the stores of four words below, 16 ragged requests of up to 128K tokens 130.3 -> 125.1, 37 of 55K
-  // 190.5 -> 178.7, 12 of 33K 45.8 -> 43.0; four separate calls 115.6 -> 115.1.  Steps of several waves without cache state: 36.6 -> 36.9 (the
-  // attention ends them); the medoid step, which has 4 us to wait: 10 us longer.
-  for (bool dry = r.rehearse; ; dry = false) {
-  const bool made_up = dry && sel != nullptr;
-  int n_clusters = made_up ? kDryClusters : min(C, kDryClusters);
+  // 190.5 -> 178.7, 12 of 33K 45.8 -> 43.0.  Steps of several waves without cache state: 36.6 -> 36.9 (the attention ends them);
+  // the medoid step, which has 4 us to wait: 10 us longer.  Not in a kernel of its own, which does not know what it waits for: on an idle
+  // stream the call takes 35 us, 41 with a rehearsal on made-up clusters; 64 requests x 32 heads x 128 pages (256 CTAs) 34, and 41;
+  // 16 x 64 x 512 (512 CTAs) 45, and 64; only four separate calls in a row gained by it (114.2 us, and 113.7).
+  for (bool dry = !kAlone && r.rehearse; ; dry = false) {
+  int n_clusters = min(C, kDryClusters);
   int32_t* freq_out = cache.freq;
   float* score_out = cache.score;
   if (dry) {
@@ -416,11 +420,9 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   } else {
   uniq = r.uniq;
   queue_of = r.queue_of;
-  pdl_wait();                                            // the flags / the selection come from the previous kernel
-  pdl_launch_dependents();                               // the next kernel in the stream may be scheduled while this one runs
-  if (sel != nullptr) {
-    c_all = __ldcg(cluster_base + geo.B);
-    C = (int)min((long long)geo.Cmax, c_all);
+  if (sel == nullptr) {
+    pdl_wait();                                          // the flags come from the previous kernel
+    pdl_launch_dependents();
   }
   n_clusters = C;
   err = (c_all > geo.Cmax) ? SWARM_DEV_BAD_CLUSTER : 0u;
@@ -516,7 +518,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   const uint32_t ring = shared_addr(s_pass);
   auto request = [&](int row) {                            // (entries beyond the tables arrive as zeros)
     const int c = row * kRow + 4 * tid, have = min(4, n_clusters - c);
-    if (row < rows && have > 0 && !made_up) {
+    if (row < rows && have > 0) {
       const uint32_t at = ring + (row % kDepth) * kRowBytes;
       copy_async<16>(at + 16 * tid, replica_mask + c, 4 * have);
       if (need_sz) copy_async<8>(at + kThreads * 16 + 8 * tid, cluster_size + c, 2 * have);
@@ -529,11 +531,6 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   for (int row = 0; row < kDepth; ++row) request(row);
-  if (made_up && tid < kDryClusters / 4) {                 // clusters of two replicas and two weights
-    uint32_t* at = s_pass;
-    *reinterpret_cast<uint4*>(at + 4 * tid) = make_uint4(3u, 3u, 3u, 3u);
-    at[kThreads * 4 + 2 * tid] = at[kThreads * 4 + 2 * tid + 1] = 0x00070008u;
-  }
   int n = 0, n_serial = 0;                                 // clusters to fetch so far, and those for the serial pass
   const bool spill = n_clusters > cap;                     // the list may outgrow shared memory: it is written to global memory as well
   // submission order (optional): (replica class, queue) keys, kept in shared memory so that the ordering pass at the
@@ -559,7 +556,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
       f = at[kThreads * 6 + tid];
       if (dry) f = c0 + 4 <= n_clusters ? 0x01010101u : 0u;
       else if (f) __stcg(reinterpret_cast<uint32_t*>(flags + c0), 0u);   // leave zeros for the next call
-      if (kCached && !made_up) {                           // (a made-up cluster has no cache state: nothing is resident, no counts)
+      if (kCached) {
         if (cache_vec) {
           const int4 f4 = *reinterpret_cast<const int4*>(at + kThreads * 7 + 4 * tid);
           fr[0] = f4.x; fr[1] = f4.y; fr[2] = f4.z; fr[3] = f4.w;

@@ -1731,8 +1731,7 @@ def test_resolutions_in_a_row_with_cache_state(pages, shift):
 
 
 def test_resolution_directly_behind_an_update_of_its_tables():
-    """The separate call runs its code once on made-up clusters while the kernel before it is still running, and reads none of its
-    tables until that has finished."""
+    """The separate call finds its tables as the operations in front of it in the stream left them."""
     w = W.generate(CASES["c3_small"], seed=29, device=DEV)
     sess = Session(w)
     sess.step()
