@@ -708,7 +708,11 @@ int32_t step_impl(swarm_ctx* ctx, const swarm_inputs* in, const swarm_outputs* o
   // serial pass is the longest item of the step).
   a.n_splits = pick_splits(ctx, true, /*fused=*/true);
   a.n_more = pick_more(ctx, true, a.n_splits, /*fused=*/true);
-  rs.rehearse = links.tk.selmap_ll != nullptr || rs.has_cache;   // where the resolution ends the step (figures: resolve_body)
+  // Where the resolution ends the step (figures: resolve_body), and never in a second half: its predecessor is the caller's, which
+  // may be an admission that is still writing what a rehearsal with cache state reads, and the selection is long finished (the two
+  // halves with an operation on the flags between them, with cache state: one request at 128K tokens 39 us, 47 with a rehearsal; 12 of
+  // 33K 68, and 74).
+  rs.rehearse = links.tk.selmap_ll != nullptr || (whole && rs.has_cache);
   SWARM_TRY(launch_attention(ctx->geo, a, status, st, /*overlap=*/true, &rs));
   return SWARM_OK;
 }

@@ -1730,6 +1730,51 @@ def test_resolutions_in_a_row_with_cache_state(pages, shift):
     sess.close()
 
 
+@pytest.mark.parametrize("shift", [0, 4])
+@pytest.mark.parametrize("name", ["c1_small", "c3_small", "c5_small"])
+def test_second_half_directly_behind_an_admission(name, shift):
+    """The resolution of a step in two halves counts on what an admission between the halves has written, although the admission lets
+    the second half start before it has written anything; the attention does not notice either."""
+    w = W.generate(CASES[name], seed=31, device=DEV)
+    C, T_BASE, T_TR = w.n_clusters, 80.0, 2.5
+    rng = np.random.default_rng(C)
+    wish = [torch.from_numpy(rng.integers(0, 9, size=C).astype(np.float32)).to(DEV) for _ in range(3)]   # scores that decide the admissions
+    capacity = int(w.cluster_size.sum()) // 3
+    sizes = w.cluster_size.cpu().numpy().view(np.uint16)
+    admitted = [oracle.cache_admit(x.cpu().numpy(), sizes, capacity)[0] for x in wish]
+    resident, freq = torch.zeros(C, dtype=torch.uint8, device=DEV), torch.zeros(shift + C, dtype=torch.int32, device=DEV)
+    score, n_hit = torch.zeros(shift + C, device=DEV), torch.zeros(4, dtype=torch.int32, device=DEV)
+    sess = Session(w)
+    sess.step()
+    torch.cuda.synchronize()
+    out, lse = sess.o.out.clone(), sess.o.lse.clone()
+    B.swarm_set_cache(sess.ctx, resident=resident, freq=freq[shift:], score=score[shift:], n_hit=n_hit, t_base=T_BASE, t_transfer=T_TR)
+    for _ in range(4):
+        turns = 5
+        freq.zero_()
+        torch.cuda.synchronize()
+        for turn in range(turns):
+            sess.step_begin()
+            B.swarm_cache_admit(wish[turn % 3], w.cluster_size, capacity, resident)
+            sess.step_end()
+        torch.cuda.synchronize()
+        assert sess.status() == 0
+        tabs = parity.host_tables(w)
+        want_freq = np.zeros(C, dtype=np.int32)
+        for turn in range(turns):
+            uniq, qof, load, hits, want_freq, want_score = oracle.resolve_cached(
+                sess.o.sel.cpu().numpy(), sess.o.n_sel.cpu().numpy(), tabs["page_base"], tabs["page2cluster"], tabs["cluster_base"],
+                tabs["replica_mask"], tabs["cluster_size"], admitted[turn % 3], want_freq, w.cfg.n_queues, T_BASE, T_TR)
+        n = int(sess.o.n_uniq[0])
+        assert n == len(uniq) and int(n_hit[0]) == hits
+        assert np.array_equal(freq[shift:].cpu().numpy(), want_freq)
+        assert np.array_equal(sess.o.uniq[:n].cpu().numpy(), uniq) and np.array_equal(sess.o.queue_of[:n].cpu().numpy(), qof)
+        assert np.allclose(score[shift:].cpu().numpy(), want_score, rtol=1e-6, atol=1e-6)
+        assert (sess.o.out - out).abs().max().item() <= 1e-4 and (sess.o.lse - lse).abs().max().item() <= 1e-4   # (other ranges: other sums)
+    B.swarm_set_cache(sess.ctx)
+    sess.close()
+
+
 def test_resolution_directly_behind_an_update_of_its_tables():
     """The separate call finds its tables as the operations in front of it in the stream left them."""
     w = W.generate(CASES["c3_small"], seed=29, device=DEV)
