@@ -711,8 +711,9 @@ int32_t step_impl(swarm_ctx* ctx, const swarm_inputs* in, const swarm_outputs* o
   // Where the resolution ends the step (figures: resolve_body), and never in a second half: its predecessor is the caller's, which
   // may be an admission that is still writing what a rehearsal with cache state reads, and the selection is long finished (the two
   // halves with an operation on the flags between them, with cache state: one request at 128K tokens 39 us, 47 with a rehearsal; 12 of
-  // 33K 68, and 74).
-  rs.rehearse = links.tk.selmap_ll != nullptr || (whole && rs.has_cache);
+  // 33K 68, and 74).  Nor behind a gather, with cache state, where it is hidden in some shapes only (one request at
+  // 128K tokens 51.6-53.7 us, with a rehearsal 52.7-57.8; 2 of 8K 31-32, and 32-38; 4 of 128K 66-71, and 65-69).
+  rs.rehearse = links.tk.selmap_ll != nullptr || (whole && rs.has_cache && o->k_out == nullptr);
   SWARM_TRY(launch_attention(ctx->geo, a, status, st, /*overlap=*/true, &rs));
   return SWARM_OK;
 }
