@@ -61,7 +61,7 @@ attn_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
   if (kFused != 0 && blockIdx.x == 0) {
     // (the body is written for kThreads threads; the CTA's other warps leave, and a CTA-wide barrier counts the
     // threads that have not left)
-    if (threadIdx.x < resolve_detail::kThreads) resolve_detail::resolve_body<kFused == 2, false>(rs, 0, 1);
+    if (threadIdx.x < resolve_detail::kThreads) resolve_detail::resolve_body<kFused == 2>(rs, 0, 1);
     return;
   }
   const int cta = (int)blockIdx.x - (kFused != 0 ? 1 : 0);

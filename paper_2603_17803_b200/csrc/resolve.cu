@@ -9,7 +9,7 @@ using namespace resolve_detail;
 
 template <bool kCached>
 __global__ void __launch_bounds__(kThreads) resolve_kernel(ResolveArgs r) {
-  resolve_body<kCached, true>(r, (int)blockIdx.x, (int)gridDim.x);
+  resolve_body<kCached>(r, (int)blockIdx.x, (int)gridDim.x);
 }
 
 }  // namespace

@@ -351,13 +351,12 @@ __host__ __device__ constexpr int serial_words(bool submit) {
 static_assert(serial_words(false) * 4 <= (int)kResolveSmemBytes && serial_words(true) * 4 <= (int)kResolveSmemBytes,
               "the lists and their blanks fit behind the tables");
 
-// `cta` of `n_ctas` CTAs of kThreads threads run the body with kResolveSmemBytes of dynamic shared memory.  kAlone: in a kernel of
-// its own, which may be given a selection to mark (inside the attention kernel that code would only be more to fetch).
-template <bool kCached, bool kAlone>
+// `cta` of `n_ctas` CTAs of kThreads threads run the body with kResolveSmemBytes of dynamic shared memory.
+template <bool kCached>
 __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int n_ctas) {
   const Geometry& geo = r.geo;
   const swarm_cache& cache = r.cache;
-  const int32_t* __restrict__ sel = kAlone ? r.sel : nullptr;
+  const int32_t* __restrict__ sel = r.sel;
   const int32_t* __restrict__ n_sel = r.n_sel;
   const int64_t* __restrict__ page_base = r.page_base;
   const int32_t* __restrict__ page2cluster = r.page2cluster;
@@ -400,7 +399,7 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   unsigned err = 0u, step_no = 0u;
   // Every instruction below runs once per step, on an SM that has not fetched it since the step before, and while the
   // attention kernel streams a fetch from L2 takes 2-3 us.  A CTA that is resident before its selection has finished runs
-  // the body once on the first clusters of the tables, as if they were all activated: nothing but shared memory is written.
+  // the body once on the first clusters of the tables, as if they were all activated: nothing but scratch is written.
   // A rehearsal takes about 10 us.  It pays where
   // the CTA waits as long anyway and the resolution ends the step: one request at 128K tokens 28.7 -> 28.1 us, at 32K tokens 18.0 -> 17.8;
   // with cache state, together with the stores of four words below, 16 ragged requests of up to 128K tokens 130.3 -> 125.1, 37 of 55K
@@ -408,13 +407,16 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   // the medoid step, which has 4 us to wait: 10 us longer.  Not in a kernel of its own, which does not know what it waits for: on an idle
   // stream the call takes 35 us, 41 with a rehearsal on made-up clusters; 64 requests x 32 heads x 128 pages (256 CTAs) 34, and 41;
   // 16 x 64 x 512 (512 CTAs) 45, and 64; only four separate calls in a row gained by it (114.2 us, and 113.7).
-  for (bool dry = !kAlone && r.rehearse; ; dry = false) {
+  for (bool dry = r.rehearse; ; dry = false) {
   int n_clusters = min(C, kDryClusters);
   int32_t* freq_out = cache.freq;
   float* score_out = cache.score;
   if (dry) {
     uniq = s_dry.uniq;
-    queue_of = s_dry.queue_of;
+    // (With cache state in global memory: where the pointer may be into either, the pass over a list too long for shared memory, 16384
+    // clusters of 64 requests, was compiled slower: the step 645 us instead of 585.  So it was without cache state, 757 instead of 663,
+    // when code only a kernel of its own runs was left out of the attention kernel.)
+    queue_of = kCached ? reinterpret_cast<uint8_t*>(items) : s_dry.queue_of;
     freq_out = s_dry.freq;
     score_out = s_dry.score;
   } else {
