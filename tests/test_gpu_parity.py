@@ -1775,6 +1775,46 @@ def test_second_half_directly_behind_an_admission(name, shift):
     sess.close()
 
 
+def test_counters_that_a_step_does_not_move_can_be_moved_by_others():
+    """A step writes the counters of the activated and the resident clusters.  The others, among them neighbours in the same 16 bytes, belong
+    to whoever wants them meanwhile: a second stream counts them up beside the steps, and no count is lost on either side."""
+    w = W.generate(small("c2_128k", ctx_len=16 * 4096, top_k=64, n_topics=0, cluster_pages=1), seed=37, device=DEV)
+    C, steps = w.n_clusters, 60
+    sess = Session(w)
+    sess.step()
+    torch.cuda.synchronize()
+    resident = (torch.arange(C, device=DEV) % 5 == 0).to(torch.uint8)
+    moved = resident != 0
+    moved[sess.o.uniq[: int(sess.o.n_uniq[0])].long()] = True
+    others = torch.nonzero(~moved).flatten()
+    words = moved[: C // 4 * 4].view(-1, 4).sum(1)
+    assert int(((words > 0) & (words < 4)).sum()) > 100      # 16 bytes shared by both sides
+    freq, score = torch.zeros(C, dtype=torch.int32, device=DEV), torch.zeros(C, device=DEV)
+    B.swarm_set_cache(sess.ctx, resident=resident, freq=freq, score=score, t_base=80.0, t_transfer=2.5)
+    want = torch.zeros(C, dtype=torch.int32, device=DEV)
+    sess.step()                                             # what one step does to the counters
+    torch.cuda.synchronize()
+    once = freq.clone()
+    freq.zero_()
+    ones = torch.ones(len(others), dtype=torch.int32, device=DEV)
+    side, main = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    rounds = 0
+    for _ in range(steps):
+        sess.step(stream=main)
+        with torch.cuda.stream(side):
+            for _ in range(4):
+                freq.index_add_(0, others, ones)
+                rounds += 1
+    torch.cuda.synchronize()
+    assert sess.status() == 0
+    want = once * steps
+    want[others] += rounds
+    assert torch.equal(freq, want)
+    B.swarm_set_cache(sess.ctx)
+    sess.close()
+
+
 def test_resolution_directly_behind_an_update_of_its_tables():
     """The separate call finds its tables as the operations in front of it in the stream left them."""
     w = W.generate(CASES["c3_small"], seed=29, device=DEV)
