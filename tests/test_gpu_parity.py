@@ -1836,6 +1836,30 @@ def test_resolution_directly_behind_an_update_of_its_tables():
     sess.close()
 
 
+@pytest.mark.parametrize("name", ["c1_small", "c3_small", "c5_small"])
+def test_resolution_directly_behind_a_selection(name):
+    """The kernel in front of the separate call is the selection, which lets the resolution start before it has written anything: queries
+    that change every turn, nothing waits on the host, and every turn's schedule is that of its own selection."""
+    w = W.generate(CASES[name], seed=29, device=DEV)
+    sess = Session(w)
+    qs = [w.q, (w.q.float() * -1.0).to(torch.bfloat16), (w.q.float() * 0.5 + 0.125).to(torch.bfloat16)]
+    got = []
+    for turn in range(9):
+        sess.set_query(qs[turn % 3])
+        torch.cuda.synchronize()                            # (the two calls enqueued together, the device idle in front of them)
+        sess.select()
+        sess.resolve()
+        o = sess.o
+        got.append([x.clone() for x in (o.sel, o.n_sel, o.uniq, o.queue_of, o.n_uniq, o.queue_load)])
+    torch.cuda.synchronize()
+    assert sess.status() == 0
+    assert not torch.equal(got[0][0], got[1][0])
+    tabs = parity.host_tables(w)
+    for sel, n_sel, uniq, queue_of, n_uniq, load in ([x.cpu().numpy() for x in g] for g in got):
+        parity.check_resolve(w, tabs, sel, n_sel, uniq, queue_of, n_uniq[0], load)
+    sess.close()
+
+
 @pytest.mark.parametrize("batch,hq,pages,cluster_pages,k_c,window", [(1, 4, 1023, 1, 70, 0), (2, 2, 1025, 1, 5, 3), (3, 2, 2049, 1, 300, 0), (1, 2, 4097, 1, 3964, 0),
                                                                      (1, 2, 4097, 1, 3965, 0), (2, 66, 4500, 1, 40, 2), (2, 4, 1500, 41, 9, 0)])
 def test_medoid_step_at_the_limits_of_its_selection(batch, hq, pages, cluster_pages, k_c, window):
