@@ -468,7 +468,8 @@ __global__ void __launch_bounds__(kRoundThreads, 1) rounds_kernel(ClusterArgs a,
   // Every CTA counts the entries of each density, those in front of its own stretch of entries apart (two counts to a word), and
   // adds up the denser ones; an entry's place is what is denser, what is as dense in front of the stretch, and what is as dense
   // in front of it inside the stretch.  Bound by barriers and the atomics on a few popular counts.  (8192 entries: 7 us; comparing every
-  // entry with every other, 12 us.  The whole call 299.7 -> 292.7, 3911 entries 211 -> 205.)
+  // entry with every other, 12 us.  The whole call, both in turn three times: 8192 entries in 128 topics 264-269 -> 255-256, 16384 in 128
+  // 622 -> 597, 32768 in 256 1885 -> 1758; 3911 entries and fewer take the same time either way.)
   {
     uint32_t* hist = reinterpret_cast<uint32_t*>(dyn);     // [n] by n - 1 - density: all entries << 16 | those in front of the stretch
     const int stretch = (n + G - 1) / G, first = min(n, me * stretch), last = min(n, first + stretch);

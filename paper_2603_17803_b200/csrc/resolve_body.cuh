@@ -222,8 +222,9 @@ __device__ __forceinline__ void warps_arrive(int id) { asm volatile("bar.arrive 
 // Levels and table of the clusters [first, min(n, first + kChunk)) (one warp).  Returns the number of levels; the
 // cluster's level goes into the bits of wgt (weight << 5) from 21 on.  Rolled loops that look at the lists twice: what the code
 // costs is its fetch, once per step on an SM that has not run it since the step before.  (Unrolled over the 11 clusters, in registers: a
-// separate call on 983 clusters, 116.2 us with the calls around it, now 114.1; the medoid step of 1950 clusters 54.1, now 52.6; one
-// request at 128K tokens, 566 clusters, 30.8, now 30.5.)
+// separate call on 983 clusters, 116.5 us with the calls around it, now 114.3; the medoid step of 1950 clusters 54.1, now 53.3; six
+// ragged requests of up to 80K tokens 36.2, now 35.5.  Code that has just run is the slower one for it: the separate call over and over
+// 22.4, now 23.0.)
 __device__ __forceinline__ int levels_build(const uint32_t* mask, uint32_t* wgt, int n, int first, uint32_t* table) {
   const int lane = threadIdx.x & 31;
   const int i0 = first + lane * kStretch, i1 = min(n, i0 + kStretch);
@@ -402,8 +403,8 @@ __device__ __forceinline__ void resolve_body(const ResolveArgs& r, int cta, int 
   // the body once on the first clusters of the tables, as if they were all activated: nothing but scratch is written.
   // A rehearsal takes about 10 us.  It pays where
   // the CTA waits as long anyway and the resolution ends the step: one request at 128K tokens 28.7 -> 28.1 us, at 32K tokens 18.0 -> 17.8;
-  // with cache state, together with the stores of four words below, 16 ragged requests of up to 128K tokens 130.3 -> 125.1, 37 of 55K
-  // 190.5 -> 178.7, 12 of 33K 45.8 -> 43.0.  Steps of several waves without cache state: 36.6 -> 36.9 (the attention ends them);
+  // with cache state 16 ragged requests of up to 128K tokens and an admission 125.0 -> 124.6, 37 of 55K 177.8 -> 177.4, 3 of 114K 80.8 ->
+  // 79.0, 12 of 33K 43.3 -> 42.4.  Steps of several waves without cache state: 36.6 -> 36.9 (the attention ends them);
   // the medoid step, which has 4 us to wait: 10 us longer.  Not in a kernel of its own, which does not know what it waits for: on an idle
   // stream the call takes 35 us, 41 with a rehearsal on made-up clusters; 64 requests x 32 heads x 128 pages (256 CTAs) 34, and 41;
   // 16 x 64 x 512 (512 CTAs) 45, and 64; only four separate calls in a row gained by it (114.2 us, and 113.7).

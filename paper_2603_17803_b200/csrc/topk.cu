@@ -514,8 +514,8 @@ __device__ __forceinline__ bool topk_regs_body(SelectState<THREADS>& st, const G
 // (up to 512 threads: 40 registers, which is what a scorer CTA leaves of each quarter of an SM's registers)
 // kExpand: the list is one of clusters, and the CTA goes on to turn the selected ones into the head's page bitmap and the cluster
 // flags.  Bound by two dependent trips to memory; as a kernel of its own behind this one it paid for the boundary between the kernels
-// as well (5 ragged requests of up to 100K tokens: the step 54.0 -> 51.2 us, 2 of 12K 20.5 -> 18.7, 4 of up to 375K 31.3 -> 30.1).  The heads
-// announced one by one to the attention on top of that: 51.6, 19.5 and 28.4, a release more per head; not kept.
+// as well (5 ragged requests of up to 100K tokens: the step 51.8 -> 49.5 us, 2 of 12K 19.8 -> 18.7, 4 of up to 375K 31.0 -> 30.4).  The heads
+// announced one by one to the attention on top of that: slower in the first two, faster in the third, a release more per head; not kept.
 template <int THREADS, int ITEMS, bool kEarly, bool kExpand>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1536 / THREADS)
 topk_regs_kernel(Geometry geo, const float* __restrict__ scores, const int32_t* __restrict__ ctx_len,
@@ -900,7 +900,10 @@ SelectKind select_kind(int Pmax, long long lists) {
 }
 // Selections in registers expand their clusters themselves while the bitmap row and the list take no more than this: beside the
 // selection's own state it stays below the 48 KiB that need no opt-in, and in all but the longest contexts (100000 tokens and 32
-// clusters: 912 bytes) a CTA still fits beside a scorer CTA.
+// clusters: 912 bytes) a CTA still fits beside a scorer CTA.  With many lists and near the limit, against the kernel of its own:
+// 64 requests of 8K tokens and 16 clusters 187.0 us (189.5), 64 of 32K and 32 clusters 368 (373), one of 1M tokens (rows of 8 KB) 33.0 (34.7),
+// of 1.9M (15 KB) 41.1 (42.9), 8 of 1.9M 118.6 (120.7), 4 of 128K and 512 clusters 284.7 (289.6); slower in 64 of 120K with eight heads and
+// 64 clusters each, 179 (173), 64 ragged ones of up to 128K 498 (495) and 16 of 256K with 256 clusters 1195 (1182).
 constexpr size_t kExpandSmem = 16 * 1024;
 static size_t expand_smem(int k, int pitch) { return (size_t)pitch + 4 * (size_t)k; }
 bool select_expands(const Geometry& geo, int pitch) {
